@@ -68,7 +68,7 @@ struct PCount {
 #pragma unroll 1
     for (int k = 0; k < kSortSteps; ++k) {
       const int64_t base = (int64_t)item * kSortChunk + (k * 256 + (threadIdx.x & ~31)) * kSortBatch;
-      if (base < b.g.np) row_count_warp<T>(b.pos, b.g.np, b.g.n, b.g.delta, b.g.row_count, b.g.status, base);
+      if (base < b.g.np) row_count_warp<T>(b.pos, b.g.np, b.g.n, b.g.cell, b.g.row_count, b.g.status, base);
     }
   }
 };
@@ -165,7 +165,7 @@ struct PScatter {
     for (int k = 0; k < kSortSteps; ++k) {
       const int64_t base = (int64_t)item * kSortChunk + (k * 256 + (threadIdx.x & ~31)) * kSortBatch;
       if (base < b.g.np)
-        row_scatter_warp<T>(b.pos, b.g.np, b.g.n, b.g.delta, b.g.row_cursor, b.g.perm, b.g.rec, base, nullptr);
+        row_scatter_warp<T>(b.pos, b.g.np, b.g.n, b.g.cell, b.g.row_cursor, b.g.perm, b.g.rec, base, nullptr);
     }
   }
 };
@@ -293,8 +293,8 @@ struct PGather {
   static constexpr int THREADS = kGatherTPB;
   static constexpr size_t SMEM = 0;
   __device__ static void run(const BoxArgs& b, int item) {
-    interp_fd_chunk<T>(b.pos, b.g.np, b.g.n, b.g.delta, reinterpret_cast<const T*>(b.g.g),
-                       reinterpret_cast<T*>(b.vel), b.kick, nullptr, b.g.status, item);
+    interp_fd_chunk<T>(b.pos, b.g.np, b.g.n, b.g.cell, reinterpret_cast<const T*>(b.g.g),
+                       reinterpret_cast<T*>(b.vel), b.kick, nullptr, b.g.status, item, kGatherChunk);
   }
 };
 

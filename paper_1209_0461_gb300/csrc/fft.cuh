@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include "consts.cuh"
+#include "nupm_internal.h"
 #include "../../include/nupm.h"
 
 namespace nupm {
@@ -899,7 +900,7 @@ template <typename T, int N, class Q>
 __global__ void __launch_bounds__(XiCfg<T, N>::THREADS, 1)
 k_xinv_interp(const cx<T>* __restrict__ g, int64_t field_elems, const cx<T>* __restrict__ tw_m,
               const cx<T>* __restrict__ tw_n, const T* __restrict__ dtab, const void* __restrict__ pos, int64_t np,
-              double delta, const int* __restrict__ row_start, const int* __restrict__ perm, T* __restrict__ vel,
+              CellSize cell, const int* __restrict__ row_start, const int* __restrict__ perm, T* __restrict__ vel,
               T kick, T* __restrict__ acc_out, int* status) {
   static_assert((N & (N - 1)) == 0, "the sliding-window gather needs a power-of-two grid");
   using Cfg = XiCfg<T, N>;
@@ -980,7 +981,7 @@ k_xinv_interp(const cx<T>* __restrict__ g, int64_t field_elems, const cx<T>* __r
           const int64_t p = perm[beg[q] + (jj - pre[q])];
           int c[3], w[3];
           const typename Q::Raw raw = Q::load(pos, np, p);
-          if (!Q::get(raw, N, delta, c, w, status)) continue;
+          if (!Q::get(raw, N, cell, c, w, status)) continue;
           const T inv = (T)1.0 / (T)65536;
           const T fx1 = (T)w[0] * inv, fy1 = (T)w[1] * inv, fz1 = (T)w[2] * inv;
           const T fx0 = (T)1 - fx1, fy0 = (T)1 - fy1, fz0 = (T)1 - fz1;

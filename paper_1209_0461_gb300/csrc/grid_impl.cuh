@@ -284,7 +284,7 @@ void xinv_interp_n(const GridArgs& g, const void* pos, void* vel, double kick, v
   const int grid = items < g.sm_count ? items : g.sm_count;
   k_xinv_interp<T, N, Quant<T>><<<grid, X::THREADS, X::SMEM, s>>>(
       reinterpret_cast<const C*>(g.g), g.field_elems, reinterpret_cast<const C*>(g.tw_m),
-      reinterpret_cast<const C*>(g.tw_n), reinterpret_cast<const T*>(g.dtab), pos, g.np, g.delta, g.row_start,
+      reinterpret_cast<const C*>(g.tw_n), reinterpret_cast<const T*>(g.dtab), pos, g.np, g.cell, g.row_start,
       g.perm, reinterpret_cast<T*>(vel), (T)kick, reinterpret_cast<T*>(acc_out), g.status);
 }
 
@@ -318,7 +318,7 @@ int grid_blocks(int64_t work, int threads, int ctas_per_sm = 16) {
 int NUPM_FN(deposit)(const GridArgs& g, const void* pos, cudaStream_t s) {
   cudaMemsetAsync(g.g, 0, (size_t)g.n * g.n * g.n * sizeof(unsigned long long), s);
   if (g.np > 0)
-    k_deposit<T><<<grid_blocks(g.np, 256), 256, 0, s>>>(pos, g.np, g.n, g.delta,
+    k_deposit<T><<<grid_blocks(g.np, 256), 256, 0, s>>>(pos, g.np, g.n, g.cell,
                                                        reinterpret_cast<unsigned long long*>(g.g), g.status);
   return PM_OK;
 }
@@ -327,14 +327,14 @@ int NUPM_FN(row_sort)(const GridArgs& g, const void* pos, cudaStream_t s) {
   const int rows = g.n * g.n;
   cudaMemsetAsync(g.row_count, 0, (size_t)(rows + 1) * sizeof(int), s);
   const int blocks = grid_blocks(g.np, 256, g.part_ctas_per_sm);
-  if (g.np > 0) k_row_count<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.delta, g.row_count, g.status);
+  if (g.np > 0) k_row_count<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.cell, g.row_count, g.status);
   const int len = rows + 1;
   const int nb = (len + 2 * kScanBlock - 1) / (2 * kScanBlock);
   k_scan_blocks<<<nb, kScanBlock, 0, s>>>(g.row_count, g.row_start, g.scan_tot, len);
   k_scan_totals<<<1, kScanBlock, 0, s>>>(g.scan_tot, nb);
   k_scan_add<<<(len + 255) / 256, 256, 0, s>>>(g.row_start, g.scan_tot, len, g.row_cursor);
   if (g.np > 0)
-    k_row_scatter<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.delta, g.row_cursor, g.perm, g.rec, g.inv);
+    k_row_scatter<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.cell, g.row_cursor, g.perm, g.rec, g.inv);
   return PM_OK;
 }
 
@@ -420,7 +420,7 @@ int NUPM_FN(interp)(const GridArgs& g, const void* pos, void* vel, double kick, 
   if (g.np > 0 && g.fd_grad && g.rows_ready && g.gather_rows == 2) {
     // forces in the sort's row order by sorted slot, then the velocities in particle order
     k_interp_rows_acc<T><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
-                           kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, g.delta, reinterpret_cast<const T*>(g.g),
+                           kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, g.cell.fd_scale, reinterpret_cast<const T*>(g.g),
                                                reinterpret_cast<T*>(g.accs));
     k_kick_inv<T><<<grid_blocks(g.np, 256, g.part_ctas_per_sm), 256, 0, s>>>(
         g.inv, reinterpret_cast<const T*>(g.accs), g.np, reinterpret_cast<T*>(vel), (T)kick,
@@ -429,21 +429,22 @@ int NUPM_FN(interp)(const GridArgs& g, const void* pos, void* vel, double kick, 
   }
   if (g.np > 0 && g.fd_grad && g.rows_ready) {   // row order of the deposit's sort: a warp per row
     k_interp_rows_fd<T><<<(unsigned)(((int64_t)g.n * g.n + kRowsPerCta - 1) / kRowsPerCta), kGatherTPB, 0, s>>>(
-        g.rec, g.row_start, g.perm, g.np, g.n, g.delta, reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel),
+        g.rec, g.row_start, g.perm, g.np, g.n, g.cell.fd_scale, reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel),
         (T)kick, reinterpret_cast<T*>(acc_out));
     return PM_OK;
   }
   if (g.np > 0 && g.fd_grad) {
-    k_interp_kick_fd<T><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
+    const int per = gather_per(g.np, g.sm_count);
+    k_interp_kick_fd<T><<<(unsigned)((g.np + (int64_t)kGatherTPB * per - 1) / ((int64_t)kGatherTPB * per)),
                           kGatherTPB, 0, s>>>(
-        pos, g.np, g.n, g.delta, reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel), (T)kick,
-        reinterpret_cast<T*>(acc_out), g.status);
+        pos, g.np, g.n, g.cell, reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel), (T)kick,
+        reinterpret_cast<T*>(acc_out), g.status, per);
     return PM_OK;
   }
   if (g.np > 0)
     // 128-thread CTAs: the gather's ~96 registers per thread then fit 5 CTAs
     // (20 warps) per SM instead of 2 x 256 threads
-    k_interp_kick<T><<<grid_blocks(g.np, 128, 2 * g.part_ctas_per_sm), 128, 0, s>>>(pos, g.np, g.n, g.delta,
+    k_interp_kick<T><<<grid_blocks(g.np, 128, 2 * g.part_ctas_per_sm), 128, 0, s>>>(pos, g.np, g.n, g.cell,
                                                            reinterpret_cast<const T*>(g.g),
                                                            2 * g.field_elems, reinterpret_cast<T*>(vel), (T)kick,
                                                            reinterpret_cast<T*>(acc_out), g.status);

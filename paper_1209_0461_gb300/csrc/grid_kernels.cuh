@@ -46,6 +46,27 @@ __device__ __forceinline__ int partner_index(int i, int n) { return i == 0 ? 0 :
 template <typename T>
 struct Quant;
 
+// V = floor(RN(x / d) 2^16) of an FP64 position in integer arithmetic (false:
+// not decided here).  The cell is V >> 16 and the weight V & 0xffff.  GB300
+// issues two FP64 operations a cycle and SM, so an IEEE division and the
+// floors that follow (about 17 FP64 operations an axis) kept the row sort and
+// the gather on that pipe: at 256^3 particles the sort took 2.26 ms and moves
+// 1 GB.  Here x = m 2^ex and 65536 / d = rm 2^er multiply as 64-bit
+// mantissas, P = floor(m rm 2^-64), and V = P >> s.  P 2^-s is within
+// T (2^-53 + 2^-62) of the true T = 65536 x / d (the reciprocal's rounding and
+// the truncated product) and RN(x / d) within T 2^-53 of it, so for T < 2^31
+// V is exact unless T lies within 2^-20 of an integer; those (one in 5e5),
+// negative, huge, zero and non-finite positions take the division.
+__device__ __forceinline__ bool quant_fast(double x, const CellSize& cs, unsigned& v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int s = 2108 - (int)(b >> 52) - cs.re;   // bias 2 x 1023, 62 of the two 64-bit mantissas' 126 + 64
+  if ((unsigned)(s - 33) > 30u) return false;    // s in [33, 63]: 1 <= T < 2^31, sign clear
+  const unsigned long long p = __umul64hi((b << 11) | (1ull << 63), cs.rm);
+  v = (unsigned)(p >> s);
+  const unsigned fr = (unsigned)((p << (64 - s)) >> 32);   // fraction of T, 2^-32 units
+  return fr - 4096u < 0xffffe000u;
+}
+
 template <>
 struct Quant<double> {   // FP64 comoving positions, double[3][np]
   struct Raw {
@@ -55,21 +76,37 @@ struct Quant<double> {   // FP64 comoving positions, double[3][np]
     const double* x = reinterpret_cast<const double*>(pos);
     return Raw{{x[p], x[np + p], x[2 * np + p]}};
   }
-  __device__ static __forceinline__ bool cells(const Raw& r, int n, double delta, int (&c)[3], int (&w)[3]) {
+  // the definition, by IEEE division: cell * 2^16 + weight, -1 for an invalid position
+  __device__ static __noinline__ long long exact(double x, int n, double delta) {
+    const double u = x / delta;                      // same IEEE division as the definition
+    if (!(fabs(u) < 4503599627370496.0)) return -1;      // non-finite or |u| >= 2^52
+    const double cf = floor(u);
+    const double o = u - cf;                         // exact
+    const int w = (int)floor(o * (double)kWeightOne);
+    // o rounds to 1 just below a cell boundary (x = -1e-20): weight 2^16 of the
+    // cell is weight 0 of the next one, and fits the record's 16 bits
+    return ((long long)wrap_index((long long)cf + (w >> kWeightBits), n) << kWeightBits) + (w & (kWeightOne - 1));
+  }
+  __device__ static __forceinline__ bool cells(const Raw& r, int n, const CellSize& cs, int (&c)[3], int (&w)[3]) {
+    bool ok = true;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double u = r.x[d] / delta;                 // same IEEE division as the definition
-      if (!(fabs(u) < 4503599627370496.0)) return false;   // non-finite or |u| >= 2^52
-      const double cf = floor(u);
-      const double o = u - cf;                         // exact
-      w[d] = (int)floor(o * (double)kWeightOne);
-      c[d] = wrap_index((long long)cf, n);
+      unsigned v;
+      if (quant_fast(r.x[d], cs, v)) {
+        c[d] = wrap_index((int)(v >> kWeightBits), n);
+        w[d] = (int)(v & (kWeightOne - 1));
+      } else {
+        const long long e = exact(r.x[d], n, cs.d);
+        ok = ok && e >= 0;
+        c[d] = (int)(e >> kWeightBits);
+        w[d] = (int)(e & (kWeightOne - 1));
+      }
     }
-    return true;
+    return ok;
   }
-  __device__ static __forceinline__ bool get(const Raw& r, int n, double delta, int (&c)[3], int (&w)[3],
+  __device__ static __forceinline__ bool get(const Raw& r, int n, const CellSize& cs, int (&c)[3], int (&w)[3],
                                              int* status) {
-    if (cells(r, n, delta, c, w)) return true;
+    if (cells(r, n, cs, c, w)) return true;
     set_status(status, PM_ERR_RANGE);
     return false;
   }
@@ -87,7 +124,7 @@ struct Quant<float> {    // int32 words [6][np]: cells rows 0-2, FP32 offsets ro
     for (int d = 0; d < 6; ++d) r.q[d] = q[d * np + p];
     return r;
   }
-  __device__ static __forceinline__ bool cells(const Raw& r, int n, double, int (&c)[3], int (&w)[3]) {
+  __device__ static __forceinline__ bool cells(const Raw& r, int n, const CellSize&, int (&c)[3], int (&w)[3]) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const float o = __int_as_float(r.q[3 + d]);
@@ -97,9 +134,9 @@ struct Quant<float> {    // int32 words [6][np]: cells rows 0-2, FP32 offsets ro
     }
     return true;
   }
-  __device__ static __forceinline__ bool get(const Raw& r, int n, double delta, int (&c)[3], int (&w)[3],
+  __device__ static __forceinline__ bool get(const Raw& r, int n, const CellSize& cs, int (&c)[3], int (&w)[3],
                                              int* status) {
-    if (cells(r, n, delta, c, w)) return true;
+    if (cells(r, n, cs, c, w)) return true;
     set_status(status, PM_ERR_RANGE);
     return false;
   }
@@ -113,7 +150,7 @@ constexpr int kInterpBatch = 2;
 // Integer addition is associative, so the grid is bit-exact in any order.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_deposit(const void* __restrict__ pos, int64_t np, int n, double delta,
+__global__ void k_deposit(const void* __restrict__ pos, int64_t np, int n, CellSize cell,
                           unsigned long long* __restrict__ grid, int* status) {
   constexpr int U = kDepositBatch;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -127,7 +164,7 @@ __global__ void k_deposit(const void* __restrict__ pos, int64_t np, int n, doubl
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       int c[3], w[3];
-      if (p0 + u * stride >= np || !Quant<T>::get(raw[u], n, delta, c, w, status)) continue;
+      if (p0 + u * stride >= np || !Quant<T>::get(raw[u], n, cell, c, w, status)) continue;
       const unsigned long long wx[2] = {(unsigned long long)(kWeightOne - w[0]), (unsigned long long)w[0]};
       const unsigned long long wy[2] = {(unsigned long long)(kWeightOne - w[1]), (unsigned long long)w[1]};
       const unsigned long long wz[2] = {(unsigned long long)(kWeightOne - w[2]), (unsigned long long)w[2]};
@@ -752,7 +789,7 @@ __global__ void k_green_plane0(const cx<T>* __restrict__ spec, cx<T>* __restrict
 // weights as the deposit) and the kick u += acc * K.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_interp_kick(const void* __restrict__ pos, int64_t np, int n, double delta,
+__global__ void k_interp_kick(const void* __restrict__ pos, int64_t np, int n, CellSize cell,
                               const T* __restrict__ grids, int64_t field_stride, T* __restrict__ vel,
                               T kick, T* __restrict__ acc_out, int* status) {
   constexpr int U = kInterpBatch;
@@ -774,7 +811,7 @@ __global__ void k_interp_kick(const void* __restrict__ pos, int64_t np, int n, d
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       int c[3], w[3];
-      ok[u] = p0 + u * 32 < np && Quant<T>::get(raw[u], n, delta, c, w, status);
+      ok[u] = p0 + u * 32 < np && Quant<T>::get(raw[u], n, cell, c, w, status);
       if (!ok[u]) continue;
       const T inv = (T)1.0 / (T)kWeightOne;
       f[u][1] = (T)w[0] * inv;
@@ -847,12 +884,79 @@ __device__ __forceinline__ void fold_weights(T f0, T f1, T (&e)[6]) {
   e[5] = -f1;
 }
 
+// +-u 2^-sh as a double, from its bits (exact; u < 2^32, no FP64 operation:
+// GB300 issues two of those a cycle and SM, and this takes about ten integer ones)
+__device__ __forceinline__ double exact_pow2(unsigned u, int sh, bool neg) {
+  const int lz = __clz(u);
+  const unsigned m = (u << lz) << 1;                      // mantissa below the leading one
+  const unsigned hi = ((unsigned)(1023 + 31 - lz - sh) << 20) | (m >> 12) | (neg ? 0x80000000u : 0u);
+  return __hiloint2double(u ? (int)hi : 0, (int)(m << 20));
+}
+// a b 2^-32 for a, b in [0, 2^16] (the product reaches 2^32 only at a = b = 2^16)
+__device__ __forceinline__ double exact_product(unsigned a, unsigned b) {
+  if (a == 65536u && b == 65536u) return 1.0;
+  return exact_pow2(a * b, 32, false);
+}
+
+// The axis weights f (CIC) and e (folded stencil) and the pair products
+// f[1][y] f[2][z], f[0][x] f[2][z], f[0][x] f[1][y] of a particle's 16-bit weights.
+template <typename T>
+struct StencilWeights {
+  T f[3][2];
+  T ex[6], ey[6], ez[6];
+  __device__ __forceinline__ explicit StencilWeights(const int (&w)[3]) {
+    const T inv = (T)1.0 / (T)kWeightOne;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      f[d][1] = (T)w[d] * inv;
+      f[d][0] = (T)1 - f[d][1];
+    }
+    fold_weights(f[0][0], f[0][1], ex);
+    fold_weights(f[1][0], f[1][1], ey);
+    fold_weights(f[2][0], f[2][1], ez);
+  }
+  __device__ __forceinline__ T yz(int y, int z) const { return f[1][y] * f[2][z]; }
+  __device__ __forceinline__ T xz(int x, int z) const { return f[0][x] * f[2][z]; }
+  __device__ __forceinline__ T xy(int x, int y) const { return f[0][x] * f[1][y]; }
+};
+
+// FP64: every one of these is an integer times a power of two (e of up to 20
+// bits, products of up to 33), so they are built exactly from their bits: the
+// same values as the products and sums above without their 30 FP64 operations,
+// a quarter of the gather's.
+template <>
+struct StencilWeights<double> {
+  unsigned F[3][2];
+  double ex[6], ey[6], ez[6];
+  __device__ __forceinline__ static void fold(unsigned f0, unsigned f1, double (&e)[6]) {
+    const int e1 = (int)f1 - 8 * (int)f0, e4 = 8 * (int)f1 - (int)f0;
+    e[0] = exact_pow2(f0, 16, false);
+    e[1] = exact_pow2((unsigned)abs(e1), 16, e1 < 0);
+    e[2] = exact_pow2(f1, 13, true);
+    e[3] = exact_pow2(f0, 13, false);
+    e[4] = exact_pow2((unsigned)abs(e4), 16, e4 < 0);
+    e[5] = exact_pow2(f1, 16, true);
+  }
+  __device__ __forceinline__ explicit StencilWeights(const int (&w)[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      F[d][1] = (unsigned)w[d];
+      F[d][0] = (unsigned)(kWeightOne - w[d]);
+    }
+    fold(F[0][0], F[0][1], ex);
+    fold(F[1][0], F[1][1], ey);
+    fold(F[2][0], F[2][1], ez);
+  }
+  __device__ __forceinline__ double yz(int y, int z) const { return exact_product(F[1][y], F[2][z]); }
+  __device__ __forceinline__ double xz(int x, int z) const { return exact_product(F[0][x], F[2][z]); }
+  __device__ __forceinline__ double xy(int x, int y) const { return exact_product(F[0][x], F[1][y]); }
+};
+
 // -S phi at one particle (cell c, 16-bit weights w), before the -1/(12 d)
 // scale: the CIC sum of the 4-point stencil at its 8 corners (see above).
 template <typename T>
 __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, const int (&c)[3], const int (&w)[3],
                                            T (&a)[3]) {
-  const T inv = (T)1.0 / (T)kWeightOne;
   int xs[6], ys[6], zs[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
@@ -909,16 +1013,7 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
       pz[dy][0][q] = r[xs[2]];
       pz[dy][1][q] = r[xs[3]];
     }
-  T f[3][2];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    f[d][1] = (T)w[d] * inv;
-    f[d][0] = (T)1 - f[d][1];
-  }
-  T ex[6], ey[6], ez[6];
-  fold_weights(f[0][0], f[0][1], ex);
-  fold_weights(f[1][0], f[1][1], ey);
-  fold_weights(f[2][0], f[2][1], ez);
+  const StencilWeights<T> W(w);
   a[0] = a[1] = a[2] = (T)0;
 #pragma unroll
   for (int dz = 0; dz < 2; ++dz)
@@ -926,24 +1021,24 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
     for (int dy = 0; dy < 2; ++dy) {
       T sx = (T)0;
 #pragma unroll
-      for (int j = 0; j < 6; ++j) sx += ex[j] * px[dz][dy][j];
-      a[0] += f[1][dy] * f[2][dz] * sx;
+      for (int j = 0; j < 6; ++j) sx += W.ex[j] * px[dz][dy][j];
+      a[0] += W.yz(dy, dz) * sx;
     }
 #pragma unroll
   for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
     for (int dx = 0; dx < 2; ++dx) {
-      const T sy = ey[0] * py[dz][dx][0] + ey[1] * py[dz][dx][1] + ey[2] * px[dz][0][2 + dx] +
-                   ey[3] * px[dz][1][2 + dx] + ey[4] * py[dz][dx][2] + ey[5] * py[dz][dx][3];
-      a[1] += f[0][dx] * f[2][dz] * sy;
+      const T sy = W.ey[0] * py[dz][dx][0] + W.ey[1] * py[dz][dx][1] + W.ey[2] * px[dz][0][2 + dx] +
+                   W.ey[3] * px[dz][1][2 + dx] + W.ey[4] * py[dz][dx][2] + W.ey[5] * py[dz][dx][3];
+      a[1] += W.xz(dx, dz) * sy;
     }
 #pragma unroll
   for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
     for (int dx = 0; dx < 2; ++dx) {
-      const T sz = ez[0] * pz[dy][dx][0] + ez[1] * pz[dy][dx][1] + ez[2] * px[0][dy][2 + dx] +
-                   ez[3] * px[1][dy][2 + dx] + ez[4] * pz[dy][dx][2] + ez[5] * pz[dy][dx][3];
-      a[2] += f[0][dx] * f[1][dy] * sz;
+      const T sz = W.ez[0] * pz[dy][dx][0] + W.ez[1] * pz[dy][dx][1] + W.ez[2] * px[0][dy][2 + dx] +
+                   W.ez[3] * px[1][dy][2 + dx] + W.ez[4] * pz[dy][dx][2] + W.ez[5] * pz[dy][dx][3];
+      a[2] += W.xy(dx, dy) * sz;
     }
 }
 
@@ -959,26 +1054,36 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
 constexpr int kGatherTPB = 64;
 constexpr int kGatherChunk = 8;
 
-// Body: chunk `chunk` of kGatherTPB x kGatherChunk particles (blockDim = kGatherTPB).
+// Particles per thread of the particle-order gather: kGatherChunk, fewer where
+// np would give under four waves of resident CTAs (12 per SM).  The chunk is a
+// serial chain of load round trips, so at 32^3 particles 64 CTAs of 8 took
+// 53 us with most SMs idle; the line is where the last, partly filled wave
+// stops mattering.
+inline int gather_per(int64_t np, int sm_count) {
+  const int64_t per = np / ((int64_t)kGatherTPB * 12 * 4 * sm_count);
+  return per < 1 ? 1 : (per > kGatherChunk ? kGatherChunk : (int)per);
+}
+
+// Body: chunk `chunk` of kGatherTPB x per particles (blockDim = kGatherTPB).
 template <typename T>
-__device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, int64_t np, int n, double delta,
-                                                const T* __restrict__ phi, T* __restrict__ vel, T kick,
-                                                T* __restrict__ acc_out, int* status, int64_t chunk) {
-  const T scale = (T)(-1.0 / (12.0 * delta));   // acc = -S phi
-  const int64_t base = chunk * kGatherTPB * kGatherChunk + threadIdx.x;
+__device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, int64_t np, int n,
+                                                const CellSize& cell, const T* __restrict__ phi, T* __restrict__ vel, T kick,
+                                                T* __restrict__ acc_out, int* status, int64_t chunk, int per) {
+  const T scale = (T)cell.fd_scale;              // acc = -S phi (a division here is ten FP64 operations a thread)
+  const int64_t base = chunk * kGatherTPB * per + threadIdx.x;
   // the next particle's position words are fetched while this one's
   // potential values are in flight (one memory round trip per particle)
   typename Quant<T>::Raw next;
   if (base < np) next = Quant<T>::load(pos, np, base);
 #pragma unroll 1
-  for (int u = 0; u < kGatherChunk; ++u) {
+  for (int u = 0; u < per; ++u) {
     const int64_t p = base + (int64_t)u * kGatherTPB;
     if (p >= np) break;
     const typename Quant<T>::Raw raw = next;
-    if (u + 1 < kGatherChunk && p + kGatherTPB < np) next = Quant<T>::load(pos, np, p + kGatherTPB);
+    if (u + 1 < per && p + kGatherTPB < np) next = Quant<T>::load(pos, np, p + kGatherTPB);
     const T u0 = vel[p], u1 = vel[np + p], u2 = vel[2 * np + p];
     int c[3], w[3];
-    if (!Quant<T>::get(raw, n, delta, c, w, status)) continue;
+    if (!Quant<T>::get(raw, n, cell, c, w, status)) continue;
     T a[3];
     fd_stencil<T>(phi, n, c, w, a);
     const T uu[3] = {u0, u1, u2};
@@ -993,9 +1098,9 @@ __device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, in
 
 template <typename T>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 12 : 8)
-k_interp_kick_fd(const void* __restrict__ pos, int64_t np, int n, double delta, const T* __restrict__ phi,
-                 T* __restrict__ vel, T kick, T* __restrict__ acc_out, int* status) {
-  interp_fd_chunk<T>(pos, np, n, delta, phi, vel, kick, acc_out, status, blockIdx.x);
+k_interp_kick_fd(const void* __restrict__ pos, int64_t np, int n, CellSize cell, const T* __restrict__ phi,
+                 T* __restrict__ vel, T kick, T* __restrict__ acc_out, int* status, int per) {
+  interp_fd_chunk<T>(pos, np, n, cell, phi, vel, kick, acc_out, status, blockIdx.x, per);
 }
 
 // The same gather in the row order of the deposit's sort: one warp per grid
@@ -1011,9 +1116,9 @@ constexpr int kRowsPerCta = 8;
 template <typename T>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 10 : 8)
 k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start,
-                 const int* __restrict__ perm, int64_t np, int n, double delta, const T* __restrict__ phi,
+                 const int* __restrict__ perm, int64_t np, int n, double fd_scale, const T* __restrict__ phi,
                  T* __restrict__ vel, T kick, T* __restrict__ acc_out) {
-  const T scale = (T)(-1.0 / (12.0 * delta));
+  const T scale = (T)fd_scale;
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
   const int rows = n * n;
@@ -1056,9 +1161,9 @@ k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restri
 template <typename T>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 12 : 8)
 k_interp_rows_acc(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start, int n,
-                  double delta, const T* __restrict__ phi, T* __restrict__ accs) {
+                  double fd_scale, const T* __restrict__ phi, T* __restrict__ accs) {
   __shared__ int s_row;
-  const T scale = (T)(-1.0 / (12.0 * delta));
+  const T scale = (T)fd_scale;
   const int rows = n * n;
   const int nrec = row_start[rows];                 // the sorted (valid) records
   const int64_t i0 = (int64_t)blockIdx.x * kGatherTPB * kGatherChunk;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/nupm.h"
 
@@ -131,6 +132,29 @@ void launch_fac_table(float* fac, double umax, double kf, double f_nu, const dou
 void launch_green_table(bool fp64, void* gtab, long long n2max, double kf, double coeff,
                         double f_nu, const double* rlist, int nk, cudaStream_t s);
 
+// Cell size of the grid and 65536 / d as a 64-bit mantissa (bit 63 set) and a
+// biased exponent, for the FP64 positions' quantisation in integers (quant_fast
+// in grid_kernels.cuh); re = -65536 (no fast path) where 65536 / d is near the
+// ends of the exponent range.
+struct CellSize {
+  double d;
+  double fd_scale;          // -1 / (12 d): acc = -S phi (k_interp_kick_fd)
+  unsigned long long rm;
+  int re;
+};
+inline CellSize cell_size(double d) {
+  CellSize c;
+  c.d = d;
+  c.fd_scale = -1.0 / (12.0 * d);
+  const double r = 65536.0 / d;
+  unsigned long long b;
+  memcpy(&b, &r, sizeof b);
+  c.rm = (b << 11) | (1ull << 63);
+  c.re = (int)(b >> 52);
+  if (c.re < 100 || c.re > 2000) c.re = -65536;
+  return c;
+}
+
 // FFT passes in launch order of one kick
 constexpr int kPassXFwd = 0, kPassYFwd = 1, kPassZFwd = 2, kPassZInv = 3, kPassYInv = 4, kPassXInv = 5;
 
@@ -139,6 +163,7 @@ struct GridArgs {
   int n;
   int64_t np;
   double box, delta, scale;       // scale = N^3 / (Np 2^48)
+  CellSize cell;                  // delta and its reciprocal for the quantisation of positions
   void* spec;                     // packed spectrum [N][N][M]
   void* g;                        // 3 packed fields (deposit grid aliases the first two)
   int64_t field_elems;            // N*N*M complex elements per field

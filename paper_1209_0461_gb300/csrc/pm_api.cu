@@ -468,6 +468,7 @@ GridArgs grid_args(const pm_ctx* c) {
   g.np = c->np;
   g.box = c->box;
   g.delta = c->delta;
+  g.cell = cell_size(c->delta);
   g.scale = (double)c->n * c->n * c->n / ((double)c->np * 281474976710656.0);   // N^3 / (Np 2^48)
   g.spec = c->spec;
   g.g = c->g;

@@ -30,7 +30,7 @@ struct RowKey<float> {
     const int32_t* q = reinterpret_cast<const int32_t*>(pos);
     return Raw{q[np + p], q[2 * np + p], q[3 * np + p], q[4 * np + p], q[5 * np + p]};
   }
-  __device__ static __forceinline__ int key(const Raw& r, int n, double) {
+  __device__ static __forceinline__ int key(const Raw& r, int n, const CellSize&) {
     const float ox = __int_as_float(r.ox), oy = __int_as_float(r.oy), oz = __int_as_float(r.oz);
     if (!(ox >= 0.0f && ox < 1.0f && oy >= 0.0f && oy < 1.0f && oz >= 0.0f && oz < 1.0f)) return -1;
     return wrap_index(r.cz, n) * n + wrap_index(r.cy, n);
@@ -46,12 +46,10 @@ struct RowKey<double> {
     const double* x = reinterpret_cast<const double*>(pos);
     return Raw{x[p], x[np + p], x[2 * np + p]};
   }
-  __device__ static __forceinline__ int key(const Raw& r, int n, double delta) {
-    const double ux = r.x / delta, uy = r.y / delta, uz = r.z / delta;
-    if (!(fabs(ux) < 4503599627370496.0 && fabs(uy) < 4503599627370496.0 && fabs(uz) < 4503599627370496.0))
-      return -1;
-    const int cy = wrap_index((long long)floor(uy), n), cz = wrap_index((long long)floor(uz), n);
-    return cz * n + cy;
+  __device__ static __forceinline__ int key(const Raw& r, int n, const CellSize& cs) {
+    int c[3], w[3];
+    const Quant<double>::Raw q{{r.x, r.y, r.z}};
+    return Quant<double>::cells(q, n, cs, c, w) ? c[2] * n + c[1] : -1;
   }
 };
 
@@ -71,7 +69,7 @@ constexpr int kSortBatch = 4;
 // One warp's kSortBatch x 32 particles from `base` on (the warp-uniform body
 // of k_row_count; also run by the batched form).
 template <typename T>
-__device__ __forceinline__ void row_count_warp(const void* __restrict__ pos, int64_t np, int n, double delta,
+__device__ __forceinline__ void row_count_warp(const void* __restrict__ pos, int64_t np, int n, const CellSize& cell,
                                                int* __restrict__ count, int* status, int64_t base) {
   constexpr int U = kSortBatch;
   const unsigned full = 0xffffffffu;
@@ -86,7 +84,7 @@ __device__ __forceinline__ void row_count_warp(const void* __restrict__ pos, int
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int64_t p = base + u * 32 + lane;
-    key[u] = p < np ? RowKey<T>::key(raw[u], n, delta) : -2;
+    key[u] = p < np ? RowKey<T>::key(raw[u], n, cell) : -2;
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -98,17 +96,17 @@ __device__ __forceinline__ void row_count_warp(const void* __restrict__ pos, int
 }
 
 template <typename T>
-__global__ void k_row_count(const void* __restrict__ pos, int64_t np, int n, double delta,
+__global__ void k_row_count(const void* __restrict__ pos, int64_t np, int n, CellSize cell,
                             int* __restrict__ count, int* status) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * kSortBatch;
   for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * kSortBatch; base < np;
        base += stride)
-    row_count_warp<T>(pos, np, n, delta, count, status, base);
+    row_count_warp<T>(pos, np, n, cell, count, status, base);
 }
 
 // One warp's kSortBatch x 32 particles from `base` on (body of k_row_scatter).
 template <typename T>
-__device__ __forceinline__ void row_scatter_warp(const void* __restrict__ pos, int64_t np, int n, double delta,
+__device__ __forceinline__ void row_scatter_warp(const void* __restrict__ pos, int64_t np, int n, const CellSize& cell,
                                                  int* __restrict__ cursor, int* __restrict__ perm,
                                                  unsigned long long* __restrict__ rec, int64_t base,
                                                  int* __restrict__ inv = nullptr) {
@@ -126,7 +124,7 @@ __device__ __forceinline__ void row_scatter_warp(const void* __restrict__ pos, i
     const int64_t p = base + u * 32 + lane;
     int c[3] = {0, 0, 0}, w[3] = {0, 0, 0};
     int key = -2;
-    if (p < np) key = Quant<T>::cells(raw[u], n, delta, c, w) ? c[2] * n + c[1] : -1;
+    if (p < np) key = Quant<T>::cells(raw[u], n, cell, c, w) ? c[2] * n + c[1] : -1;
     const unsigned peers = __match_any_sync(full, key);
     const int leader = __ffs(peers) - 1;
     int start = 0;
@@ -147,13 +145,13 @@ __device__ __forceinline__ void row_scatter_warp(const void* __restrict__ pos, i
 // perm is given, the particle index) at the same sorted slot; with inv given,
 // each particle's slot (-1 for a skipped particle) in particle order.
 template <typename T>
-__global__ void k_row_scatter(const void* __restrict__ pos, int64_t np, int n, double delta,
+__global__ void k_row_scatter(const void* __restrict__ pos, int64_t np, int n, CellSize cell,
                               int* __restrict__ cursor, int* __restrict__ perm,
                               unsigned long long* __restrict__ rec, int* __restrict__ inv) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * kSortBatch;
   for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * kSortBatch; base < np;
        base += stride)
-    row_scatter_warp<T>(pos, np, n, delta, cursor, perm, rec, base, inv);
+    row_scatter_warp<T>(pos, np, n, cell, cursor, perm, rec, base, inv);
 }
 
 // Exclusive scan of n values in three launches: per-block scans of 2048
