@@ -176,10 +176,9 @@ struct PDeposit {
   static constexpr int THREADS = F::THREADS;
   static constexpr size_t SMEM = F::SMEM;
   __device__ static void run(const BoxArgs& b, int item) {
-    constexpr int NX = N / F::TY;
     deposit_fft_x_tile<T, N>(b.g.rec, b.g.row_start, reinterpret_cast<C*>(b.g.spec), b.g.scale,
                              reinterpret_cast<const C*>(b.g.tw_m), reinterpret_cast<const C*>(b.g.tw_n), nullptr,
-                             item % NX, item / NX, b.g.status);
+                             item, b.g.status);
   }
 };
 
@@ -379,6 +378,17 @@ int row_group(int n) {
     default: return 0;
   }
 }
+int deposit_rows(int n) {
+  switch (n) {
+    case 16: return FusedCfg<T, 16>::ROWS;
+    case 32: return FusedCfg<T, 32>::ROWS;
+    case 64: return FusedCfg<T, 64>::ROWS;
+    case 128: return FusedCfg<T, 128>::ROWS;
+    case 192: return FusedCfg<T, 192>::ROWS;
+    case 256: return FusedCfg<T, 256>::ROWS;
+    default: return 1;
+  }
+}
 }  // namespace
 
 bool batch_supported(int n) { return col_width(n) > 0; }
@@ -387,7 +397,7 @@ void batch_items(int n, int64_t np, int nk, int ns, int bin_chunks, int* items) 
   const int m = n / 2;
   items[kBpCount] = items[kBpScatter] = (int)((np + kSortChunk - 1) / kSortChunk);
   items[kBpScan] = 1;
-  items[kBpDeposit] = (n / FusedCfg<T, 64>::TY) * (n / FusedCfg<T, 64>::TZ);
+  items[kBpDeposit] = n * n / deposit_rows(n);
   items[kBpY] = items[kBpZ] = items[kBpZInv] = items[kBpYInv] = (m / col_width(n)) * n;
   items[kBpBins] = bin_chunks;
   items[kBpBinReduce] = (nk + 31) / 32;

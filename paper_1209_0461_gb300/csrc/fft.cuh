@@ -156,7 +156,7 @@ NUPM_PLAN(double, 192, 12, 4, 4)
 // L/R butterflies j; butterfly j (k = j mod NS) reads in[j + i L/R], applies
 // W_{NS R}^{i k}, does a radix-R DFT and writes out[(j/NS) NS R + k + i NS].
 // Thread t owns butterflies j = t + NT b.  SM provides ld(e)/st(e, v) on the
-// thread's own transform in shared memory.
+// thread's own transform in shared memory, and sync() among its threads.
 // ---------------------------------------------------------------------------
 template <typename T, int L, int E, int NT, int R, int NS, int DIR, bool FIRST, bool LAST, class SM>
 __device__ __forceinline__ void stockham_stage(cx<T> (&v)[E], const SM& sm, int t,
@@ -170,7 +170,7 @@ __device__ __forceinline__ void stockham_stage(cx<T> (&v)[E], const SM& sm, int 
 #pragma unroll
       for (int i = 0; i < R; ++i) v[b * R + i] = sm.ld(j + i * (L / R));
     }
-    if constexpr (!LAST) __syncthreads();   // reads done before in-place writes
+    if constexpr (!LAST) SM::sync();   // reads done before in-place writes
   }
 #pragma unroll
   for (int b = 0; b < E / R; ++b) {
@@ -188,7 +188,7 @@ __device__ __forceinline__ void stockham_stage(cx<T> (&v)[E], const SM& sm, int 
       for (int i = 0; i < R; ++i) sm.st(o0 + i * NS, v[b * R + i]);
     }
   }
-  if constexpr (!LAST) __syncthreads();
+  if constexpr (!LAST) SM::sync();
 }
 
 // Full transform of length L held as E = R1 registers per thread.  On entry v
@@ -216,9 +216,8 @@ __host__ __device__ constexpr int last_radix() {
   return P::R3 > 1 ? P::R3 : (P::R2 > 1 ? P::R2 : P::R1);
 }
 
-// Plans with fewer elements per thread for the fused deposit/x kernel: more
-// threads per tile for the particle phase and fewer registers, so that the
-// shared-memory tile, not the register file, sets the CTAs per SM.
+// Plans of the fused deposit/x kernel: a transform never takes more than one
+// warp, and few elements a lane leave registers for more warps.
 template <typename T, int L>
 struct FusedPlan : Plan<T, L> {};
 template <>
@@ -229,6 +228,10 @@ template <>
 struct FusedPlan<float, 256> {
   static constexpr int R1 = 8, R2 = 8, R3 = 4;
 };
+template <>
+struct FusedPlan<float, 128> {
+  static constexpr int R1 = 8, R2 = 8, R3 = 2;
+};
 
 // Shared-memory view of one column of a W-column tile: element e of column c
 // at e*W + c + (e >> 5) * PAD (PAD breaks bank conflicts of the stage writes).
@@ -238,6 +241,7 @@ struct ColSmem {
   int c;
   __device__ __forceinline__ cx<T> ld(int e) const { return base[e * W + c + (e >> 5) * PAD]; }
   __device__ __forceinline__ void st(int e, cx<T> v) const { base[e * W + c + (e >> 5) * PAD] = v; }
+  static __device__ __forceinline__ void sync() { __syncthreads(); }
   static constexpr int words(int L) { return L * W + ((L + 31) >> 5) * PAD; }
 };
 
@@ -247,7 +251,20 @@ struct RowSmem {
   cx<T>* base;
   __device__ __forceinline__ cx<T> ld(int e) const { return base[e + (e >> 5)]; }
   __device__ __forceinline__ void st(int e, cx<T> v) const { base[e + (e >> 5)] = v; }
+  static __device__ __forceinline__ void sync() { __syncthreads(); }
   static constexpr int words(int L) { return L + ((L + 31) >> 5); }
+};
+
+// A row transformed inside one warp: one pad per 16 elements, so that the
+// stage writes of 8 and of 16 elements a lane (8-byte words) fall in distinct
+// banks, and a warp-wide sync.
+template <typename T>
+struct WarpRowSmem {
+  cx<T>* base;
+  __device__ __forceinline__ cx<T> ld(int e) const { return base[e + (e >> 4)]; }
+  __device__ __forceinline__ void st(int e, cx<T> v) const { base[e + (e >> 4)] = v; }
+  static __device__ __forceinline__ void sync() { __syncwarp(); }
+  static constexpr int words(int L) { return L + ((L + 15) >> 4); }
 };
 
 // Column tile width (consecutive x2 columns per CTA) and pad per plan.
@@ -552,29 +569,43 @@ k_fft_x_fwd(const unsigned long long* __restrict__ grid, cx<T>* __restrict__ spe
 }
 
 // ---------------------------------------------------------------------------
-// Fused a1 + forward x pass.  A CTA owns TZ x TY grid rows (z, y): it
-// deposits every particle record of the (TZ+1) x (TY+1) source rows that
-// touch them (sorted into rows by k_row_scatter) into a shared-memory tile of
-// exact 64-bit sums, then transforms those rows exactly as k_fft_x_fwd.  No
-// global deposit grid, no memset, no atomics to DRAM.  With `keep` set the
-// tile is also written out (inspection).  grid = (N / TY, N / TZ).
+// Fused a1 + forward x pass, one warp per grid row (z, y) (several rows of a
+// small grid, one after another): the warp adds up its row's deposit in shared
+// memory as exact 64-bit sums and transforms it.  A node row gets corners from
+// the particles of four source rows, (z - 1, z) x (y - 1, y), whose records
+// (sorted by k_row_scatter) the warp reads; the corner's y and z weights then
+// depend on the source row alone and every lane has two corners, x and x + 1.
+// No other warp adds to the row, so nothing waits on a barrier: the deposit,
+// the exchanges of the transform and the split step's partners (a lane
+// shuffle: X[M - k] sits in lane NT - t) are the warp's own.  No global
+// deposit grid, no memset, no atomics to DRAM.  With `keep` set the sums are
+// also written out (inspection).
+//
+// Bound: issue slots and the shared-memory pipe (16 atomic adds a particle
+// and the exchanges).  A record is read by four warps (L1 and L2 after the
+// first) where a CTA tile of 2 x 4 rows read it 1.9 times, but there two
+// thirds of the corner adds fell outside the tile, and phases waited at
+// barriers.
 // ---------------------------------------------------------------------------
 template <typename T, int N>
 struct FusedCfg {
-  static constexpr int TZ = 2, TY = 4;
-  static constexpr int ROWS = TZ * TY;
   static constexpr int M = N / 2;
   using P = FusedPlan<T, M>;
   static constexpr int E = P::R1;
   static constexpr int NT = M / E;
-  static constexpr int THREADS = ROWS * NT;
-  static constexpr size_t ACC_BYTES = (size_t)ROWS * N * 8;
-  static constexpr size_t XCH_BYTES = (size_t)ROWS * RowSmem<T>::words(M) * sizeof(cx<T>);
-  static constexpr size_t SMEM = (ACC_BYTES > XCH_BYTES ? ACC_BYTES : XCH_BYTES);
-  // CTAs per SM that the shared-memory tile allows (227 KB), at most 4 (FP32)
-  // or 2 (FP64, whose transform needs twice the registers)
+  static constexpr int G = 32 / NT;                 // rows per warp
+  static constexpr int WARPS = 4;
+  static constexpr int ROWS = G * WARPS;            // rows per CTA
+  static constexpr int THREADS = 32 * WARPS;
+  static constexpr size_t ACC_BYTES = (size_t)N * 8;
+  static constexpr size_t XCH_BYTES = (size_t)WarpRowSmem<T>::words(M) * sizeof(cx<T>);
+  static constexpr size_t ROW_BYTES = ((ACC_BYTES > XCH_BYTES ? ACC_BYTES : XCH_BYTES) + 15) / 16 * 16;
+  static constexpr size_t SMEM = ROWS * ROW_BYTES;
+  static_assert(NT >= 1 && NT <= 32 && 32 % NT == 0 && (N * N) % ROWS == 0, "whole rows per warp");
+  // CTAs per SM that the rows' shared memory allows (227 KB), at most 8 (FP32)
+  // or 3 (FP64, whose transform needs twice the registers)
   static constexpr int BY_SMEM = (int)((227u * 1024u) / (SMEM + 1024u));
-  static constexpr int CAP = sizeof(T) == 4 ? 4 : 2;
+  static constexpr int CAP = sizeof(T) == 4 ? 8 : 3;
   static constexpr int MIN_BLOCKS = BY_SMEM < 1 ? 1 : (BY_SMEM > CAP ? CAP : BY_SMEM);
 };
 
@@ -586,155 +617,107 @@ __device__ __forceinline__ unsigned int carry_of(unsigned int old, unsigned int 
   return (old + lo < old) ? 1u : 0u;
 }
 
+// The deposit of one node row (gz, gy) by one warp into lo[N], hi[N] (zeroed).
+// Returns true where a sum wrapped past 2^64.
+template <int N>
+__device__ __forceinline__ bool deposit_row_warp(const unsigned long long* __restrict__ rec,
+                                                 const int* __restrict__ row_start, int gz, int gy,
+                                                 unsigned int* lo, unsigned int* hi) {
+  const int lane = threadIdx.x & 31;
+  // the four source rows, concatenated in a virtual index j: bit 0 of s = dy's
+  // complement (0: row y - 1, whose corner is dy = 1), bit 1 the same for z
+  int b[4], pre[5];
+  pre[0] = 0;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int sz = (s & 2) ? gz : (gz == 0 ? N - 1 : gz - 1);
+    const int sy = (s & 1) ? gy : (gy == 0 ? N - 1 : gy - 1);
+    const int r = sz * N + sy;
+    b[s] = row_start[r];
+    pre[s + 1] = pre[s] + row_start[r + 1] - b[s];
+  }
+#pragma unroll
+  for (int s = 0; s < 4; ++s) b[s] -= pre[s];
+  const int total = pre[4];
+  // A cell's sum wraps past 2^64 only with 65536 or more contributions of up
+  // to 2^48 each; a row with fewer records cannot overflow, and only one with
+  // more reads back its high-word adds to detect a wrap (PM_ERR_OVERFLOW).
+  const bool careful = total >= 65536;
+  bool ovf = false;
+  constexpr int U = 4;
+  for (int j0 = lane; j0 < total; j0 += 32 * U) {
+    unsigned long long rr[U];
+    int src[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 32 * u;
+      int o = b[0], s = 0;
+#pragma unroll
+      for (int k = 1; k < 4; ++k)
+        if (j >= pre[k]) {
+          o = b[k];
+          s = k;
+        }
+      src[u] = s;
+      rr[u] = j < total ? __ldg(rec + j + o) : 0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (j0 + 32 * u >= total) continue;
+      const unsigned long long r = rr[u];
+      const unsigned wx = (unsigned)r & 0xffffu, wy = (unsigned)(r >> 16) & 0xffffu, wz = (unsigned)(r >> 32) & 0xffffu;
+      const int c0 = (int)(r >> 48) & 0x7ff;
+      const int c1 = c0 + 1 == N ? 0 : c0 + 1;
+      const unsigned cy = (src[u] & 1) ? 65536u - wy : wy, cz = (src[u] & 2) ? 65536u - wz : wz;
+      const unsigned long long A = (unsigned long long)cy * cz;   // up to 2^32
+      const unsigned long long v1 = A * wx, v0 = (A << 16) - v1;
+      const unsigned l0 = (unsigned)v0, l1 = (unsigned)v1;
+      const unsigned o0 = atomicAdd(lo + c0, l0), o1 = atomicAdd(lo + c1, l1);
+      const unsigned h0 = (unsigned)(v0 >> 32) + carry_of(o0, l0), h1 = (unsigned)(v1 >> 32) + carry_of(o1, l1);
+      if (careful) {
+        const unsigned p0 = atomicAdd(hi + c0, h0), p1 = atomicAdd(hi + c1, h1);
+        ovf = ovf || (p0 + h0 < p0) || (p1 + h1 < p1);
+      } else {
+        atomicAdd(hi + c0, h0);
+        atomicAdd(hi + c1, h1);
+      }
+    }
+  }
+  return ovf;
+}
+
+// Rows ROWS bx .. ROWS (bx + 1) - 1.
 template <typename T, int N>
 __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __restrict__ rec,
                                                    const int* __restrict__ row_start, cx<T>* __restrict__ spec,
                                                    double scale, const cx<T>* __restrict__ tw_m,
                                                    const cx<T>* __restrict__ tw_n, unsigned long long* __restrict__ keep,
-                                                   int bx, int by, int* status) {
+                                                   int bx, int* status) {
   using Cfg = FusedCfg<T, N>;
   using P = typename Cfg::P;
-  constexpr int TZ = Cfg::TZ, TY = Cfg::TY, ROWS = Cfg::ROWS, M = N / 2, E = Cfg::E, NT = Cfg::NT;
-  constexpr int RL = last_radix<T, M, P>();
+  constexpr int M = N / 2, E = Cfg::E, NT = Cfg::NT, G = Cfg::G;
+  constexpr int RL = last_radix<T, M, P>(), EB = E / RL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned long long* acc = reinterpret_cast<unsigned long long*>(smem_raw);   // 2 x [ROWS][N] words
-  // The source rows (tz0-1 .. tz0+TZ-1) x (ty0-1 .. ty0+TY-1) are, per z, one
-  // contiguous run of the row-sorted permutation, plus the wrapped row y = N-1
-  // when ty0 = 0: NSEG segments, concatenated in a virtual index j.
-  constexpr int NSEG = 2 * (TZ + 1);
-  __shared__ int seg_pre[NSEG + 1], seg_beg[NSEG];
-  const int ty0 = bx * TY, tz0 = by * TZ;
-  for (int i = threadIdx.x; i < ROWS * N / 2; i += blockDim.x)
-    reinterpret_cast<ulonglong2*>(acc)[i] = ulonglong2{0ull, 0ull};
-  // lanes of the (first) warp: all 32, or the whole block when it is smaller
-  static_assert(Cfg::THREADS < 32 || Cfg::THREADS % 32 == 0, "whole warps or a single partial warp");
-  const unsigned wm = Cfg::THREADS >= 32 ? 0xffffffffu : ((1u << Cfg::THREADS) - 1u);
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    int len = 0, b0 = 0;
-    if (lane < NSEG) {
-      const int sz = (tz0 - 1 + lane / 2 + N) % N;
-      int r0, r1;
-      if (lane & 1) {            // main run of rows
-        r0 = sz * N + (ty0 ? ty0 - 1 : 0);
-        r1 = sz * N + ty0 + TY;
-      } else {                   // wrapped row N-1 (empty unless ty0 = 0)
-        r0 = sz * N + N - 1;
-        r1 = ty0 ? r0 : r0 + 1;
-      }
-      b0 = row_start[r0];
-      len = row_start[r1] - b0;
-    }
-    int incl = len;
-#pragma unroll
-    for (int d = 1; d < 8; d <<= 1) {
-      const int o = __shfl_up_sync(wm, incl, d);
-      if (lane >= d) incl += o;
-    }
-    if (lane < NSEG) {
-      seg_beg[lane] = b0;
-      seg_pre[lane + 1] = incl;
-    }
-    if (lane == 0) seg_pre[0] = 0;
-  }
-  __syncthreads();
-  const int total = seg_pre[NSEG];
-  int bound[NSEG], off[NSEG];   // j >= bound[s] -> record index j + off[s]
-#pragma unroll
-  for (int k = 0; k < NSEG; ++k) {
-    bound[k] = seg_pre[k];
-    off[k] = seg_beg[k] - seg_pre[k];
-  }
-  // low words of the cell sums in one plane, high words in the next: the
-  // low-word adds of random x cells spread over all 32 banks
-  unsigned int* accw = reinterpret_cast<unsigned int*>(acc);
-  constexpr int PLANE = ROWS * N;
-  // window rows: z planes tz0-1 .. tz0+TZ-1 (segment / 2), y rows ws .. ws+TY
-  // (identified by the record's y cell mod 32; N >= 32 or the mask below)
-  static_assert(N < 32 || N % 32 == 0, "the y window is identified mod 32");
-  constexpr int YM = (N < 32 ? N : 32) - 1;
-  const int ws = (ty0 - 1 + N) % N;
-  // A cell's sum wraps past 2^64 only with 65536 or more contributions of up
-  // to 2^48 each; a tile with fewer records cannot overflow, and only a tile
-  // with more reads back its high-word adds to detect a wrap (PM_ERR_OVERFLOW).
-  const bool careful = total >= 65536;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* wrows = smem_raw + (size_t)warp * G * Cfg::ROW_BYTES;
+  const int row0 = (bx * Cfg::WARPS + warp) * G;
+  for (int i = lane; i < (int)(G * Cfg::ROW_BYTES / 16); i += 32) reinterpret_cast<uint4*>(wrows)[i] = uint4{0, 0, 0, 0};
+  __syncwarp();
   bool ovf = false;
-  constexpr int U = 4;
-  for (int j0 = threadIdx.x; j0 < total; j0 += blockDim.x * U) {
-    unsigned long long rr[U];
-    int zp[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int j = j0 + u * blockDim.x;
-      int o = off[0], z = 0;
-#pragma unroll
-      for (int k = 1; k < NSEG; ++k)
-        if (j >= bound[k]) {
-          o = off[k];
-          z = k >> 1;
-        }
-      zp[u] = z;
-      rr[u] = j < total ? rec[j + o] : 0ull;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (j0 + u * (int)blockDim.x >= total) continue;
-      const unsigned long long r = rr[u];
-      const unsigned wx = (unsigned)r & 0xffffu, wy = (unsigned)(r >> 16) & 0xffffu;
-      const unsigned wzz = (unsigned)(r >> 32) & 0xffffu;
-      const int cx = (int)(r >> 48) & 0x7ff;
-      const int yo = ((int)(r >> 59) - ws) & YM;      // 0 .. TY: row of the window
-      const int x1 = cx + 1 == N ? 0 : cx + 1;
-      // the particle's (up to) 8 corners in this tile: all low-word adds in
-      // flight before any carry is needed
-      int slot[8];
-      unsigned int lo[8], hi[8], old[8];
-#pragma unroll
-      for (int dz = 0; dz < 2; ++dz) {
-        const int zl = zp[u] - 1 + dz;
-        const unsigned long long wz = dz ? (unsigned long long)wzz : (unsigned long long)(65536u - wzz);
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-          const int yl = yo - 1 + dy;
-          const bool in = zl >= 0 && zl < TZ && yl >= 0 && yl < TY;
-          const unsigned long long wzy = wz * (dy ? (unsigned long long)wy : (unsigned long long)(65536u - wy));
-          const int rb = (zl * TY + yl) * N;
-#pragma unroll
-          for (int dx = 0; dx < 2; ++dx) {
-            const int k = dz * 4 + dy * 2 + dx;
-            const unsigned long long v = in ? wzy * (unsigned long long)(dx ? wx : 65536u - wx) : 0ull;
-            slot[k] = rb + (dx ? x1 : cx);
-            lo[k] = (unsigned int)v;
-            hi[k] = (unsigned int)(v >> 32);
-          }
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (lo[k] | hi[k]) old[k] = atomicAdd(accw + slot[k], lo[k]);
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (lo[k] | hi[k]) {
-          const unsigned int h = hi[k] + carry_of(old[k], lo[k]);
-          if (h) {
-            if (careful) {
-              const unsigned int oh = atomicAdd(accw + PLANE + slot[k], h);
-              ovf = ovf || (oh + h < oh);
-            } else {
-              atomicAdd(accw + PLANE + slot[k], h);
-            }
-          }
-        }
-    }
+#pragma unroll 1
+  for (int g = 0; g < G; ++g) {
+    unsigned int* lo = reinterpret_cast<unsigned int*>(wrows + g * Cfg::ROW_BYTES);
+    const int row = row0 + g;
+    ovf |= deposit_row_warp<N>(rec, row_start, row / N, row % N, lo, lo + N);
   }
-  if (__syncthreads_or(ovf) && threadIdx.x == 0 && status) atomicCAS(status, 0, PM_ERR_OVERFLOW);
-  // forward x transform of the tile's rows (as k_fft_x_fwd)
-  const int t = threadIdx.x % NT;
-  const int r = threadIdx.x / NT;
-  const int gz = tz0 + r / TY, gy = ty0 + r % TY;
-  const int64_t grow = (int64_t)gz * N + gy;
-  const uint2* lo2 = reinterpret_cast<const uint2*>(accw + r * N);           // cells 2e, 2e+1
-  const uint2* hi2 = reinterpret_cast<const uint2*>(accw + PLANE + r * N);
+  if (__any_sync(0xffffffffu, ovf) && lane == 0 && status) atomicCAS(status, 0, PM_ERR_OVERFLOW);
+  __syncwarp();
+  // forward x transform of the warp's rows (as k_fft_x_fwd), NT lanes a row
+  const int t = lane % NT, r = lane / NT;
+  const int64_t grow = row0 + r;
+  unsigned char* rowp = wrows + r * Cfg::ROW_BYTES;
+  const uint2* lo2 = reinterpret_cast<const uint2*>(rowp);                 // low words of cells 2e, 2e+1
+  const uint2* hi2 = reinterpret_cast<const uint2*>(rowp + 4 * (size_t)N);
   cx<T> v[E];
   if (keep) {
     ulonglong2* kd = reinterpret_cast<ulonglong2*>(keep + grow * N);
@@ -764,31 +747,27 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
       v[i] = {(T)((double)fa * scale - 1.0), (T)((double)fb * scale - 1.0)};
     }
   }
-  __syncthreads();   // the tile is consumed; its memory now serves the exchange buffers
-  RowSmem<T> sm{reinterpret_cast<cx<T>*>(smem_raw) + r * RowSmem<T>::words(M)};
-  fft_regs<T, M, -1, RowSmem<T>, P>(v, sm, t, tw_m);
-  if constexpr (P::R2 > 1) __syncthreads();
-#pragma unroll
-  for (int b = 0; b < E / RL; ++b)
-#pragma unroll
-    for (int i = 0; i < RL; ++i) sm.st(t + NT * b + i * (M / RL), v[b * RL + i]);
-  __syncthreads();
+  __syncwarp();   // the sums are consumed; their memory now serves the exchange
+  const WarpRowSmem<T> sm{reinterpret_cast<cx<T>*>(rowp)};
+  fft_regs<T, M, -1, WarpRowSmem<T>, P>(v, sm, t, tw_m);
+  // v[b RL + i] = Z[t + NT (b + EB i)]; the split step of k = t + NT j needs
+  // Z[M - k], in lane NT - t at j' = E - 1 - j (lane 0: its own j' = E - j)
   cx<T>* dst = spec + grow * M;
+  const int peer = (lane & ~(NT - 1)) | ((NT - t) & (NT - 1));
+  auto at = [&](int j) { return v[(j % EB) * RL + j / EB]; };
 #pragma unroll
-  for (int i = 0; i < E; ++i) {
-    const int k = t + NT * i;
-    const cx<T> zk = sm.ld(k);
-    cx<T> out;
-    if (k == 0) {
-      out = {zk.x + zk.y, zk.x - zk.y};
-    } else {
-      const cx<T> zm = cconj(sm.ld(M - k));
-      const cx<T> ev = cscale(zk + zm, (T)0.5);
-      const cx<T> od = cscale(zk - zm, (T)0.5);
-      const cx<T> wv = twid_table<-1>(tw_n, k);
-      const cx<T> wo = cmul(wv, od);
-      out = {ev.x + wo.y, ev.y - wo.x};
-    }
+  for (int j = 0; j < E; ++j) {
+    const cx<T> q = at(E - 1 - j), own = at((E - j) % E);
+    cx<T> zp = {__shfl_sync(0xffffffffu, q.x, peer), __shfl_sync(0xffffffffu, q.y, peer)};
+    if (t == 0) zp = own;
+    const int k = t + NT * j;
+    const cx<T> zk = at(j);
+    const cx<T> zm = cconj(zp);
+    const cx<T> ev = cscale(zk + zm, (T)0.5);
+    const cx<T> od = cscale(zk - zm, (T)0.5);
+    const cx<T> wo = cmul(twid_table<-1>(tw_n, k), od);
+    cx<T> out = {ev.x + wo.y, ev.y - wo.x};
+    if (j == 0 && t == 0) out = {zk.x + zk.y, zk.x - zk.y};
     dst[k] = out;
   }
 }
@@ -798,7 +777,7 @@ __global__ void __launch_bounds__(FusedCfg<T, N>::THREADS, FusedCfg<T, N>::MIN_B
 k_deposit_fft_x(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start,
                 cx<T>* __restrict__ spec, double scale, const cx<T>* __restrict__ tw_m, const cx<T>* __restrict__ tw_n,
                 unsigned long long* __restrict__ keep, int* status) {
-  deposit_fft_x_tile<T, N>(rec, row_start, spec, scale, tw_m, tw_n, keep, blockIdx.x, blockIdx.y, status);
+  deposit_fft_x_tile<T, N>(rec, row_start, spec, scale, tw_m, tw_n, keep, blockIdx.x, status);
 }
 
 // ---------------------------------------------------------------------------
