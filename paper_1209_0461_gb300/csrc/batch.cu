@@ -176,7 +176,8 @@ struct PDeposit {
   static constexpr int THREADS = F::THREADS;
   static constexpr size_t SMEM = F::SMEM;
   __device__ static void run(const BoxArgs& b, int item) {
-    deposit_fft_x_tile<T, N>(b.g.rec, b.g.row_start, reinterpret_cast<C*>(b.g.spec), b.g.scale,
+    deposit_fft_x_tile<T, N>(b.g.rec, b.g.row_start, reinterpret_cast<C*>(b.g.spec),
+                             DepositScale{b.g.scale, b.g.scale_hi, b.g.scale_lo},
                              reinterpret_cast<const C*>(b.g.tw_m), reinterpret_cast<const C*>(b.g.tw_n), nullptr,
                              item, b.g.status);
   }

@@ -597,7 +597,8 @@ struct FusedCfg {
   static constexpr int WARPS = 4;
   static constexpr int ROWS = G * WARPS;            // rows per CTA
   static constexpr int THREADS = 32 * WARPS;
-  static constexpr size_t ACC_BYTES = (size_t)N * 8;
+  static constexpr int HI = N + 2;                  // first high word of a row's sums (words 0 .. N low)
+  static constexpr size_t ACC_BYTES = (size_t)2 * HI * 4;
   static constexpr size_t XCH_BYTES = (size_t)WarpRowSmem<T>::words(M) * sizeof(cx<T>);
   static constexpr size_t ROW_BYTES = ((ACC_BYTES > XCH_BYTES ? ACC_BYTES : XCH_BYTES) + 15) / 16 * 16;
   static constexpr size_t SMEM = ROWS * ROW_BYTES;
@@ -613,84 +614,87 @@ struct FusedCfg {
 // word's returned old value gives the carry into the high word.  Integer
 // addition stays associative, so the sum is bit-exact in any order, and the
 // high-word adds may trail the low-word adds of other corners.
-__device__ __forceinline__ unsigned int carry_of(unsigned int old, unsigned int lo) {
-  return (old + lo < old) ? 1u : 0u;
+__device__ __forceinline__ unsigned add_carry(unsigned old, unsigned lo, unsigned hi) {
+  unsigned t, h;
+  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, 0;" : "=r"(t), "=r"(h) : "r"(old), "r"(lo), "r"(hi));
+  return h;
 }
 
-// The deposit of one node row (gz, gy) by one warp into lo[N], hi[N] (zeroed).
-// Returns true where a sum wrapped past 2^64.
-template <int N>
-__device__ __forceinline__ bool deposit_row_warp(const unsigned long long* __restrict__ rec,
-                                                 const int* __restrict__ row_start, int gz, int gy,
-                                                 unsigned int* lo, unsigned int* hi) {
-  const int lane = threadIdx.x & 31;
-  // the four source rows, concatenated in a virtual index j: bit 0 of s = dy's
-  // complement (0: row y - 1, whose corner is dy = 1), bit 1 the same for z
-  int b[4], pre[5];
-  pre[0] = 0;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int sz = (s & 2) ? gz : (gz == 0 ? N - 1 : gz - 1);
-    const int sy = (s & 1) ? gy : (gy == 0 ? N - 1 : gy - 1);
-    const int r = sz * N + sy;
-    b[s] = row_start[r];
-    pre[s + 1] = pre[s] + row_start[r + 1] - b[s];
-  }
-#pragma unroll
-  for (int s = 0; s < 4; ++s) b[s] -= pre[s];
-  const int total = pre[4];
-  // A cell's sum wraps past 2^64 only with 65536 or more contributions of up
-  // to 2^48 each; a row with fewer records cannot overflow, and only one with
-  // more reads back its high-word adds to detect a wrap (PM_ERR_OVERFLOW).
-  const bool careful = total >= 65536;
+// Adds the records rec[0 .. len) of one source row into the node row's sums
+// (low words lo[0 .. N], high words lo[kHi ..]; the corner x + 1 of the last
+// cell goes to word N, folded into word 0 at the end).  The corner's y weight
+// is wy sy + ay (wy, or 2^16 - wy), z alike.  Returns true where a sum wrapped
+// past 2^64 (looked for only with CAREFUL).
+template <int kHi, bool CAREFUL>
+__device__ __forceinline__ bool deposit_segment(const unsigned long long* __restrict__ rec, int len, int sy, int ay,
+                                                int sz, int az, unsigned* lo) {
+  constexpr int U = 4;   // records in flight a lane
   bool ovf = false;
-  constexpr int U = 4;
-  for (int j0 = lane; j0 < total; j0 += 32 * U) {
-    unsigned long long rr[U];
-    int src[U];
+  for (int j0 = threadIdx.x & 31; j0 < len; j0 += 32 * U) {
+    uint2 rr[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (j0 + 32 * u < len) rr[u] = __ldg(reinterpret_cast<const uint2*>(rec) + j0 + 32 * u);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int j = j0 + 32 * u;
-      int o = b[0], s = 0;
-#pragma unroll
-      for (int k = 1; k < 4; ++k)
-        if (j >= pre[k]) {
-          o = b[k];
-          s = k;
-        }
-      src[u] = s;
-      rr[u] = j < total ? __ldg(rec + j + o) : 0ull;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (j0 + 32 * u >= total) continue;
-      const unsigned long long r = rr[u];
-      const unsigned wx = (unsigned)r & 0xffffu, wy = (unsigned)(r >> 16) & 0xffffu, wz = (unsigned)(r >> 32) & 0xffffu;
-      const int c0 = (int)(r >> 48) & 0x7ff;
-      const int c1 = c0 + 1 == N ? 0 : c0 + 1;
-      const unsigned cy = (src[u] & 1) ? 65536u - wy : wy, cz = (src[u] & 2) ? 65536u - wz : wz;
-      const unsigned long long A = (unsigned long long)cy * cz;   // up to 2^32
-      const unsigned long long v1 = A * wx, v0 = (A << 16) - v1;
-      const unsigned l0 = (unsigned)v0, l1 = (unsigned)v1;
-      const unsigned o0 = atomicAdd(lo + c0, l0), o1 = atomicAdd(lo + c1, l1);
-      const unsigned h0 = (unsigned)(v0 >> 32) + carry_of(o0, l0), h1 = (unsigned)(v1 >> 32) + carry_of(o1, l1);
-      if (careful) {
-        const unsigned p0 = atomicAdd(hi + c0, h0), p1 = atomicAdd(hi + c1, h1);
-        ovf = ovf || (p0 + h0 < p0) || (p1 + h1 < p1);
-      } else {
-        atomicAdd(hi + c0, h0);
-        atomicAdd(hi + c1, h1);
-      }
+      if (j0 + 32 * u >= len) break;
+      const uint2 r = rr[u];
+      const unsigned wx = r.x & 0xffffu, vx = 65536u - wx;
+      const unsigned cy = (unsigned)((int)(r.x >> 16) * sy + ay), cz = (unsigned)((int)(r.y & 0xffffu) * sz + az);
+      const unsigned long long A = (unsigned long long)cy * cz;    // up to 2^32: its high word is 0 or 1
+      const unsigned Al = (unsigned)A, Ah = (unsigned)(A >> 32);
+      const unsigned long long v0 = (unsigned long long)Al * vx, v1 = (unsigned long long)Al * wx;
+      unsigned* p = lo + ((r.y >> 16) & 0x7ffu);
+      const unsigned o0 = atomicAdd(p, (unsigned)v0), o1 = atomicAdd(p + 1, (unsigned)v1);
+      const unsigned h0 = add_carry(o0, (unsigned)v0, (unsigned)(v0 >> 32) + Ah * vx);
+      const unsigned h1 = add_carry(o1, (unsigned)v1, (unsigned)(v1 >> 32) + Ah * wx);
+      const unsigned q0 = atomicAdd(p + kHi, h0), q1 = atomicAdd(p + kHi + 1, h1);
+      if constexpr (CAREFUL) ovf = ovf || (q0 + h0 < q0) || (q1 + h1 < q1);
     }
   }
   return ovf;
 }
 
+// The deposit of one node row (gz, gy) by one warp into its zeroed sums.
+// Returns true where a sum wrapped past 2^64.
+template <int N, int kHi>
+__device__ __forceinline__ bool deposit_row_warp(const unsigned long long* __restrict__ rec,
+                                                 const int* __restrict__ row_start, int gz, int gy, unsigned* lo) {
+  int b[4], len[4], total = 0;   // source rows: bit 0 set = row gy (else gy - 1), bit 1 = plane gz (else gz - 1)
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int r = ((gz + N - 1 + (s >> 1)) % N) * N + (gy + N - 1 + (s & 1)) % N;
+    b[s] = row_start[r];
+    len[s] = row_start[r + 1] - b[s];
+    total += len[s];
+  }
+  // A cell's sum wraps past 2^64 only with 65536 or more contributions of up
+  // to 2^48 each; a row with fewer records cannot overflow, and only one with
+  // more reads back its high-word adds to detect a wrap (PM_ERR_OVERFLOW).
+  bool ovf = false;
+#pragma unroll 1
+  for (int s = 0; s < 4; ++s) {
+    const int sy = (s & 1) ? -1 : 1, ay = (s & 1) ? 65536 : 0, sz = (s & 2) ? -1 : 1, az = (s & 2) ? 65536 : 0;
+    const int bs = s == 0 ? b[0] : s == 1 ? b[1] : s == 2 ? b[2] : b[3];
+    const int ls = s == 0 ? len[0] : s == 1 ? len[1] : s == 2 ? len[2] : len[3];
+    if (total < 65536) deposit_segment<kHi, false>(rec + bs, ls, sy, ay, sz, az, lo);
+    else ovf |= deposit_segment<kHi, true>(rec + bs, ls, sy, ay, sz, az, lo);
+  }
+  return ovf;
+}
+
+// delta = F s - 1, with s 2^32 and s in FP32 for F = hi 2^32 + lo (made on the
+// host: in the kernel they would be FP64 operations of every thread).
+struct DepositScale {
+  double s;
+  float hi, lo;
+};
+
 // Rows ROWS bx .. ROWS (bx + 1) - 1.
 template <typename T, int N>
 __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __restrict__ rec,
                                                    const int* __restrict__ row_start, cx<T>* __restrict__ spec,
-                                                   double scale, const cx<T>* __restrict__ tw_m,
+                                                   DepositScale scale, const cx<T>* __restrict__ tw_m,
                                                    const cx<T>* __restrict__ tw_n, unsigned long long* __restrict__ keep,
                                                    int bx, int* status) {
   using Cfg = FusedCfg<T, N>;
@@ -706,9 +710,18 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
   bool ovf = false;
 #pragma unroll 1
   for (int g = 0; g < G; ++g) {
-    unsigned int* lo = reinterpret_cast<unsigned int*>(wrows + g * Cfg::ROW_BYTES);
     const int row = row0 + g;
-    ovf |= deposit_row_warp<N>(rec, row_start, row / N, row % N, lo, lo + N);
+    ovf |= deposit_row_warp<N, Cfg::HI>(rec, row_start, row / N, row % N,
+                                        reinterpret_cast<unsigned*>(wrows + g * Cfg::ROW_BYTES));
+  }
+  __syncwarp();
+  if (lane < G) {   // word N is cell 0's
+    unsigned* lo = reinterpret_cast<unsigned*>(wrows + lane * Cfg::ROW_BYTES);
+    const unsigned l0 = lo[0], h0 = lo[Cfg::HI], lN = lo[N], hN = lo[Cfg::HI + N];
+    const unsigned h = add_carry(l0, lN, hN);
+    lo[0] = l0 + lN;
+    lo[Cfg::HI] = h0 + h;
+    ovf = ovf || h0 + h < h0 || h < hN;
   }
   if (__any_sync(0xffffffffu, ovf) && lane == 0 && status) atomicCAS(status, 0, PM_ERR_OVERFLOW);
   __syncwarp();
@@ -717,7 +730,7 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
   const int64_t grow = row0 + r;
   unsigned char* rowp = wrows + r * Cfg::ROW_BYTES;
   const uint2* lo2 = reinterpret_cast<const uint2*>(rowp);                 // low words of cells 2e, 2e+1
-  const uint2* hi2 = reinterpret_cast<const uint2*>(rowp + 4 * (size_t)N);
+  const uint2* hi2 = reinterpret_cast<const uint2*>(rowp + 4 * (size_t)Cfg::HI);
   cx<T> v[E];
   if (keep) {
     ulonglong2* kd = reinterpret_cast<ulonglong2*>(keep + grow * N);
@@ -730,7 +743,7 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
   }
   if constexpr (sizeof(T) == 4) {
     // F = hi 2^32 + lo: delta = hi (s 2^32) + (lo s - 1) in FP32 FMAs
-    const float hs = (float)(scale * 4294967296.0), ls = (float)scale;
+    const float hs = scale.hi, ls = scale.lo;
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       const uint2 l = lo2[t + NT * i], h = hi2[t + NT * i];
@@ -744,7 +757,7 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
       const uint2 l = lo2[t + NT * i], h = hi2[t + NT * i];
       const unsigned long long fa = (unsigned long long)l.x | ((unsigned long long)h.x << 32);
       const unsigned long long fb = (unsigned long long)l.y | ((unsigned long long)h.y << 32);
-      v[i] = {(T)((double)fa * scale - 1.0), (T)((double)fb * scale - 1.0)};
+      v[i] = {(T)((double)fa * scale.s - 1.0), (T)((double)fb * scale.s - 1.0)};
     }
   }
   __syncwarp();   // the sums are consumed; their memory now serves the exchange
@@ -775,7 +788,7 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
 template <typename T, int N>
 __global__ void __launch_bounds__(FusedCfg<T, N>::THREADS, FusedCfg<T, N>::MIN_BLOCKS)
 k_deposit_fft_x(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start,
-                cx<T>* __restrict__ spec, double scale, const cx<T>* __restrict__ tw_m, const cx<T>* __restrict__ tw_n,
+                cx<T>* __restrict__ spec, DepositScale scale, const cx<T>* __restrict__ tw_m, const cx<T>* __restrict__ tw_n,
                 unsigned long long* __restrict__ keep, int* status) {
   deposit_fft_x_tile<T, N>(rec, row_start, spec, scale, tw_m, tw_n, keep, blockIdx.x, status);
 }

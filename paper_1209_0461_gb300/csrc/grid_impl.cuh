@@ -267,7 +267,7 @@ void deposit_fft_x_n(const GridArgs& g, const void* pos, bool keep, cudaStream_t
     attr = true;
   }
   k_deposit_fft_x<T, N><<<N * N / F::ROWS, F::THREADS, F::SMEM, s>>>(
-      g.rec, g.row_start, reinterpret_cast<C*>(g.spec), g.scale, reinterpret_cast<const C*>(g.tw_m),
+      g.rec, g.row_start, reinterpret_cast<C*>(g.spec), DepositScale{g.scale, g.scale_hi, g.scale_lo}, reinterpret_cast<const C*>(g.tw_m),
       reinterpret_cast<const C*>(g.tw_n), keep ? reinterpret_cast<unsigned long long*>(g.g) : nullptr, g.status);
 }
 
@@ -420,7 +420,7 @@ int NUPM_FN(interp)(const GridArgs& g, const void* pos, void* vel, double kick, 
   if (g.np > 0 && g.fd_grad && g.rows_ready && g.gather_rows == 2) {
     // forces in the sort's row order by sorted slot, then the velocities in particle order
     k_interp_rows_acc<T><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
-                           kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, g.cell.fd_scale, reinterpret_cast<const T*>(g.g),
+                           kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, fd_scale_of<T>(g.cell), reinterpret_cast<const T*>(g.g),
                                                reinterpret_cast<T*>(g.accs));
     k_kick_inv<T><<<grid_blocks(g.np, 256, g.part_ctas_per_sm), 256, 0, s>>>(
         g.inv, reinterpret_cast<const T*>(g.accs), g.np, reinterpret_cast<T*>(vel), (T)kick,
@@ -429,7 +429,7 @@ int NUPM_FN(interp)(const GridArgs& g, const void* pos, void* vel, double kick, 
   }
   if (g.np > 0 && g.fd_grad && g.rows_ready) {   // row order of the deposit's sort: a warp per row
     k_interp_rows_fd<T><<<(unsigned)(((int64_t)g.n * g.n + kRowsPerCta - 1) / kRowsPerCta), kGatherTPB, 0, s>>>(
-        g.rec, g.row_start, g.perm, g.np, g.n, g.cell.fd_scale, reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel),
+        g.rec, g.row_start, g.perm, g.np, g.n, fd_scale_of<T>(g.cell), reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel),
         (T)kick, reinterpret_cast<T*>(acc_out));
     return PM_OK;
   }

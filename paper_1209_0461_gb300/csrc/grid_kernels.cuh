@@ -1069,7 +1069,7 @@ template <typename T>
 __device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, int64_t np, int n,
                                                 const CellSize& cell, const T* __restrict__ phi, T* __restrict__ vel, T kick,
                                                 T* __restrict__ acc_out, int* status, int64_t chunk, int per) {
-  const T scale = (T)cell.fd_scale;              // acc = -S phi (a division here is ten FP64 operations a thread)
+  const T scale = fd_scale_of<T>(cell);          // acc = -S phi
   const int64_t base = chunk * kGatherTPB * per + threadIdx.x;
   // the next particle's position words are fetched while this one's
   // potential values are in flight (one memory round trip per particle)
@@ -1116,9 +1116,8 @@ constexpr int kRowsPerCta = 8;
 template <typename T>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 10 : 8)
 k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start,
-                 const int* __restrict__ perm, int64_t np, int n, double fd_scale, const T* __restrict__ phi,
+                 const int* __restrict__ perm, int64_t np, int n, T scale, const T* __restrict__ phi,
                  T* __restrict__ vel, T kick, T* __restrict__ acc_out) {
-  const T scale = (T)fd_scale;
   const int lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
   const int rows = n * n;
@@ -1161,9 +1160,8 @@ k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restri
 template <typename T>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 12 : 8)
 k_interp_rows_acc(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start, int n,
-                  double fd_scale, const T* __restrict__ phi, T* __restrict__ accs) {
+                  T scale, const T* __restrict__ phi, T* __restrict__ accs) {
   __shared__ int s_row;
-  const T scale = (T)fd_scale;
   const int rows = n * n;
   const int nrec = row_start[rows];                 // the sorted (valid) records
   const int64_t i0 = (int64_t)blockIdx.x * kGatherTPB * kGatherChunk;

@@ -138,14 +138,21 @@ void launch_green_table(bool fp64, void* gtab, long long n2max, double kf, doubl
 // ends of the exponent range.
 struct CellSize {
   double d;
-  double fd_scale;          // -1 / (12 d): acc = -S phi (k_interp_kick_fd)
+  double fd_scale;          // -1 / (12 d): acc = -S phi (k_interp_kick_fd), and in FP32 (a
+  float fd_scale_f;         // conversion in the kernel is an FP64 operation a thread)
   unsigned long long rm;
   int re;
 };
+template <typename T>
+__host__ __device__ inline T fd_scale_of(const CellSize& c) {
+  if constexpr (sizeof(T) == 4) return c.fd_scale_f;
+  else return c.fd_scale;
+}
 inline CellSize cell_size(double d) {
   CellSize c;
   c.d = d;
   c.fd_scale = -1.0 / (12.0 * d);
+  c.fd_scale_f = (float)c.fd_scale;
   const double r = 65536.0 / d;
   unsigned long long b;
   memcpy(&b, &r, sizeof b);
@@ -163,6 +170,7 @@ struct GridArgs {
   int n;
   int64_t np;
   double box, delta, scale;       // scale = N^3 / (Np 2^48)
+  float scale_hi, scale_lo;       // scale 2^32 and scale in FP32
   CellSize cell;                  // delta and its reciprocal for the quantisation of positions
   void* spec;                     // packed spectrum [N][N][M]
   void* g;                        // 3 packed fields (deposit grid aliases the first two)

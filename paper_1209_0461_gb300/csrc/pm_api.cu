@@ -470,6 +470,8 @@ GridArgs grid_args(const pm_ctx* c) {
   g.delta = c->delta;
   g.cell = cell_size(c->delta);
   g.scale = (double)c->n * c->n * c->n / ((double)c->np * 281474976710656.0);   // N^3 / (Np 2^48)
+  g.scale_hi = (float)(g.scale * 4294967296.0);
+  g.scale_lo = (float)g.scale;
   g.spec = c->spec;
   g.g = c->g;
   g.field_elems = c->field_elems;
