@@ -289,11 +289,12 @@ struct PXInv {
   }
 };
 
+template <int N>
 struct PGather {
   static constexpr int THREADS = kGatherTPB;
   static constexpr size_t SMEM = 0;
   __device__ static void run(const BoxArgs& b, int item) {
-    interp_fd_chunk<T>(b.pos, b.g.np, b.g.n, b.g.cell, reinterpret_cast<const T*>(b.g.g),
+    interp_fd_chunk<T, (N & (N - 1)) == 0>(b.pos, b.g.np, N, b.g.cell, reinterpret_cast<const T*>(b.g.g),
                        reinterpret_cast<T*>(b.vel), b.kick, nullptr, b.g.status, item, kGatherChunk);
   }
 };
@@ -351,7 +352,7 @@ void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEve
   launch_pass<PZInv<N>>(p, kBpZInv, PZInv<N>::SMEM, s);
   launch_pass<PCol<N, +1, false, true>>(p, kBpYInv, PCol<N, +1, false, true>::SMEM, s);
   launch_pass<PXInv<N>>(p, kBpXInv, PXInv<N>::SMEM, s);
-  launch_pass<PGather>(p, kBpGather, 0, s);
+  launch_pass<PGather<N>>(p, kBpGather, 0, s);
 }
 
 }  // namespace

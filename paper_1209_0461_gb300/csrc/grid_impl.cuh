@@ -309,6 +309,31 @@ int grid_blocks(int64_t work, int threads, int ctas_per_sm = 16) {
   return (int)b;
 }
 
+// The gather with the real-space gradient, in the order that the tuning asks
+// for (POW2: the grid size is a power of two, so the wraps are masks).
+template <bool POW2>
+void gather_fd(const GridArgs& g, const void* pos, void* vel, double kick, void* acc_out, cudaStream_t s) {
+  const T* phi = reinterpret_cast<const T*>(g.g);
+  T* v = reinterpret_cast<T*>(vel);
+  T* acc = reinterpret_cast<T*>(acc_out);
+  const T scale = fd_scale_of<T>(g.cell);
+  if (g.rows_ready && g.gather_rows == 2) {
+    // forces in the sort's row order by sorted slot, then the velocities in particle order
+    k_interp_rows_acc<T, POW2><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
+                                 kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, scale, phi,
+                                                     reinterpret_cast<T*>(g.accs));
+    k_kick_inv<T><<<grid_blocks(g.np, 256, g.part_ctas_per_sm), 256, 0, s>>>(
+        g.inv, reinterpret_cast<const T*>(g.accs), g.np, v, (T)kick, acc);
+  } else if (g.rows_ready) {   // row order of the deposit's sort: a warp per row
+    k_interp_rows_fd<T, POW2><<<(unsigned)(((int64_t)g.n * g.n + kRowsPerCta - 1) / kRowsPerCta), kGatherTPB, 0, s>>>(
+        g.rec, g.row_start, g.perm, g.np, g.n, scale, phi, v, (T)kick, acc);
+  } else {
+    const int per = gather_per(g.np, g.sm_count);
+    k_interp_kick_fd<T, POW2><<<(unsigned)((g.np + (int64_t)kGatherTPB * per - 1) / ((int64_t)kGatherTPB * per)),
+                                kGatherTPB, 0, s>>>(pos, g.np, g.n, g.cell, phi, v, (T)kick, acc, g.status, per);
+  }
+}
+
 }  // namespace
 
 #define NUPM_CAT2(a, b) a##b
@@ -417,28 +442,9 @@ int NUPM_FN(green)(const GridArgs& g, cudaStream_t s) {
 }
 
 int NUPM_FN(interp)(const GridArgs& g, const void* pos, void* vel, double kick, void* acc_out, cudaStream_t s) {
-  if (g.np > 0 && g.fd_grad && g.rows_ready && g.gather_rows == 2) {
-    // forces in the sort's row order by sorted slot, then the velocities in particle order
-    k_interp_rows_acc<T><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
-                           kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, fd_scale_of<T>(g.cell), reinterpret_cast<const T*>(g.g),
-                                               reinterpret_cast<T*>(g.accs));
-    k_kick_inv<T><<<grid_blocks(g.np, 256, g.part_ctas_per_sm), 256, 0, s>>>(
-        g.inv, reinterpret_cast<const T*>(g.accs), g.np, reinterpret_cast<T*>(vel), (T)kick,
-        reinterpret_cast<T*>(acc_out));
-    return PM_OK;
-  }
-  if (g.np > 0 && g.fd_grad && g.rows_ready) {   // row order of the deposit's sort: a warp per row
-    k_interp_rows_fd<T><<<(unsigned)(((int64_t)g.n * g.n + kRowsPerCta - 1) / kRowsPerCta), kGatherTPB, 0, s>>>(
-        g.rec, g.row_start, g.perm, g.np, g.n, fd_scale_of<T>(g.cell), reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel),
-        (T)kick, reinterpret_cast<T*>(acc_out));
-    return PM_OK;
-  }
   if (g.np > 0 && g.fd_grad) {
-    const int per = gather_per(g.np, g.sm_count);
-    k_interp_kick_fd<T><<<(unsigned)((g.np + (int64_t)kGatherTPB * per - 1) / ((int64_t)kGatherTPB * per)),
-                          kGatherTPB, 0, s>>>(
-        pos, g.np, g.n, g.cell, reinterpret_cast<const T*>(g.g), reinterpret_cast<T*>(vel), (T)kick,
-        reinterpret_cast<T*>(acc_out), g.status, per);
+    if ((g.n & (g.n - 1)) == 0) gather_fd<true>(g, pos, vel, kick, acc_out, s);
+    else gather_fd<false>(g, pos, vel, kick, acc_out, s);
     return PM_OK;
   }
   if (g.np > 0)

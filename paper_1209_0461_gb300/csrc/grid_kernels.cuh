@@ -36,6 +36,12 @@ __device__ __forceinline__ int wrap_index(long long c, int n) {
   const long long r = c % n;
   return (int)(r < 0 ? r + n : r);
 }
+// The same with the kind of n known at compile time (POW2: the mask alone).
+template <bool POW2, typename I>
+__device__ __forceinline__ int wrap_to(I c, int n) {
+  if constexpr (POW2) return (int)(c & (I)(n - 1));
+  else return wrap_index(c, n);
+}
 // (n - i) mod n for i in [0, n): the index of the Hermitian partner.
 __device__ __forceinline__ int partner_index(int i, int n) { return i == 0 ? 0 : n - i; }
 
@@ -87,13 +93,14 @@ struct Quant<double> {   // FP64 comoving positions, double[3][np]
     // cell is weight 0 of the next one, and fits the record's 16 bits
     return ((long long)wrap_index((long long)cf + (w >> kWeightBits), n) << kWeightBits) + (w & (kWeightOne - 1));
   }
+  template <bool POW2 = false>
   __device__ static __forceinline__ bool cells(const Raw& r, int n, const CellSize& cs, int (&c)[3], int (&w)[3]) {
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       unsigned v;
       if (quant_fast(r.x[d], cs, v)) {
-        c[d] = wrap_index((int)(v >> kWeightBits), n);
+        c[d] = wrap_to<POW2>((int)(v >> kWeightBits), n);
         w[d] = (int)(v & (kWeightOne - 1));
       } else {
         const long long e = exact(r.x[d], n, cs.d);
@@ -104,9 +111,10 @@ struct Quant<double> {   // FP64 comoving positions, double[3][np]
     }
     return ok;
   }
+  template <bool POW2 = false>
   __device__ static __forceinline__ bool get(const Raw& r, int n, const CellSize& cs, int (&c)[3], int (&w)[3],
                                              int* status) {
-    if (cells(r, n, cs, c, w)) return true;
+    if (cells<POW2>(r, n, cs, c, w)) return true;
     set_status(status, PM_ERR_RANGE);
     return false;
   }
@@ -124,19 +132,21 @@ struct Quant<float> {    // int32 words [6][np]: cells rows 0-2, FP32 offsets ro
     for (int d = 0; d < 6; ++d) r.q[d] = q[d * np + p];
     return r;
   }
+  template <bool POW2 = false>
   __device__ static __forceinline__ bool cells(const Raw& r, int n, const CellSize&, int (&c)[3], int (&w)[3]) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const float o = __int_as_float(r.q[3 + d]);
       if (!(o >= 0.0f && o < 1.0f)) return false;
-      w[d] = (int)floorf(o * (float)kWeightOne);       // exact scaling by 2^16
-      c[d] = wrap_index((int)r.q[d], n);
+      w[d] = __float2int_rd(o * (float)kWeightOne);    // exact scaling by 2^16
+      c[d] = wrap_to<POW2>((int)r.q[d], n);
     }
     return true;
   }
+  template <bool POW2 = false>
   __device__ static __forceinline__ bool get(const Raw& r, int n, const CellSize& cs, int (&c)[3], int (&w)[3],
                                              int* status) {
-    if (cells(r, n, cs, c, w)) return true;
+    if (cells<POW2>(r, n, cs, c, w)) return true;
     set_status(status, PM_ERR_RANGE);
     return false;
   }
@@ -867,9 +877,10 @@ __global__ void k_interp_kick(const void* __restrict__ pos, int64_t np, int n, C
 // so each particle reads 56 potential values (four 6-point runs along x,
 // eight 4-point runs along y and along z) instead of 3 x 8 force values.
 // ---------------------------------------------------------------------------
+template <bool POW2>
 __device__ __forceinline__ int wrap_near(int c, int d, int n) {
   int v = c + d;   // d in [-2, 3], c in [0, n), n >= 16
-  if ((n & (n - 1)) == 0) return v & (n - 1);
+  if constexpr (POW2) return v & (n - 1);
   v = v < 0 ? v + n : v;
   return v >= n ? v - n : v;
 }
@@ -954,65 +965,91 @@ struct StencilWeights<double> {
 
 // -S phi at one particle (cell c, 16-bit weights w), before the -1/(12 d)
 // scale: the CIC sum of the 4-point stencil at its 8 corners (see above).
-template <typename T>
+// The 56 values lie on 20 (y, z) rows.  Away from the ends of the rows one
+// address a row serves its loads by constant offsets; the few particles there
+// take the wrapped indices.  FP32 x runs: aligned 8-byte loads from x0 - 2
+// rounded down to even (three, a fourth when x0 is odd).
+// Bound: the L1 data pipe (two wavefronts a load: 32 neighbouring particles
+// span two 128-byte lines) and the load queue; 64 KB-register CTAs (14 or 16
+// of 64 threads per SM) spill and run slower (0.40 and 0.44 ms against 0.345
+// at 256^3), 4-byte loads of the x runs too (0.372; 3.55 against 3.09 ms at
+// 1024^3).  With wrapped indices for all particles and a run-time test of n in
+// every wrap it took 0.365 and 3.19 ms.
+template <typename T, bool POW2>
 __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, const int (&c)[3], const int (&w)[3],
                                            T (&a)[3]) {
-  int xs[6], ys[6], zs[6];
+  uint32_t yo[6], zo[6];   // row offsets; indices < 2^30 for n <= 1024
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
-    xs[j] = wrap_near(c[0], j - 2, n);
-    ys[j] = wrap_near(c[1], j - 2, n);
-    zs[j] = wrap_near(c[2], j - 2, n);
+    yo[j] = (uint32_t)wrap_near<POW2>(c[1], j - 2, n) * (uint32_t)n;
+    zo[j] = (uint32_t)wrap_near<POW2>(c[2], j - 2, n) * (uint32_t)(n * n);
   }
-  // (y, z) row starts; indices < 2^30 for n <= 1024
-  auto row = [&](int y, int z) { return ((uint32_t)z * (uint32_t)n + (uint32_t)y) * (uint32_t)n; };
   T px[2][2][6];   // [dz][dy][x0-2 .. x0+3]
   T py[2][2][4];   // [dz][dx][y0-2, y0-1, y0+2, y0+3]
   T pz[2][2][4];   // [dy][dx][z0-2, z0-1, z0+2, z0+3]
   constexpr int kFar[4] = {0, 1, 4, 5};
-  // FP32 x runs away from the row ends: aligned 8-byte loads from a = (x0 - 2)
-  // rounded down to even cover x0 - 2 .. x0 + 3 (three loads, a fourth when
-  // x0 is odd), picked by o = (x0 - 2) & 1
-  const int a2 = (c[0] - 2) & ~1;
-  if (sizeof(T) == 4 && c[0] >= 2 && a2 + 8 <= n) {
-    const int o = (c[0] - 2) & 1;
+  // (FP64 takes the wrapped indices throughout: its bound is the FP64 pipe, and
+  // both branches' 56 values in flight would spill)
+  if (sizeof(T) == 4 && c[0] >= 2 && c[0] + 4 <= n) {
+    const T* b = phi + c[0];
+    const int odd = c[0] & 1;
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
       for (int dy = 0; dy < 2; ++dy) {
-        const float2* r2 = reinterpret_cast<const float2*>(phi + row(ys[2 + dy], zs[2 + dz]) + a2);
-        const float2 q0 = r2[0], q1 = r2[1], q2 = r2[2];
-        const float2 q3 = o ? r2[3] : make_float2(0.0f, 0.0f);
+        const T* r = b + (zo[2 + dz] + yo[2 + dy]);
+        const float2* r2 = reinterpret_cast<const float2*>(r - odd);
+        const float2 q0 = r2[-1], q1 = r2[0], q2 = r2[1];
+        const float2 q3 = odd ? r2[2] : make_float2(0.0f, 0.0f);
         const float w8[8] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y};
 #pragma unroll
-        for (int j = 0; j < 6; ++j) px[dz][dy][j] = (T)(o ? w8[j + 1] : w8[j]);
+        for (int j = 0; j < 6; ++j) px[dz][dy][j] = (T)(odd ? w8[j + 1] : w8[j]);
+      }
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const T* r = b + (zo[2 + dz] + yo[kFar[q]]);
+        py[dz][0][q] = r[0];
+        py[dz][1][q] = r[1];
+      }
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const T* r = b + (zo[kFar[q]] + yo[2 + dy]);
+        pz[dy][0][q] = r[0];
+        pz[dy][1][q] = r[1];
       }
   } else {
+    int xs[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) xs[j] = wrap_near<POW2>(c[0], j - 2, n);
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
       for (int dy = 0; dy < 2; ++dy) {
-        const T* r = phi + row(ys[2 + dy], zs[2 + dz]);
+        const T* r = phi + (zo[2 + dz] + yo[2 + dy]);
 #pragma unroll
         for (int j = 0; j < 6; ++j) px[dz][dy][j] = r[xs[j]];
       }
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const T* r = phi + (zo[2 + dz] + yo[kFar[q]]);
+        py[dz][0][q] = r[xs[2]];
+        py[dz][1][q] = r[xs[3]];
+      }
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const T* r = phi + (zo[kFar[q]] + yo[2 + dy]);
+        pz[dy][0][q] = r[xs[2]];
+        pz[dy][1][q] = r[xs[3]];
+      }
   }
-#pragma unroll
-  for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const T* r = phi + row(ys[kFar[q]], zs[2 + dz]);
-      py[dz][0][q] = r[xs[2]];
-      py[dz][1][q] = r[xs[3]];
-    }
-#pragma unroll
-  for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const T* r = phi + row(ys[2 + dy], zs[kFar[q]]);
-      pz[dy][0][q] = r[xs[2]];
-      pz[dy][1][q] = r[xs[3]];
-    }
   const StencilWeights<T> W(w);
   a[0] = a[1] = a[2] = (T)0;
 #pragma unroll
@@ -1065,7 +1102,7 @@ inline int gather_per(int64_t np, int sm_count) {
 }
 
 // Body: chunk `chunk` of kGatherTPB x per particles (blockDim = kGatherTPB).
-template <typename T>
+template <typename T, bool POW2>
 __device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, int64_t np, int n,
                                                 const CellSize& cell, const T* __restrict__ phi, T* __restrict__ vel, T kick,
                                                 T* __restrict__ acc_out, int* status, int64_t chunk, int per) {
@@ -1083,9 +1120,9 @@ __device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, in
     if (u + 1 < per && p + kGatherTPB < np) next = Quant<T>::load(pos, np, p + kGatherTPB);
     const T u0 = vel[p], u1 = vel[np + p], u2 = vel[2 * np + p];
     int c[3], w[3];
-    if (!Quant<T>::get(raw, n, cell, c, w, status)) continue;
+    if (!Quant<T>::template get<POW2>(raw, n, cell, c, w, status)) continue;
     T a[3];
-    fd_stencil<T>(phi, n, c, w, a);
+    fd_stencil<T, POW2>(phi, n, c, w, a);
     const T uu[3] = {u0, u1, u2};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -1096,11 +1133,11 @@ __device__ __forceinline__ void interp_fd_chunk(const void* __restrict__ pos, in
   }
 }
 
-template <typename T>
+template <typename T, bool POW2>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 12 : 8)
 k_interp_kick_fd(const void* __restrict__ pos, int64_t np, int n, CellSize cell, const T* __restrict__ phi,
                  T* __restrict__ vel, T kick, T* __restrict__ acc_out, int* status, int per) {
-  interp_fd_chunk<T>(pos, np, n, cell, phi, vel, kick, acc_out, status, blockIdx.x, per);
+  interp_fd_chunk<T, POW2>(pos, np, n, cell, phi, vel, kick, acc_out, status, blockIdx.x, per);
 }
 
 // The same gather in the row order of the deposit's sort: one warp per grid
@@ -1113,7 +1150,7 @@ k_interp_kick_fd(const void* __restrict__ pos, int64_t np, int n, CellSize cell,
 // (its warps round robin), dispatched in order as the particle-order gather.
 constexpr int kRowsPerCta = 8;
 
-template <typename T>
+template <typename T, bool POW2>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 10 : 8)
 k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start,
                  const int* __restrict__ perm, int64_t np, int n, T scale, const T* __restrict__ phi,
@@ -1132,7 +1169,7 @@ k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restri
       const int c[3] = {(int)(r >> 48) & 0x7ff, cy, cz};
       const int w[3] = {(int)(r & 0xffffu), (int)((r >> 16) & 0xffffu), (int)((r >> 32) & 0xffffu)};
       T a[3];
-      fd_stencil<T>(phi, n, c, w, a);
+      fd_stencil<T, POW2>(phi, n, c, w, a);
       const T u[3] = {u0, u1, u2};
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -1157,7 +1194,7 @@ k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restri
 // gather), CTAs dispatched in index order.  The CTA finds the row of its first
 // record by bisection of row_start; each thread then advances its row as its
 // records advance (rows are sorted), so empty rows cost nothing.
-template <typename T>
+template <typename T, bool POW2>
 __global__ void __launch_bounds__(kGatherTPB, sizeof(T) == 4 ? 12 : 8)
 k_interp_rows_acc(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start, int n,
                   T scale, const T* __restrict__ phi, T* __restrict__ accs) {
@@ -1186,7 +1223,7 @@ k_interp_rows_acc(const unsigned long long* __restrict__ rec, const int* __restr
     const int c[3] = {(int)(rr >> 48) & 0x7ff, cy, cz};
     const int w[3] = {(int)(rr & 0xffffu), (int)((rr >> 16) & 0xffffu), (int)((rr >> 32) & 0xffffu)};
     T a[3];
-    fd_stencil<T>(phi, n, c, w, a);
+    fd_stencil<T, POW2>(phi, n, c, w, a);
     if constexpr (sizeof(T) == 4) {
       reinterpret_cast<float4*>(accs)[i] = make_float4(a[0] * scale, a[1] * scale, a[2] * scale, 0.0f);
     } else {
@@ -1235,9 +1272,9 @@ __global__ void k_fd_force_field(const T* __restrict__ phi, int n, int comp, dou
     int idx[5];
 #pragma unroll
     for (int o = -2; o <= 2; ++o) {
-      const int xx = comp == 0 ? wrap_near(x, o, n) : x;
-      const int yy = comp == 1 ? wrap_near(y, o, n) : y;
-      const int zz = comp == 2 ? wrap_near(z, o, n) : z;
+      const int xx = comp == 0 ? wrap_index(x + o, n) : x;
+      const int yy = comp == 1 ? wrap_index(y + o, n) : y;
+      const int zz = comp == 2 ? wrap_index(z + o, n) : z;
       idx[o + 2] = (zz * n + yy) * n + xx;
     }
     out[i] = scale * ((phi[idx[0]] - phi[idx[4]]) + (T)8 * (phi[idx[3]] - phi[idx[1]]));
