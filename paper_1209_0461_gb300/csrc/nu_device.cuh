@@ -115,12 +115,6 @@ __device__ __forceinline__ double s_table(const NuArgs& A, double u) {
   return (2 * t3 - 3 * t2 + 1) * s0 + (t3 - 2 * t2 + t) * d0 + (-2 * t3 + 3 * t2) * s1 + (t3 - t2) * d1;
 }
 
-struct Panel {
-  double lo, hi;
-  int seg;   // history interval: -1 before node 0, j in [0, n-1) between nodes, n-1 the last
-};
-
-// One warp per (bin, species, chunk of 32 panels): partial IC, J_hist, W_cur.
 // The l = 1 term of Eq. deltaI-multipole for the initial moments of Sec. 4.1
 // (delta f_1 = f_0' m a_i theta / k), K(y) = -(1/y) int u^2 f'(u) j_1(u y) du /
 // ((3/2) zeta(3)), f = 1 / (e^u + 1), by Gauss-Legendre panels on [0, 50] of
@@ -129,6 +123,10 @@ struct Panel {
 // Beyond y = kMultipoleYMax (where K < 1e-10) the integrated-by-parts value
 // I(y) stands in.
 constexpr double kMultipoleYMax = 256.0;
+// 2^m, m in [-2, 1000], exactly
+__device__ __forceinline__ double exp2_int(int m) { return __hiloint2double((1023 + m) << 20, 0); }
+constexpr int kMaxGraded = 128;   // graded points looked at (ell 2^126 exceeds any ln a range)
+
 __device__ static double sph_j1(double z) {
   if (z < 1e-2) {
     const double z2 = z * z;
@@ -158,11 +156,76 @@ __device__ static double nu_K_warp(double y, const NuArgs& A, int lane) {
   return -acc / (y * 1.5 * kRelZeta3);
 }
 
-// Body: the panel chunk `item` (< nk ns kNuChunks) of (bin, species), one warp
-// (warp w of the CTA's four uses panel scratch w).
+// Break points of one bin's panels in descending order from u_e down to u_i:
+// the stored nodes and the graded points u_e - ell 2^m (m = -2, -1, ...) that
+// lie strictly between the two.  Each lane places its nodes and graded points by their
+// rank (a node's: the nodes and graded points above it; a graded point's: the
+// graded points and nodes above it, ties with the graded point first, which
+// leaves a panel of zero width).  hu: ln a_j of the n stored nodes, ascending, in
+// shared memory.  Returns the number of panels, pts[p + 1] .. pts[p] the p-th.
+// (One lane merging the two lists took most of the kernel: 150 serial steps of
+// dependent FP64 operations at 128 nodes, repeated by every warp of the bin.)
+__device__ __forceinline__ int nu_break_points(const double* hu, int n, double ue, double ui, double ell, double* pts) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  // nodes inside (u_i, u_e): [j0, j1)
+  int j0 = 0, j1 = 0;
+  for (int i = lane; i < n; i += 32) {
+    j0 += hu[i] <= ui ? 1 : 0;
+    j1 += hu[i] < ue ? 1 : 0;
+  }
+  j0 = __reduce_add_sync(full, j0);
+  j1 = __reduce_add_sync(full, j1);
+  // graded points above u_i: a prefix of m = -2, -1, ... (they fall with m)
+  int G = 0;
+  for (int base = 0; base < kMaxGraded; base += 32) {
+    const bool in = ue - ell * exp2_int(base + lane - 2) > ui;
+    const unsigned m = __ballot_sync(full, in);
+    G += __popc(m);
+    if (m != full) break;
+  }
+  if (G > kMaxGraded) G = kMaxGraded;
+  const int room = kMaxPanels - 1;   // entries after u_e, u_i included
+  int np = j1 - j0 + G + 1;
+  if (np > room) np = room;
+  if (lane == 0) pts[0] = ue;
+  for (int g = lane; g < G; g += 32) {
+    const double u = ue - ell * exp2_int(g - 2);
+    int lo = j0, hi = j1;                // nodes above u: [lo, j1)
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (hu[mid] > u) hi = mid; else lo = mid + 1;
+    }
+    const int r = 1 + g + (j1 - lo);
+    if (r < np) pts[r] = u;
+  }
+  for (int j = j0 + lane; j < j1; j += 32) {
+    const double u = hu[j];
+    int lo = 0, hi = G;                  // graded points at or above u: [0, lo)
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (ue - ell * exp2_int(mid - 2) >= u) lo = mid + 1; else hi = mid;
+    }
+    const int r = 1 + (j1 - 1 - j) + lo;
+    if (r < np) pts[r] = u;
+  }
+  if (lane == 0) pts[np] = ui;
+  __syncwarp();
+  return ue > ui ? np : 0;
+}
+
+// Body: chunk `item` (< nk ns kNuChunks) of a (bin, species), one warp (warp w
+// of the CTA's four uses scratch w).  The panels' quadrature points are dealt
+// out as (panel, node) pairs i = p Q + q, 32 a warp step, over the bin's
+// chunks, so that a few panels still fill many warps (the FP64 chain of one
+// point is long: exp, a square root, the s table and I(x)).
 __device__ __forceinline__ void nu_panels_item(const NuArgs& A, int item) {
-  __shared__ Panel panels[4][kMaxPanels];
-  __shared__ int npan[4];
+  __shared__ double pts_s[4][kMaxPanels + 1];
+  __shared__ double hu_s[kMaxPanels];
+  __syncthreads();   // (batched form: the previous item is done with the scratch)
+  const int n = A.n_hist;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) hu_s[i] = A.hist_u[i];
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (item >= A.nk * A.ns * kNuChunks) return;
   const int chunk = item % kNuChunks;
@@ -180,86 +243,48 @@ __device__ __forceinline__ void nu_panels_item(const NuArgs& A, int item) {
   const double kappa = kb * A.kappa_scale[s];
   const double Ha = A.rel ? sqrt(rel_e2(A.a, A.bg)) : sqrt(A.omega_m * exp(-3.0 * A.ue) + A.omega_l);
   const double ell = (kappa > 0.0) ? A.a * A.a * Ha / kappa : 1e300;
-  const int n = A.n_hist;
-  Panel* P = panels[warp];
-  if (lane == 0) {
-    // merge (descending from ln a): history nodes inside (u_i, u_e) and graded points
-    int np = 0;
-    double cur = A.ue;
-    int j = n - 1;                       // next history node below cur
-    while (j >= 0 && !(A.hist_u[j] < A.ue)) --j;
-    int mexp = -2;
-    double gpt = A.ue - ell * ldexp(1.0, mexp);
-    while (cur > A.ui && np < kMaxPanels) {
-      const double hn = (j >= 0 && A.hist_u[j] > A.ui) ? A.hist_u[j] : A.ui;
-      const double gp = (gpt > A.ui) ? gpt : A.ui;
-      const double nxt = hn > gp ? hn : gp;
-      // the interval index of (nxt, cur): the history node at or below nxt
-      P[np].lo = nxt;
-      P[np].hi = cur;
-      P[np].seg = j;                     // cur lies above node j (or below node 0 if j < 0)
-      ++np;
-      if (nxt == hn && j >= 0 && A.hist_u[j] > A.ui) --j;
-      if (nxt == gp && gpt > A.ui) {
-        ++mexp;
-        gpt = A.ue - ell * ldexp(1.0, mexp);
-      }
-      while (gpt >= nxt && gpt > A.ui) {   // skip graded points at or above the new cur
-        ++mexp;
-        gpt = A.ue - ell * ldexp(1.0, mexp);
-      }
-      cur = nxt;
-    }
-    npan[warp] = np;
-  }
-  __syncwarp();
-  const int np = npan[warp];
+  double* pts = pts_s[warp];
+  const int np = nu_break_points(hu_s, n, A.ue, A.ui, ell, pts);
   const int Q = A.quad;
   double jh = 0.0, wc = 0.0;
-  for (int pi = chunk * 32 + lane; pi < np; pi += 32 * A.nchunks) {
-    const Panel pn = P[pi];
-    if (!(pn.hi > pn.lo)) continue;
-    const double half = 0.5 * (pn.hi - pn.lo);
+  for (int i = chunk * 32 + lane; i < np * Q; i += 32 * A.nchunks) {
+    const int p = i / Q, q = i - p * Q;
+    const double hi = pts[p], lo = pts[p + 1];
+    if (!(hi > lo)) continue;
+    const double half = 0.5 * (hi - lo);
     // P_M^{1/2} on this panel: h(u) = h0 + (h1 - h0) (u - u0) / (u1 - u0) (history part)
-    // plus the current-node hat on the last interval
-    const int seg = pn.seg;
-    double u0 = 0.0, u1 = 1.0, h0 = 0.0, h1 = 0.0;
-    bool last = false, before = false;
-    if (n == 0) {
-      last = true;                      // h == h_cur on [u_i, u_e]
-    } else if (seg < 0) {
-      before = true;                    // constant h_0 before the first node
-      h0 = A.hist[b];
-    } else if (seg == n - 1) {
-      last = true;
-      u0 = A.hist_u[n - 1];
-      u1 = A.ue;
-      h0 = A.hist[(int64_t)(n - 1) * A.nk + b];
-    } else {
-      u0 = A.hist_u[seg];
-      u1 = A.hist_u[seg + 1];
-      h0 = A.hist[(int64_t)seg * A.nk + b];
-      h1 = A.hist[(int64_t)(seg + 1) * A.nk + b];
+    // plus the current-node hat on the last interval; seg: the last node below hi
+    int l = 0, r = n;
+    while (l < r) {
+      const int mid = (l + r) >> 1;
+      if (hu_s[mid] < hi) l = mid + 1; else r = mid;
     }
-    for (int q = 0; q < Q; ++q) {
-      const double u = pn.lo + half * (A.gl[q] + 1.0);
-      const double wq = half * A.gl[kMaxQuad + q];
-      const double ap = exp(u);
-      const double Hp = A.rel ? sqrt(rel_e2(ap, A.bg)) : sqrt(A.omega_m / (ap * ap * ap) + A.omega_l);
-      const double ds = s_end - s_table(A, u);
-      const double x = kappa * ds;
-      const double I = A.use_fit ? nu_I_fit(x) : nu_I_table(x, A.icheb);
-      const double base = wq * I * ds / (ap * Hp);
-      if (n == 0) {
-        wc += base;
-      } else if (before) {
-        jh += base * h0;
-      } else if (last) {
-        const double tau = (u - u0) / (u1 - u0);
+    const int seg = l - 1;
+    const double u = lo + half * (A.gl[q] + 1.0);
+    const double wq = half * A.gl[kMaxQuad + q];
+    const double ap = exp(u);
+    // 1 / (a H): a H = sqrt(Omega_M / a + Omega_L a^2) for matter + Lambda
+    double iaH;
+    if (A.rel) iaH = 1.0 / (ap * sqrt(rel_e2(ap, A.bg)));
+    else iaH = rsqrt(A.omega_m / ap + A.omega_l * (ap * ap));
+    const double ds = s_end - s_table(A, u);
+    const double x = kappa * ds;
+    const double I = A.use_fit ? nu_I_fit(x) : nu_I_table(x, A.icheb);
+    const double base = wq * I * ds * iaH;
+    if (n == 0) {                       // h == h_cur on [u_i, u_e]
+      wc += base;
+    } else if (seg < 0) {               // constant h_0 before the first node
+      jh += base * A.hist[b];
+    } else {
+      const bool last = seg == n - 1;
+      const double u0 = hu_s[seg], u1 = last ? A.ue : hu_s[seg + 1];
+      const double h0 = A.hist[(int64_t)seg * A.nk + b];
+      const double tau = (u - u0) / (u1 - u0);
+      if (last) {
         jh += base * h0 * (1.0 - tau);
         wc += base * tau;
       } else {
-        const double tau = (u - u0) / (u1 - u0);
+        const double h1 = A.hist[(int64_t)(seg + 1) * A.nk + b];
         jh += base * (h0 + (h1 - h0) * tau);
       }
     }
@@ -331,7 +356,7 @@ __device__ __forceinline__ void nu_finish_bin(const NuArgs& A, int b) {
 // Compacted (ln k_b, R_b) of the non-empty bins, in bin order, for the Green
 // and fac tables: rlist[0..c) = ln k_b, rlist[nk..nk+c) = R_b, rlist[2 nk] = c.
 // One block of nk <= 1024 threads.
-__device__ __forceinline__ void nu_rlist_block(const double* __restrict__ bins, const double* __restrict__ R, int nk,
+__device__ __forceinline__ void nu_rlist_block(const double* bins, const double* R, int nk,
                                                double* __restrict__ rlist) {
   __shared__ int warp_cnt[32];
   const int b = threadIdx.x, lane = b & 31, warp = b >> 5;

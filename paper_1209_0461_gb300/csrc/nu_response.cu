@@ -27,18 +27,18 @@ namespace nupm {
 
 __global__ void k_nu_panels(NuArgs A) { nu_panels_item(A, blockIdx.x * 4 + (threadIdx.x >> 5)); }
 
-__global__ void k_nu_finish(NuArgs A) { nu_finish_bin(A, blockIdx.x * blockDim.x + threadIdx.x); }
+// Finish of every bin and the list of the non-empty ones, in one CTA (nk <= 1024).
+__global__ void __launch_bounds__(1024) k_nu_finish(NuArgs A) {
+  nu_finish_bin(A, threadIdx.x);
+  __syncthreads();
+  nu_rlist_block(A.bins, A.R, A.nk, A.rlist);
+}
 
 // Fixed-order sum of the per-CTA bin partials: out[i] = sum_blk partials[blk][i]
 // (bin_reduce_group: a CTA of kReduceWarps warps, 32 outputs).
 __global__ void __launch_bounds__(kReduceWarps * 32) k_bin_reduce(const double* __restrict__ partials, int nblk,
                                                                  int len, double* __restrict__ out) {
   bin_reduce_group(partials, nblk, len, out, blockIdx.x * 32);
-}
-
-__global__ void k_nu_rlist(const double* __restrict__ bins, const double* __restrict__ R, int nk,
-                           double* __restrict__ rlist) {
-  nu_rlist_block(bins, R, nk, rlist);
 }
 
 // Chebyshev pieces of I(x) (nu_I_table): block s evaluates the exact I at the
@@ -64,8 +64,7 @@ void launch_nu_panels(const NuArgs& a, cudaStream_t s) {
 }
 
 void launch_nu_finish(const NuArgs& a, cudaStream_t s) {
-  k_nu_finish<<<(a.nk + 127) / 128, 128, 0, s>>>(a);
-  k_nu_rlist<<<1, ((a.nk + 31) / 32) * 32, 0, s>>>(a.bins, a.R, a.nk, a.rlist);
+  k_nu_finish<<<1, ((a.nk + 31) / 32) * 32, 0, s>>>(a);
 }
 
 void launch_nu_response(const NuArgs& a, cudaStream_t s) {
@@ -74,58 +73,66 @@ void launch_nu_response(const NuArgs& a, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- surrogate
-// Features of bin b for the learned response (FP64, one thread per bin):
+// Features of bin b for the learned response (FP64, eight lanes per bin, one
+// Chebyshev point each):
 //   (ln k_b, ln a, M_nu, Omega_nu, c_0 .. c_7), c_j the Chebyshev coefficients
 // on 8 points of g(u) = ln(P_M^{1/2}(u) / P_cdm^{1/2}(a)), u = ln a' in
 // [ln a_i, ln a]; P_M^{1/2} linear in u between the nodes (hist_u[j], hist[j][b])
-// closed by (ln a, P_cdm^{1/2}), constant before the first node.
+// closed by (ln a, P_cdm^{1/2}), constant before the first node.  The lanes find
+// their node by bisection and exchange g by shuffles (one thread a bin, with a
+// linear search per point, took 101 us at 256 bins and 128 nodes: a chain of
+// dependent loads).
 __global__ void k_nu_features(NuArgs A, double m_nu, double omega_nu, float* __restrict__ X) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= A.nk) return;
-  float* row = X + (int64_t)b * 12;
+  // cos(pi k / 16), k = 0 .. 16
+  constexpr double kCos16[17] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                                 0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                                 0.19509032201612826785, 0.0, -0.19509032201612826785, -0.38268343236508977173,
+                                 -0.55557023301960222474, -0.70710678118654752440, -0.83146961230254523708,
+                                 -0.92387953251128675613, -0.98078528040323044913, -1.0};
+  __shared__ double c16[32];
+  if (threadIdx.x < 32) c16[threadIdx.x] = kCos16[threadIdx.x <= 16 ? threadIdx.x : 32 - threadIdx.x];
+  __syncthreads();
+  const int b0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, m = threadIdx.x & 7;
+  const int b = b0 < A.nk ? b0 : A.nk - 1;          // whole groups of eight take part in the shuffles
   const double cnt = A.bins[b];
-  if (!(cnt > 0.0)) {
-    for (int i = 0; i < 12; ++i) row[i] = 0.0f;
-    return;
-  }
+  const bool some = cnt > 0.0;
   const double L3 = A.box * A.box * A.box;
   const double n3 = (double)A.ngrid * A.ngrid * A.ngrid;
-  const double pcdm = sqrt(A.bins[2 * A.nk + b] / cnt * L3 / (n3 * n3));
-  const double kb = A.bins[A.nk + b] / cnt;
-  double g[8];
-  for (int m = 0; m < 8; ++m) {
-    const double t = cospi((m + 0.5) / 8.0);
-    const double u = A.ui + 0.5 * (t + 1.0) * (A.ue - A.ui);
-    double h = pcdm;
-    if (A.n_hist > 0) {
-      if (u <= A.hist_u[0]) {
-        h = A.hist[b];
-      } else {
-        int j = 0;
-        while (j + 1 < A.n_hist && A.hist_u[j + 1] < u) ++j;
-        const double u0 = A.hist_u[j], h0 = A.hist[(int64_t)j * A.nk + b];
-        const double u1 = j + 1 < A.n_hist ? A.hist_u[j + 1] : A.ue;
-        const double h1 = j + 1 < A.n_hist ? A.hist[(int64_t)(j + 1) * A.nk + b] : pcdm;
-        h = h0 + (h1 - h0) * (u - u0) / (u1 - u0);
-      }
+  const double pcdm = some ? sqrt(A.bins[2 * A.nk + b] / cnt * L3 / (n3 * n3)) : 0.0;
+  const double u = A.ui + 0.5 * (c16[2 * m + 1] + 1.0) * (A.ue - A.ui);
+  double h = pcdm;
+  if (A.n_hist > 0) {
+    int lo = 0, hi = A.n_hist;                      // nodes below u: [0, lo)
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (A.hist_u[mid] < u) lo = mid + 1; else hi = mid;
     }
-    g[m] = (h > 0.0 && pcdm > 0.0) ? log(h / pcdm) : 0.0;
+    if (lo == 0) {
+      h = A.hist[b];
+    } else {
+      const int j = lo - 1;
+      const double u0 = A.hist_u[j], h0 = A.hist[(int64_t)j * A.nk + b];
+      const double u1 = lo < A.n_hist ? A.hist_u[lo] : A.ue;
+      const double h1 = lo < A.n_hist ? A.hist[(int64_t)lo * A.nk + b] : pcdm;
+      h = h0 + (h1 - h0) * (u - u0) / (u1 - u0);
+    }
   }
-  row[0] = (float)log(kb);
-  row[1] = (float)A.ue;
-  row[2] = (float)m_nu;
-  row[3] = (float)omega_nu;
-  for (int jc = 0; jc < 8; ++jc) {
-    double c = 0.0;
-    for (int m = 0; m < 8; ++m) c += g[m] * cospi(jc * (m + 0.5) / 8.0);
-    row[4 + jc] = (float)(0.25 * c);
+  const double g = (h > 0.0 && pcdm > 0.0) ? log(h / pcdm) : 0.0;
+  double c = 0.0;                                   // lane m holds coefficient c_m
+#pragma unroll
+  for (int k = 0; k < 8; ++k) c += __shfl_sync(0xffffffffu, g, k, 8) * c16[(m * (2 * k + 1)) & 31];
+  if (b0 >= A.nk) return;
+  float* row = X + (int64_t)b * 12;
+  row[4 + m] = some ? (float)(0.25 * c) : 0.0f;
+  if (m < 4) {
+    const double v = m == 0 ? (some ? log(A.bins[A.nk + b] / cnt) : 0.0) : m == 1 ? A.ue : m == 2 ? m_nu : omega_nu;
+    row[m] = some ? (float)v : 0.0f;
   }
 }
 
 // R_b = exp(ln R_b) from the surrogate, then P_nu^{1/2} and P_M^{1/2} as the
 // exact finish does (empty bins: 0).
-__global__ void k_nu_from_lnR(NuArgs A, const float* __restrict__ lnR) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void from_lnR_bin(const NuArgs& A, const float* __restrict__ lnR, int b) {
   if (b >= A.nk) return;
   const double cnt = A.bins[b];
   double R = 0.0, pnu = 0.0, pm = 0.0;
@@ -145,13 +152,18 @@ __global__ void k_nu_from_lnR(NuArgs A, const float* __restrict__ lnR) {
   if (A.pm_user) A.pm_user[b] = pm;
 }
 
+__global__ void __launch_bounds__(1024) k_nu_from_lnR(NuArgs A, const float* __restrict__ lnR) {
+  from_lnR_bin(A, lnR, threadIdx.x);
+  __syncthreads();
+  nu_rlist_block(A.bins, A.R, A.nk, A.rlist);
+}
+
 void launch_nu_features(const NuArgs& a, double m_nu, double omega_nu, float* X, cudaStream_t s) {
-  k_nu_features<<<(a.nk + 127) / 128, 128, 0, s>>>(a, m_nu, omega_nu, X);
+  k_nu_features<<<(a.nk * 8 + 127) / 128, 128, 0, s>>>(a, m_nu, omega_nu, X);
 }
 
 void launch_nu_from_lnR(const NuArgs& a, const float* lnR, cudaStream_t s) {
-  k_nu_from_lnR<<<(a.nk + 127) / 128, 128, 0, s>>>(a, lnR);
-  k_nu_rlist<<<1, ((a.nk + 31) / 32) * 32, 0, s>>>(a.bins, a.R, a.nk, a.rlist);
+  k_nu_from_lnR<<<1, ((a.nk + 31) / 32) * 32, 0, s>>>(a, lnR);
 }
 
 // ---------------------------------------------------------------- Green table

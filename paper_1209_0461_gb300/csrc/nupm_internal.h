@@ -16,7 +16,7 @@ constexpr double kTnu0eV = 1.68e-4;       // T_nu,0 [eV], Sec. 2.1 (value as pri
 constexpr double kOmegaNuEv = 93.14;      // Omega_nu h^2 = sum m / 93.14 eV, Sec. 2.1
 constexpr int kMaxQuad = 16;
 constexpr int kMaxPanels = 320;           // history nodes + graded points + ends
-constexpr int kNuChunks = 10;             // warps per (bin, species), 32 panels each
+constexpr int kNuChunks = 10;             // warps per (bin, species) at most (nu_panels_item)
 
 // Integer n^2 thresholds of the |k| bins: T_b = ceil((e_b L / 2 pi)^2), b = 0..nk,
 // for edges e_b log-spaced on [2 pi / L, sqrt(3) pi N / L (1 + 1e-12)]; a mode is in

@@ -1019,8 +1019,9 @@ NuArgs nu_args(pm_ctx* c, double a, const double* sqrtPM_hist, int32_t n_hist, c
   // panel chunks in use: the panels are the history nodes, the graded points
   // a - ell 2^m (m >= -2) above a_i, at most log2((ln a - ln a_i) / ell) + 3 of
   // them with ell = a^2 H / kappa smallest at the largest |k| of the grid, and
-  // the ends; 32 panels a chunk.  A chunk's warp strides over the panels by the
-  // chunk count, so the bound sets the split of the work, not which panels count.
+  // the ends; quad nodes a panel, 32 (panel, node) points a chunk.  A chunk's warp
+  // strides over the points by the chunk count, so the bound sets the split of the
+  // work, not which points count.
   {
     double kap = 0.0;
     for (int s = 0; s < c->ns; ++s) kap = A.kappa_scale[s] > kap ? A.kappa_scale[s] : kap;
@@ -1030,7 +1031,7 @@ NuArgs nu_args(pm_ctx* c, double a, const double* sqrtPM_hist, int32_t n_hist, c
       const double r = (A.ue - A.ui) * kap / (a * a * hubble(c, a));
       npan += 3 + (r > 1.0 ? (int)ceil(log2(r)) : 0);
     }
-    const int ch = (npan + 31) / 32;
+    const int ch = (npan * c->quad + 31) / 32;
     A.nchunks = ch < 1 ? 1 : (ch > kNuChunks ? kNuChunks : ch);
   }
   A.parts = c->d_parts;
@@ -1085,7 +1086,7 @@ int pm_nu_response(pm_ctx* c, double a, const double* a_hist, const double* sqrt
     return fail(c, PM_ERR_ORDER, "pm_nu_response before pm_deposit");
   }
   const bool nu = c->ns > 0 && c->f_nu > 0;
-  Stage stage(c, PM_ST_RESPONSE, (nu && !use_prep ? 1 : 0) + 3);   // [panels,] finish, bin list, table
+  Stage stage(c, PM_ST_RESPONSE, (nu && !use_prep ? 1 : 0) + 2);   // [panels,] finish + bin list, table
   NuArgs A = nu_args(c, a, sqrtPM_hist, n_hist, sqrtPnu_prev, ratio_out, sqrtPnu_out, sqrtPM_out);
   if (use_prep) A.hist_u = c->d_hist_u2;
   if (nu && !use_prep) launch_nu_panels(A, c->stream);
@@ -1165,7 +1166,7 @@ int pm_nu_response_mlp(pm_ctx* c, pm_mlp* mlp, double a, const double* a_hist, c
   int rc = response_prepare(c, a, a_hist, sqrtPM_hist, n_hist);
   if (rc != PM_OK) return rc;
   NuArgs A = surrogate_args(c, a, sqrtPM_hist, n_hist, ratio_out, sqrtPnu_out, sqrtPM_out);
-  Stage stage(c, PM_ST_RESPONSE, (c->ns > 0 && c->f_nu > 0) ? 4 : 2);
+  Stage stage(c, PM_ST_RESPONSE, (c->ns > 0 && c->f_nu > 0) ? 4 : 2);   // features, network, finish + list, table
   if (c->ns > 0 && c->f_nu > 0) {
     launch_nu_features(A, c->p.m_nu_total_eV, c->omega_nu, c->d_X, c->stream);
     rc = mlp_forward_on(mlp, c->d_X, c->nk, c->d_lnR, c->stream);
