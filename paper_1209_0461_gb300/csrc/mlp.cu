@@ -7,11 +7,13 @@
 // Layout of the flat parameter vector (FP32 master copy):
 //   W1 [128][n_in], b1 [128], W2 [128][128], b2 [128], w3 [128], b3 [1]
 //
-// Kernels (one CTA of 128 threads per SM, persistent over tiles of 32
-// samples; thread j owns hidden unit j of both layers):
-//   k_mlp_forward   y = y_mu + y_sigma * out(x)                 (inference)
-//   k_mlp_backward  per-CTA partial gradients and loss, fixed tile order
-//   k_mlp_reduce    sum of the CTA partials in CTA order (deterministic)
+// Kernels:
+//   k_mlp_forward   y = y_mu + y_sigma * out(x): a warp per 16 samples, layer 2
+//                   on the tensor cores from activations split in three BF16
+//   k_mlp_backward  per-CTA partial gradients and loss, fixed tile order; one CTA
+//                   of 256 threads per SM, tiles of 32 samples, register tiles of
+//                   two hidden units x eight samples (FP32)
+//   k_mlp_reduce    sum of the CTA partials in a fixed order (deterministic)
 //   k_mlp_adam      Adam on the master copy, then the BF16 weight copies
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -29,21 +31,39 @@ namespace {
 
 constexpr int kW = 128;        // hidden width
 constexpr int kMaxIn = 16;     // input features (<=)
-constexpr int kTS = 32;        // samples per tile
+constexpr int kTS = 32;        // samples per tile of the backward pass
 constexpr int kHP = 36;        // padded row of the [unit][sample] tiles (16-byte rows)
-constexpr int kWP = 129;       // padded row of the 128x128 shared matrices
+constexpr int kWP = 129;       // padded row of the 128x128 shared matrix
+constexpr int kBwdThreads = 256;
 
-// Shared-memory layout (floats) of the two kernels.
+// Shared-memory layout (floats) of the backward kernel.
 struct MlpSmem {
   static constexpr int W2 = 0;                        // W2s[k][j] = W2[j][k], rows of kWP
-  static constexpr int DW2 = W2 + kW * kWP;            // dW2 partial, same layout
-  static constexpr int H1 = DW2 + kW * kWP;            // h1T[k][s], rows of kHP
+  static constexpr int H1 = W2 + kW * kWP;             // h1T[k][s], rows of kHP
   static constexpr int DZ2 = H1 + kW * kHP;            // dz2T[j][s]
   static constexpr int XH = DZ2 + kW * kHP;            // xh[s][i], rows of kMaxIn
-  static constexpr int OUT = XH + kTS * kMaxIn;        // out / dout per sample
-  static constexpr int RED = OUT + kTS;                // [4 warps][kTS] reduction
-  static constexpr int TOTAL = RED + 4 * kTS;
+  static constexpr int OUT = XH + kTS * kMaxIn;        // squared residuals
+  static constexpr int DOUT = OUT + kTS;               // dL/dout per sample
+  static constexpr int RED = DOUT + kTS;               // [8 warps][8 samples] reduction
+  static constexpr int TOTAL = RED + 64;
   static constexpr size_t BYTES = (size_t)TOTAL * sizeof(float);
+  static_assert(H1 % 4 == 0 && XH % 4 == 0, "16-byte rows");
+  static_assert(4 * kW * (kMaxIn + 3) <= TOTAL - H1, "the end sums reuse what follows W2");
+};
+
+// Shared memory of the forward kernel: W2 as B fragments of m16n8k16
+// [k tile][n tile][lane] (8 bytes), W1 rows of kW1P floats, b1, (b2, w3) pairs
+// per unit, one staging tile of 16 x kXP inputs per warp.
+constexpr int kFwdWarps = 4;
+constexpr int kW1P = 20;       // rows of two units apart by 40 words: the quads' 16-byte reads miss each other's banks
+constexpr int kXP = 20;
+struct FwdSmem {
+  static constexpr int B = 0;
+  static constexpr int W1 = B + kW * kW * 2;
+  static constexpr int B1 = W1 + kW * kW1P * 4;
+  static constexpr int BW = B1 + kW * 4;
+  static constexpr int X = BW + kW * 8;
+  static constexpr int BYTES = X + kFwdWarps * 16 * kXP * 4;
 };
 
 struct MlpArgs {
@@ -67,221 +87,389 @@ struct MlpArgs {
 
 __device__ __forceinline__ float bf(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// Forward pass of one tile of kTS samples (rows s0 .. s0 + kTS - 1; rows past
-// n are zero inputs whose results are ignored).  Leaves h1T, this thread's
-// h2[s] (unit j) and out[s] (normalised) in shared memory / registers.
-__device__ __forceinline__ void tile_forward(const MlpArgs& A, float* sm, int64_t s0, float (&h2)[kTS]) {
-  const int j = threadIdx.x, lane = j & 31, warp = j >> 5;
-  float* xh = sm + MlpSmem::XH;
-  float* h1T = sm + MlpSmem::H1;
-  const float* W2s = sm + MlpSmem::W2;
-  float* outs = sm + MlpSmem::OUT;
-  float* red = sm + MlpSmem::RED;
-  for (int idx = j; idx < kTS * kMaxIn; idx += kW) {   // unused columns and rows past n: 0
-    const int s = idx / kMaxIn, i = idx - s * kMaxIn;
-    const int64_t row = s0 + s;
-    xh[idx] = (i < A.n_in && row < A.n) ? (A.X[row * A.n_in + i] - A.mu[i]) / A.sig[i] : 0.0f;
+// h = hi + mid + lo to 2^-27 relative, each a BF16 (products with the BF16
+// weights are then exact); two neighbouring values packed per word.
+__device__ __forceinline__ void split3(float x, float y, uint32_t (&w)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(x, y);
+    w[i] = *reinterpret_cast<const uint32_t*>(&p);
+    x -= __low2float(p);
+    y -= __high2float(p);
+  }
+}
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t a0, const uint32_t a1, const uint32_t a2,
+                                         const uint32_t a3, uint2 b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
+}
+
+// One warp per 16 samples.  Lane (g, q) = (lane / 4, lane % 4) holds rows g and
+// g + 8; layer 1 is evaluated straight into the A fragments of layer 2: per k
+// tile of 16 hidden units the lane needs units 2q, 2q + 1, 2q + 8, 2q + 9 of
+// its two rows.  Layer 2, 128 x 128 with BF16 weights, runs on the tensor
+// cores with h1 as three BF16 words, so no activation is rounded; each k tile's
+// product starts from zero (low word first) and is added to the FP32 sum in
+// round-to-nearest, because the tensor cores' own accumulation truncates.
+// The warp-level mma is taken rather than a tcgen05 tile: what bounds the kernel is
+// the 256 tanh and the FP32 work of a sample, and the fragments stay in
+// registers between the layers.  500k samples take 0.248 ms (74 TFLOP/s; error
+// against 64 bits 4.8e-8); one CTA of 128 threads per SM, each thread a hidden
+// unit of 32 samples in FP32, took 1.07 ms (four warps per SM; 5.6e-8).
+__global__ void __launch_bounds__(kFwdWarps * 32, 3) k_mlp_forward(MlpArgs A) {
+  extern __shared__ __align__(16) unsigned char smf[];
+  uint2* Bs = reinterpret_cast<uint2*>(smf + FwdSmem::B);
+  float* W1s = reinterpret_cast<float*>(smf + FwdSmem::W1);
+  float* b1s = reinterpret_cast<float*>(smf + FwdSmem::B1);
+  float2* bw = reinterpret_cast<float2*>(smf + FwdSmem::BW);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+  float* xs = reinterpret_cast<float*>(smf + FwdSmem::X) + warp * 16 * kXP;
+  // fragment (kt, nt, lane): W2[8 nt + g][16 kt + 2q + {0, 1}] and + 8
+  for (int i = threadIdx.x; i < 8 * 16 * 32; i += blockDim.x) {
+    const int l = i & 31, nt = (i >> 5) & 15, kt = i >> 9;
+    const __nv_bfloat16* w = A.W2 + (8 * nt + (l >> 2)) * kW + 16 * kt + 2 * (l & 3);
+    Bs[i] = make_uint2(*reinterpret_cast<const uint32_t*>(w), *reinterpret_cast<const uint32_t*>(w + 8));
+  }
+  for (int i = threadIdx.x; i < kW * kMaxIn; i += blockDim.x) {
+    const int u = i / kMaxIn, c = i % kMaxIn;
+    W1s[u * kW1P + c] = c < A.n_in ? bf(A.W1[u * A.n_in + c]) : 0.0f;
+  }
+  for (int i = threadIdx.x; i < kW; i += blockDim.x) {
+    b1s[i] = A.b1[i];
+    bw[i] = make_float2(A.b2[i], bf(A.w3[i]));
   }
   __syncthreads();
-  // layer 1: unit j for every sample of the tile
-  {
-    float w[kMaxIn];
-#pragma unroll
-    for (int i = 0; i < kMaxIn; ++i) w[i] = i < A.n_in ? bf(A.W1[j * A.n_in + i]) : 0.0f;
-    const float b = A.b1[j];
-#pragma unroll 4
-    for (int s = 0; s < kTS; ++s) {
-      float acc = b;
-#pragma unroll
-      for (int i = 0; i < kMaxIn; ++i) acc = fmaf(w[i], xh[s * kMaxIn + i], acc);
-      h1T[j * kHP + s] = tanhf(acc);
+  const float b3 = A.b3[0];
+  const int64_t tiles = (A.n + 15) / 16;
+  for (int64_t t = (int64_t)blockIdx.x * kFwdWarps + warp; t < tiles; t += (int64_t)gridDim.x * kFwdWarps) {
+    const int64_t s0 = t * 16;
+    __syncwarp();
+    for (int i = lane; i < 16 * kMaxIn; i += 32) {   // unused columns and rows past n: 0
+      const int r = i / kMaxIn, c = i % kMaxIn;
+      const int64_t row = s0 + r;
+      xs[r * kXP + c] = (c < A.n_in && row < A.n) ? (A.X[row * A.n_in + c] - A.mu[c]) / A.sig[c] : 0.0f;
     }
-  }
-  __syncthreads();
-  // layer 2: h2[s] = tanh(b2[j] + sum_k W2[j][k] h1[s][k])
-  {
-    const float b = A.b2[j];
+    __syncwarp();
+    float x[2][kMaxIn];
 #pragma unroll
-    for (int s = 0; s < kTS; ++s) h2[s] = b;
-#pragma unroll 2
-    for (int k = 0; k < kW; ++k) {
-      const float w = W2s[k * kWP + j];
-      const float4* hk = reinterpret_cast<const float4*>(h1T + k * kHP);
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
-      for (int q = 0; q < kTS / 4; ++q) {
-        const float4 hv = hk[q];
-        h2[4 * q + 0] = fmaf(w, hv.x, h2[4 * q + 0]);
-        h2[4 * q + 1] = fmaf(w, hv.y, h2[4 * q + 1]);
-        h2[4 * q + 2] = fmaf(w, hv.z, h2[4 * q + 2]);
-        h2[4 * q + 3] = fmaf(w, hv.w, h2[4 * q + 3]);
+      for (int c = 0; c < kMaxIn; c += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(xs + (g + 8 * r) * kXP + c);
+        x[r][c] = v.x;
+        x[r][c + 1] = v.y;
+        x[r][c + 2] = v.z;
+        x[r][c + 3] = v.w;
+      }
+    float z[16][4];
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) z[nt][0] = z[nt][1] = z[nt][2] = z[nt][3] = 0.0f;
+#pragma unroll 1
+    for (int kt = 0; kt < 8; ++kt) {
+      uint32_t a[4][3];   // [fragment word][hi, mid, lo]
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {   // units 16 kt + 8 p + 2 q + {0, 1}
+        const int u = 16 * kt + 8 * p + 2 * q;
+        float h[2][2];                // [row][unit]
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float acc0 = b1s[u + e], acc1 = acc0;
+#pragma unroll
+          for (int c = 0; c < kMaxIn; c += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(W1s + (u + e) * kW1P + c);
+            acc0 = fmaf(w.x, x[0][c], acc0);
+            acc1 = fmaf(w.x, x[1][c], acc1);
+            acc0 = fmaf(w.y, x[0][c + 1], acc0);
+            acc1 = fmaf(w.y, x[1][c + 1], acc1);
+            acc0 = fmaf(w.z, x[0][c + 2], acc0);
+            acc1 = fmaf(w.z, x[1][c + 2], acc1);
+            acc0 = fmaf(w.w, x[0][c + 3], acc0);
+            acc1 = fmaf(w.w, x[1][c + 3], acc1);
+          }
+          h[0][e] = tanhf(acc0);
+          h[1][e] = tanhf(acc1);
+        }
+        split3(h[0][0], h[0][1], a[2 * p]);
+        split3(h[1][0], h[1][1], a[2 * p + 1]);
+      }
+      const uint2* bk = Bs + kt * 16 * 32 + lane;
+#pragma unroll
+      for (int nt = 0; nt < 16; ++nt) {
+        const uint2 b = bk[nt * 32];
+        float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        mma_bf16(c, a[0][2], a[1][2], a[2][2], a[3][2], b);
+        mma_bf16(c, a[0][1], a[1][1], a[2][1], a[3][1], b);
+        mma_bf16(c, a[0][0], a[1][0], a[2][0], a[3][0], b);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) z[nt][e] += c[e];
       }
     }
+    // layer 3 over the lane's 32 columns, then over the four lanes of the row
+    float o0 = 0.0f, o1 = 0.0f;
 #pragma unroll
-    for (int s = 0; s < kTS; ++s) h2[s] = tanhf(h2[s]);
-  }
-  // layer 3: out[s] = b3 + sum_j w3[j] h2[s][j], fixed reduction tree
-  const float w3j = bf(A.w3[j]);
+    for (int nt = 0; nt < 16; ++nt)
 #pragma unroll
-  for (int s = 0; s < kTS; ++s) {
-    float v = w3j * h2[s];
+      for (int e = 0; e < 2; ++e) {
+        const float2 w = bw[8 * nt + 2 * q + e];
+        o0 = fmaf(w.y, tanhf(z[nt][e] + w.x), o0);
+        o1 = fmaf(w.y, tanhf(z[nt][2 + e] + w.x), o1);
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp * kTS + s] = v;
-  }
-  __syncthreads();
-  if (j < kTS) outs[j] = A.b3[0] + ((red[j] + red[kTS + j]) + (red[2 * kTS + j] + red[3 * kTS + j]));
-  __syncthreads();
-}
-
-__device__ __forceinline__ void load_w2(const MlpArgs& A, float* sm) {
-  float* W2s = sm + MlpSmem::W2;
-  for (int idx = threadIdx.x; idx < kW * kW; idx += kW) {
-    const int jj = idx / kW, k = idx - jj * kW;          // W2[jj][k]
-    W2s[k * kWP + jj] = bf(A.W2[idx]);
-  }
-}
-
-__global__ void __launch_bounds__(kW, 1) k_mlp_forward(MlpArgs A) {
-  extern __shared__ __align__(16) float sm[];
-  load_w2(A, sm);
-  __syncthreads();
-  float h2[kTS];
-  const int64_t tiles = (A.n + kTS - 1) / kTS;
-  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int64_t s0 = t * kTS;
-    tile_forward(A, sm, s0, h2);
-    if (threadIdx.x < kTS && s0 + threadIdx.x < A.n)
-      A.out[s0 + threadIdx.x] = A.y_mu + A.y_sig * sm[MlpSmem::OUT + threadIdx.x];
-    __syncthreads();
+    for (int m = 1; m < 4; m <<= 1) {
+      o0 += __shfl_xor_sync(0xffffffffu, o0, m);
+      o1 += __shfl_xor_sync(0xffffffffu, o1, m);
+    }
+    if (q == 0) {
+      if (s0 + g < A.n) A.out[s0 + g] = A.y_mu + A.y_sig * (o0 + b3);
+      if (s0 + g + 8 < A.n) A.out[s0 + g + 8] = A.y_mu + A.y_sig * (o1 + b3);
+    }
   }
 }
 
 // Partial gradient of L = (1/n) sum (out - (Y - y_mu)/y_sig)^2 over the tiles
 // blockIdx.x, blockIdx.x + gridDim.x, ... (in that order), written to
 // partial[blockIdx.x][0..P) in the flat parameter layout, the partial loss
-// at [P].
-__global__ void __launch_bounds__(kW, 1) k_mlp_backward(MlpArgs A) {
+// at [P].  Thread (jj, sg) = (tid % 64, tid / 64) owns hidden units jj and
+// jj + 64 for the samples 8 sg .. 8 sg + 7 (layers 1 and 2 and their
+// gradients: 16 multiply-adds for two scalar and two 16-byte shared reads) and, for dW2, the
+// same two units against k = 32 sg .. 32 sg + 31 over all samples, kept in 64
+// registers across tiles.  29 us for 4096 samples; one CTA of 128 threads with
+// dW2 in shared memory, four warps per SM, took 48 us.
+__global__ void __launch_bounds__(kBwdThreads, 1) k_mlp_backward(MlpArgs A) {
   extern __shared__ __align__(16) float sm[];
-  const int j = threadIdx.x;
+  const int tid = threadIdx.x, jj = tid & 63, sg = tid >> 6, lane = tid & 31, warp = tid >> 5;
+  const int ju[2] = {jj, jj + 64};
   float* W2s = sm + MlpSmem::W2;
-  float* dW2s = sm + MlpSmem::DW2;
   float* h1T = sm + MlpSmem::H1;
   float* dz2T = sm + MlpSmem::DZ2;
   float* xh = sm + MlpSmem::XH;
   float* outs = sm + MlpSmem::OUT;
-  load_w2(A, sm);
-  for (int idx = j; idx < kW * kWP; idx += kW) dW2s[idx] = 0.0f;
-  float dW1[kMaxIn];
+  float* dout = sm + MlpSmem::DOUT;
+  float* red = sm + MlpSmem::RED;
+  for (int idx = tid; idx < kW * kW; idx += kBwdThreads) {
+    const int j = idx / kW, k = idx % kW;                // W2[j][k]
+    W2s[k * kWP + j] = bf(A.W2[idx]);
+  }
+  float dW2[2][32], dW1[2][kMaxIn], db1[2] = {0.0f, 0.0f}, db2[2] = {0.0f, 0.0f}, dw3[2] = {0.0f, 0.0f};
+  float db3 = 0.0f, loss = 0.0f, w3[2], b1[2], b2[2];
 #pragma unroll
-  for (int i = 0; i < kMaxIn; ++i) dW1[i] = 0.0f;
-  float db1 = 0.0f, db2 = 0.0f, dw3 = 0.0f, db3 = 0.0f, loss = 0.0f;
-  const float inv_n = 1.0f / (float)A.n;
-  const float w3j = bf(A.w3[j]);
-  __syncthreads();
-  float h2[kTS];
+  for (int e = 0; e < 2; ++e) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) dW2[e][k] = 0.0f;
+#pragma unroll
+    for (int i = 0; i < kMaxIn; ++i) dW1[e][i] = 0.0f;
+    w3[e] = bf(A.w3[ju[e]]);
+    b1[e] = A.b1[ju[e]];
+    b2[e] = A.b2[ju[e]];
+  }
+  const float inv_n = 1.0f / (float)A.n, b3 = A.b3[0];
   const int64_t tiles = (A.n + kTS - 1) / kTS;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int64_t s0 = t * kTS;
-    tile_forward(A, sm, s0, h2);
-    // dL/dout per sample (zero past n)
-    if (j < kTS) {
-      const int64_t row = s0 + j;
-      float d = 0.0f;
-      if (row < A.n) {
-        const float r = outs[j] - (A.Y[row] - A.y_mu) / A.y_sig;
-        d = 2.0f * r * inv_n;
-        outs[j] = r * r;       // squared residual (read by thread 0 below)
-      } else {
-        outs[j] = 0.0f;
-      }
-      sm[MlpSmem::RED + j] = d;
+    for (int idx = tid; idx < kTS * kMaxIn; idx += kBwdThreads) {   // unused columns and rows past n: 0
+      const int s = idx / kMaxIn, i = idx % kMaxIn;
+      const int64_t row = s0 + s;
+      xh[idx] = (i < A.n_in && row < A.n) ? (A.X[row * A.n_in + i] - A.mu[i]) / A.sig[i] : 0.0f;
     }
     __syncthreads();
-    if (j == 0)
-      for (int s = 0; s < kTS; ++s) loss += outs[s];
-    const float* dout = sm + MlpSmem::RED;
-    // layer 3 and the pre-activation gradient of layer 2 (unit j)
-    float dz2[kTS];
+    // layer 1
+    float h1[2][8];
 #pragma unroll
-    for (int s = 0; s < kTS; ++s) {
-      const float d = dout[s];
-      dw3 = fmaf(d, h2[s], dw3);
-      if (j == 0) db3 += d;
-      dz2[s] = d * w3j * (1.0f - h2[s] * h2[s]);
-      db2 += dz2[s];
-      dz2T[j * kHP + s] = dz2[s];
+    for (int e = 0; e < 2; ++e) {
+      float w[kMaxIn];
+#pragma unroll
+      for (int i = 0; i < kMaxIn; ++i) w[i] = i < A.n_in ? bf(A.W1[ju[e] * A.n_in + i]) : 0.0f;
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        float acc = b1[e];
+#pragma unroll
+        for (int i = 0; i < kMaxIn; ++i) acc = fmaf(w[i], xh[(8 * sg + s) * kMaxIn + i], acc);
+        h1[e][s] = tanhf(acc);
+      }
+      float4* d = reinterpret_cast<float4*>(h1T + ju[e] * kHP + 8 * sg);
+      d[0] = make_float4(h1[e][0], h1[e][1], h1[e][2], h1[e][3]);
+      d[1] = make_float4(h1[e][4], h1[e][5], h1[e][6], h1[e][7]);
     }
-    // dW2[j][k] += sum_s dz2[s] h1[s][k]
-#pragma unroll 2
+    __syncthreads();
+    // layer 2: h2[s] = tanh(b2[j] + sum_k W2[j][k] h1[s][k])
+    float h2[2][8];
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int s = 0; s < 8; ++s) h2[e][s] = b2[e];
+#pragma unroll 4
     for (int k = 0; k < kW; ++k) {
-      const float4* hk = reinterpret_cast<const float4*>(h1T + k * kHP);
-      float acc = 0.0f;
+      const float wa = W2s[k * kWP + jj], wb = W2s[k * kWP + jj + 64];
+      const float4* hk = reinterpret_cast<const float4*>(h1T + k * kHP + 8 * sg);
+      const float4 u = hk[0], v = hk[1];
+      const float hv[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int q = 0; q < kTS / 4; ++q) {
-        const float4 hv = hk[q];
-        acc = fmaf(dz2[4 * q + 0], hv.x, acc);
-        acc = fmaf(dz2[4 * q + 1], hv.y, acc);
-        acc = fmaf(dz2[4 * q + 2], hv.z, acc);
-        acc = fmaf(dz2[4 * q + 3], hv.w, acc);
+      for (int s = 0; s < 8; ++s) {
+        h2[0][s] = fmaf(wa, hv[s], h2[0][s]);
+        h2[1][s] = fmaf(wb, hv[s], h2[1][s]);
       }
-      dW2s[k * kWP + j] += acc;
+    }
+    // layer 3: out[s] = b3 + sum_j w3[j] h2[s][j], fixed reduction tree
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      h2[0][s] = tanhf(h2[0][s]);
+      h2[1][s] = tanhf(h2[1][s]);
+      float v = fmaf(w3[0], h2[0][s], w3[1] * h2[1][s]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) red[warp * 8 + s] = v;
     }
     __syncthreads();
-    // thread j now acts as layer-1 unit k = j: dh1[s] = sum_jj W2[jj][k] dz2[s][jj]
-    {
-      const int k = j;
-      float dh[kTS];
-#pragma unroll
-      for (int s = 0; s < kTS; ++s) dh[s] = 0.0f;
-#pragma unroll 2
-      for (int jj = 0; jj < kW; ++jj) {
-        const float w = W2s[k * kWP + jj];
-        const float4* dz = reinterpret_cast<const float4*>(dz2T + jj * kHP);
-#pragma unroll
-        for (int q = 0; q < kTS / 4; ++q) {
-          const float4 dv = dz[q];
-          dh[4 * q + 0] = fmaf(w, dv.x, dh[4 * q + 0]);
-          dh[4 * q + 1] = fmaf(w, dv.y, dh[4 * q + 1]);
-          dh[4 * q + 2] = fmaf(w, dv.z, dh[4 * q + 2]);
-          dh[4 * q + 3] = fmaf(w, dv.w, dh[4 * q + 3]);
-        }
+    // dL/dout per sample (zero past n)
+    if (tid < kTS) {
+      const int64_t row = s0 + tid;
+      const int w0 = 2 * (tid >> 3) * 8 + (tid & 7);
+      float d = 0.0f, r2 = 0.0f;
+      if (row < A.n) {
+        const float r = b3 + (red[w0] + red[w0 + 8]) - (A.Y[row] - A.y_mu) / A.y_sig;
+        d = 2.0f * r * inv_n;
+        r2 = r * r;
       }
-#pragma unroll
+      dout[tid] = d;
+      outs[tid] = r2;
+    }
+    __syncthreads();
+    if (tid == 0)
       for (int s = 0; s < kTS; ++s) {
-        const float h = h1T[k * kHP + s];
-        const float dz1 = dh[s] * (1.0f - h * h);
-        db1 += dz1;
+        loss += outs[s];
+        db3 += dout[s];
+      }
+    // the pre-activation gradient of layer 2
 #pragma unroll
-        for (int i = 0; i < kMaxIn; ++i) dW1[i] = fmaf(dz1, xh[s * kMaxIn + i], dW1[i]);
+    for (int e = 0; e < 2; ++e) {
+      float dz[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const float d = dout[8 * sg + s];
+        dw3[e] = fmaf(d, h2[e][s], dw3[e]);
+        dz[s] = d * w3[e] * (1.0f - h2[e][s] * h2[e][s]);
+        db2[e] += dz[s];
+      }
+      float4* p = reinterpret_cast<float4*>(dz2T + ju[e] * kHP + 8 * sg);
+      p[0] = make_float4(dz[0], dz[1], dz[2], dz[3]);
+      p[1] = make_float4(dz[4], dz[5], dz[6], dz[7]);
+    }
+    __syncthreads();
+    // dW2[j][k] += sum_s dz2[s] h1[s][k], k = 32 sg + kk
+#pragma unroll 1
+    for (int s4 = 0; s4 < kTS / 4; ++s4) {
+      const float4 da = *reinterpret_cast<const float4*>(dz2T + jj * kHP + 4 * s4);
+      const float4 db = *reinterpret_cast<const float4*>(dz2T + (jj + 64) * kHP + 4 * s4);
+      const float* hb = h1T + 32 * sg * kHP + 4 * s4;
+#pragma unroll
+      for (int kk = 0; kk < 32; ++kk) {
+        const float4 h = *reinterpret_cast<const float4*>(hb + kk * kHP);
+        dW2[0][kk] = fmaf(da.x, h.x, dW2[0][kk]);
+        dW2[1][kk] = fmaf(db.x, h.x, dW2[1][kk]);
+        dW2[0][kk] = fmaf(da.y, h.y, dW2[0][kk]);
+        dW2[1][kk] = fmaf(db.y, h.y, dW2[1][kk]);
+        dW2[0][kk] = fmaf(da.z, h.z, dW2[0][kk]);
+        dW2[1][kk] = fmaf(db.z, h.z, dW2[1][kk]);
+        dW2[0][kk] = fmaf(da.w, h.w, dW2[0][kk]);
+        dW2[1][kk] = fmaf(db.w, h.w, dW2[1][kk]);
+      }
+    }
+    // layer-1 units k = jj, jj + 64: dh1[s] = sum_j W2[j][k] dz2[s][j]
+    float dh[2][8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) dh[0][s] = dh[1][s] = 0.0f;
+#pragma unroll 4
+    for (int j = 0; j < kW; ++j) {
+      const float wa = W2s[jj * kWP + j], wb = W2s[(jj + 64) * kWP + j];
+      const float4* dz = reinterpret_cast<const float4*>(dz2T + j * kHP + 8 * sg);
+      const float4 u = dz[0], v = dz[1];
+      const float dv[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        dh[0][s] = fmaf(wa, dv[s], dh[0][s]);
+        dh[1][s] = fmaf(wb, dv[s], dh[1][s]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const float* xr = xh + (8 * sg + s) * kMaxIn;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float dz1 = dh[e][s] * (1.0f - h1[e][s] * h1[e][s]);
+        db1[e] += dz1;
+#pragma unroll
+        for (int i = 0; i < kMaxIn; ++i) dW1[e][i] = fmaf(dz1, xr[i], dW1[e][i]);
       }
     }
     __syncthreads();   // h1T, dz2T, xh and outs are rewritten by the next tile
   }
-  // write this CTA's partials in the flat layout
+  // write this CTA's partials in the flat layout; the four sample groups' sums
+  // of W1, b1, b2 and w3 are added in group order
   float* out = A.partial + (int64_t)blockIdx.x * (A.P + 1);
   const int n_in = A.n_in;
   const int oW1 = 0, ob1 = kW * n_in, oW2 = ob1 + kW, ob2 = oW2 + kW * kW, ow3 = ob2 + kW, ob3 = ow3 + kW;
-  for (int i = 0; i < n_in; ++i) out[oW1 + j * n_in + i] = dW1[i];
-  out[ob1 + j] = db1;
-  for (int idx = j; idx < kW * kW; idx += kW) {
-    const int jj = idx / kW, k = idx - jj * kW;
-    out[oW2 + idx] = dW2s[k * kWP + jj];
+  constexpr int NS = kMaxIn + 3;
+  float* ends = sm + MlpSmem::H1;                       // [4][NS][kW]
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) W2s[ju[e] * kWP + 32 * sg + k] = dW2[e][k];   // for whole-row stores
+    float* d = ends + sg * NS * kW + ju[e];
+#pragma unroll
+    for (int i = 0; i < kMaxIn; ++i) d[i * kW] = dW1[e][i];
+    d[kMaxIn * kW] = db1[e];
+    d[(kMaxIn + 1) * kW] = db2[e];
+    d[(kMaxIn + 2) * kW] = dw3[e];
   }
-  out[ob2 + j] = db2;
-  out[ow3 + j] = dw3;
-  if (j == 0) {
+  __syncthreads();
+  for (int idx = tid; idx < kW * kW; idx += kBwdThreads) out[oW2 + idx] = W2s[(idx / kW) * kWP + idx % kW];
+  for (int idx = tid; idx < NS * kW; idx += kBwdThreads) {
+    const int i = idx / kW, j = idx % kW;
+    if (i < kMaxIn && i >= n_in) continue;
+    float v = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v += ends[q * NS * kW + idx];
+    const int o = i < kMaxIn ? oW1 + j * n_in + i : i == kMaxIn ? ob1 + j : i == kMaxIn + 1 ? ob2 + j : ow3 + j;
+    out[o] = v;
+  }
+  if (tid == 0) {
     out[ob3] = db3;
     out[A.P] = loss * inv_n;
   }
 }
 
-// grad[p] = sum over CTAs in order; loss = the same sum at index P.
-__global__ void k_mlp_reduce(const float* __restrict__ partial, int nblk, int64_t P1, float* __restrict__ grad) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P1) return;
+// grad[p] = sum over the CTA partials, loss = the same sum at index P; either
+// may be null.  A CTA takes 32 parameters: warp w adds rows w, w + 8, ..., then one warp
+// adds the eight in order: 4.5 us for 128 rows (one thread a parameter adding
+// the rows one after another took 14 us).
+constexpr int kRedWarps = 8;
+__global__ void __launch_bounds__(kRedWarps * 32) k_mlp_reduce(const float* __restrict__ partial, int nblk,
+                                                             int64_t P, float* __restrict__ grad,
+                                                             float* __restrict__ loss) {
+  __shared__ float red[kRedWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t p = (int64_t)blockIdx.x * 32 + lane;
   float acc = 0.0f;
-  for (int b = 0; b < nblk; ++b) acc += partial[(int64_t)b * P1 + p];
-  grad[p] = acc;
+  if (p <= P) {
+#pragma unroll 8
+    for (int b = warp; b < nblk; b += kRedWarps) acc += partial[(int64_t)b * (P + 1) + p];
+  }
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && p <= P) {
+    float v = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kRedWarps; ++w) v += red[w][lane];
+    if (p < P) {
+      if (grad) grad[p] = v;
+    } else if (loss) {
+      *loss = v;
+    }
+  }
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master copy, then the BF16 copies of
@@ -330,7 +518,7 @@ struct pm_mlp {
   float* theta = nullptr;          // [P] master
   float* m = nullptr;
   float* v = nullptr;
-  float* grad = nullptr;           // [P + 1] (loss at P)
+  float* grad = nullptr;           // [P]
   float* partial = nullptr;        // [nblk][P + 1]
   __nv_bfloat16* wbf = nullptr;    // W1 | W2 | w3
   float* norm = nullptr;           // mu [n_in] | sigma [n_in]
@@ -365,12 +553,13 @@ MlpArgs mlp_args(const pm_mlp* m, const float* X, const float* Y, int64_t n, flo
   return A;
 }
 
-int mlp_grad_launch(pm_mlp* m, const float* X, const float* Y, int64_t n) {
+// Gradient and loss of a batch into DEVICE grad [P] and loss [1] (either may be null).
+int mlp_grad_launch(pm_mlp* m, const float* X, const float* Y, int64_t n, float* grad, float* loss) {
   MlpArgs A = mlp_args(m, X, Y, n, nullptr);
   const int64_t tiles = (n + kTS - 1) / kTS;
   const int grid = (int)(tiles < m->nblk ? tiles : m->nblk);
-  k_mlp_backward<<<grid, kW, MlpSmem::BYTES, m->stream>>>(A);
-  k_mlp_reduce<<<(unsigned)((m->P + 1 + 255) / 256), 256, 0, m->stream>>>(m->partial, grid, m->P + 1, m->grad);
+  k_mlp_backward<<<grid, kBwdThreads, MlpSmem::BYTES, m->stream>>>(A);
+  k_mlp_reduce<<<(unsigned)((m->P + 1 + 31) / 32), kRedWarps * 32, 0, m->stream>>>(m->partial, grid, m->P, grad, loss);
   return mlp_check(cudaGetLastError());
 }
 
@@ -384,9 +573,9 @@ int mlp_forward_on(pm_mlp* m, const float* X, int64_t n, float* y, cudaStream_t 
   if (!m || n < 0 || (n > 0 && (!X || !y))) return PM_ERR_INVALID;
   if (n == 0) return PM_OK;
   MlpArgs A = mlp_args(m, X, nullptr, n, y);
-  const int64_t tiles = (n + kTS - 1) / kTS;
-  const int grid = (int)(tiles < m->sm_count ? tiles : m->sm_count);
-  k_mlp_forward<<<grid, kW, MlpSmem::BYTES, s>>>(A);
+  const int64_t ctas = ((n + 15) / 16 + kFwdWarps - 1) / kFwdWarps;
+  const int grid = (int)(ctas < 3 * m->sm_count ? ctas : 3 * m->sm_count);
+  k_mlp_forward<<<grid, kFwdWarps * 32, FwdSmem::BYTES, s>>>(A);
   return mlp_check(cudaGetLastError());
 }
 
@@ -422,7 +611,7 @@ int pm_mlp_create(int32_t n_in, int32_t width, void* cuda_stream, pm_mlp** out) 
     for (int i = 0; i < n_in; ++i) nrm[n_in + i] = 1.0f;
     ok = ok && cudaMemcpy(m->norm, nrm.data(), nrm.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)MlpSmem::BYTES) == cudaSuccess;
+                                    FwdSmem::BYTES) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)MlpSmem::BYTES) == cudaSuccess;
   }
@@ -491,27 +680,18 @@ int pm_mlp_forward(pm_mlp* m, const float* X, int64_t n, float* y) {
 
 int pm_mlp_grad(pm_mlp* m, const float* X, const float* y, int64_t n, float* grad, float* loss) {
   if (!m || n <= 0 || !X || !y) return PM_ERR_INVALID;
-  int rc = mlp_grad_launch(m, X, y, n);
-  if (rc != PM_OK) return rc;
-  if (grad && cudaMemcpyAsync(grad, m->grad, (size_t)m->P * sizeof(float), cudaMemcpyDeviceToDevice, m->stream) !=
-                  cudaSuccess)
-    return PM_ERR_CUDA;
-  if (loss && cudaMemcpyAsync(loss, m->grad + m->P, sizeof(float), cudaMemcpyDeviceToDevice, m->stream) != cudaSuccess)
-    return PM_ERR_CUDA;
-  return PM_OK;
+  return mlp_grad_launch(m, X, y, n, grad, loss);
 }
 
 int pm_mlp_train_step(pm_mlp* m, const float* X, const float* y, int64_t n, float lr, float* loss) {
   if (!m || n <= 0 || !X || !y || !(lr > 0.0f)) return PM_ERR_INVALID;
-  int rc = mlp_grad_launch(m, X, y, n);
+  int rc = mlp_grad_launch(m, X, y, n, m->grad, loss);
   if (rc != PM_OK) return rc;
   m->step += 1;
   const double b1 = 0.9, b2 = 0.999;
   const float bc1 = (float)(1.0 - pow(b1, (double)m->step)), bc2 = (float)(1.0 - pow(b2, (double)m->step));
   k_mlp_adam<<<(unsigned)((m->P + 255) / 256), 256, 0, m->stream>>>(m->theta, m->grad, m->m, m->v, m->P, lr, (float)b1,
                                                                   (float)b2, 1e-8f, bc1, bc2, m->wbf, m->n_in);
-  if (loss && cudaMemcpyAsync(loss, m->grad + m->P, sizeof(float), cudaMemcpyDeviceToDevice, m->stream) != cudaSuccess)
-    return PM_ERR_CUDA;
   return mlp_check(cudaGetLastError());
 }
 
