@@ -309,6 +309,35 @@ int grid_blocks(int64_t work, int threads, int ctas_per_sm = 16) {
   return (int)b;
 }
 
+// Forces by sorted slot from shared-memory tiles (FP32 grids of up to 512 points; false otherwise).
+template <int N>
+void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
+  using Cfg = GatherTile<N>;
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_gather_tile_acc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+    attr = true;
+  }
+  k_gather_tile_acc<N><<<Cfg::TILES, Cfg::THREADS, Cfg::SMEM, s>>>(
+      g.rec, g.row_start, scale, reinterpret_cast<const float*>(g.g), reinterpret_cast<float*>(g.accs));
+}
+template <typename U>
+bool gather_tiled(const GridArgs& g, U scale, cudaStream_t s) {
+  if constexpr (sizeof(U) == 4) {
+    switch (g.n) {
+      case 16: gather_tile_n<16>(g, scale, s); return true;
+      case 32: gather_tile_n<32>(g, scale, s); return true;
+      case 64: gather_tile_n<64>(g, scale, s); return true;
+      case 128: gather_tile_n<128>(g, scale, s); return true;
+      case 192: gather_tile_n<192>(g, scale, s); return true;
+      case 256: gather_tile_n<256>(g, scale, s); return true;
+      case 512: gather_tile_n<512>(g, scale, s); return true;
+      default: return false;
+    }
+  }
+  return false;
+}
+
 // The gather with the real-space gradient, in the order that the tuning asks
 // for (POW2: the grid size is a power of two, so the wraps are masks).
 template <bool POW2>
@@ -319,9 +348,10 @@ void gather_fd(const GridArgs& g, const void* pos, void* vel, double kick, void*
   const T scale = fd_scale_of<T>(g.cell);
   if (g.rows_ready && g.gather_rows == 2) {
     // forces in the sort's row order by sorted slot, then the velocities in particle order
-    k_interp_rows_acc<T, POW2><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
-                                 kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, scale, phi,
-                                                     reinterpret_cast<T*>(g.accs));
+    if (!gather_tiled<T>(g, scale, s))
+      k_interp_rows_acc<T, POW2><<<(unsigned)((g.np + kGatherTPB * kGatherChunk - 1) / (kGatherTPB * kGatherChunk)),
+                                   kGatherTPB, 0, s>>>(g.rec, g.row_start, g.n, scale, phi,
+                                                       reinterpret_cast<T*>(g.accs));
     k_kick_inv<T><<<grid_blocks(g.np, 256, g.part_ctas_per_sm), 256, 0, s>>>(
         g.inv, reinterpret_cast<const T*>(g.accs), g.np, v, (T)kick, acc);
   } else if (g.rows_ready) {   // row order of the deposit's sort: a warp per row

@@ -963,6 +963,42 @@ struct StencilWeights<double> {
   __device__ __forceinline__ double xy(int x, int y) const { return exact_product(F[0][x], F[1][y]); }
 };
 
+// The CIC sum of the folded stencils from the 56 potential values of a particle:
+// px [dz][dy][x0-2 .. x0+3], py [dz][dx][y0-2, y0-1, y0+2, y0+3], pz [dy][dx]
+// [z0-2, z0-1, z0+2, z0+3].  Every gather sums through here, so the forces do
+// not depend on its order.
+template <typename T>
+__device__ __forceinline__ void fd_combine(const T (&px)[2][2][6], const T (&py)[2][2][4], const T (&pz)[2][2][4],
+                                           const int (&w)[3], T (&a)[3]) {
+  const StencilWeights<T> W(w);
+  a[0] = a[1] = a[2] = (T)0;
+#pragma unroll
+  for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      T sx = (T)0;
+#pragma unroll
+      for (int j = 0; j < 6; ++j) sx += W.ex[j] * px[dz][dy][j];
+      a[0] += W.yz(dy, dz) * sx;
+    }
+#pragma unroll
+  for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+    for (int dx = 0; dx < 2; ++dx) {
+      const T sy = W.ey[0] * py[dz][dx][0] + W.ey[1] * py[dz][dx][1] + W.ey[2] * px[dz][0][2 + dx] +
+                   W.ey[3] * px[dz][1][2 + dx] + W.ey[4] * py[dz][dx][2] + W.ey[5] * py[dz][dx][3];
+      a[1] += W.xz(dx, dz) * sy;
+    }
+#pragma unroll
+  for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+    for (int dx = 0; dx < 2; ++dx) {
+      const T sz = W.ez[0] * pz[dy][dx][0] + W.ez[1] * pz[dy][dx][1] + W.ez[2] * px[0][dy][2 + dx] +
+                   W.ez[3] * px[1][dy][2 + dx] + W.ez[4] * pz[dy][dx][2] + W.ez[5] * pz[dy][dx][3];
+      a[2] += W.xy(dx, dy) * sz;
+    }
+}
+
 // -S phi at one particle (cell c, 16-bit weights w), before the -1/(12 d)
 // scale: the CIC sum of the 4-point stencil at its 8 corners (see above).
 // The 56 values lie on 20 (y, z) rows.  Away from the ends of the rows one
@@ -1050,33 +1086,7 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
         pz[dy][1][q] = r[xs[3]];
       }
   }
-  const StencilWeights<T> W(w);
-  a[0] = a[1] = a[2] = (T)0;
-#pragma unroll
-  for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-    for (int dy = 0; dy < 2; ++dy) {
-      T sx = (T)0;
-#pragma unroll
-      for (int j = 0; j < 6; ++j) sx += W.ex[j] * px[dz][dy][j];
-      a[0] += W.yz(dy, dz) * sx;
-    }
-#pragma unroll
-  for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-    for (int dx = 0; dx < 2; ++dx) {
-      const T sy = W.ey[0] * py[dz][dx][0] + W.ey[1] * py[dz][dx][1] + W.ey[2] * px[dz][0][2 + dx] +
-                   W.ey[3] * px[dz][1][2 + dx] + W.ey[4] * py[dz][dx][2] + W.ey[5] * py[dz][dx][3];
-      a[1] += W.xz(dx, dz) * sy;
-    }
-#pragma unroll
-  for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-    for (int dx = 0; dx < 2; ++dx) {
-      const T sz = W.ez[0] * pz[dy][dx][0] + W.ez[1] * pz[dy][dx][1] + W.ez[2] * px[0][dy][2 + dx] +
-                   W.ez[3] * px[1][dy][2 + dx] + W.ez[4] * pz[dy][dx][2] + W.ez[5] * pz[dy][dx][3];
-      a[2] += W.xy(dx, dy) * sz;
-    }
+  fd_combine<T>(px, py, pz, w, a);
 }
 
 // Work order: CTA b takes the kGatherChunk x kGatherTPB consecutive particles
@@ -1259,6 +1269,142 @@ __global__ void k_kick_inv(const int* __restrict__ inv, const T* __restrict__ ac
       vel[d * np + p] = vel[d * np + p] + ad[d] * kick;
       if (acc_out) acc_out[d * np + p] = ad[d];
     }
+  }
+}
+
+// k_interp_rows_acc from shared memory, FP32 grids of up to 512 points (longer
+// rows do not fit).  A CTA owns the particles that the deposit's sort placed
+// in TZ x TY grid rows (whole rows along x) and stages the potential rows their
+// stencils touch: TZ + 1 planes of TY + 5 rows and, for the z differences, TY + 1
+// rows of the two planes on either side; each row with a halo of its periodic
+// neighbours, so that no index wraps.  A particle's 56 values are then
+// shared-memory reads at constant offsets from a few addresses.  For clustered
+// particles, whose lanes spread over their row, a read from global memory is
+// about ten L1 wavefronts, from shared memory three or four (32 lanes on 32 banks):
+// 512^3 clustered particles on 512^3 points with the velocity pass
+// 5.08 -> 3.66 ms.  (Particles near storage order gain nothing: their lanes read
+// neighbouring cells anyway, and velocities through the permutation cost more,
+// 0.45 against 0.345 ms at 256^3.)
+template <int N>
+struct GatherTile {
+  static constexpr int TY = 4, TZ = N <= 256 ? 4 : 2;
+  static constexpr int PITCH = N + 8;                     // cell x at x + 4, x in [-2, N + 2]
+  static constexpr int YA = TY + 5, RA = (TZ + 1) * YA, RB = 4 * (TY + 1), ROWS = RA + RB;
+  static constexpr size_t SMEM = (size_t)ROWS * PITCH * sizeof(float);
+  static constexpr int THREADS = N <= 256 ? 384 : 512;    // 36 warps per SM in three CTAs, 32 in two at 512
+  static constexpr int CTAS = N <= 256 ? 3 : 2;
+  static constexpr int TILES = (N / TY) * (N / TZ);
+  static_assert(N % 4 == 0 && CTAS * (SMEM + 1024) <= 227 * 1024, "tile shared memory");
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Stage the rows of the tile with first row (y0, z0).  Ends with a barrier.
+template <int N>
+__device__ __forceinline__ void gather_tile_load(const float* __restrict__ phi, float* sm, int y0, int z0) {
+  using Cfg = GatherTile<N>;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r = warp; r < Cfg::ROWS; r += Cfg::THREADS / 32) {
+    int y, z;
+    if (r < Cfg::RA) {
+      z = z0 + r / Cfg::YA;
+      y = y0 - 2 + r % Cfg::YA;
+    } else {
+      const int q = r - Cfg::RA, b = q / (Cfg::TY + 1);
+      z = z0 + (b < 2 ? b - 2 : Cfg::TZ - 1 + b);
+      y = y0 + q % (Cfg::TY + 1);
+    }
+    y = y < 0 ? y + N : y >= N ? y - N : y;
+    z = z < 0 ? z + N : z >= N ? z - N : z;
+    const float* src = phi + ((int64_t)z * N + y) * N;
+    float* dst = sm + r * Cfg::PITCH + 4;
+    for (int i = lane; i < N / 4; i += 32) cp_async16(dst + 4 * i, src + 4 * i);
+    if (lane < 2) dst[lane - 2] = src[N - 2 + lane];
+    else if (lane < 5) dst[N + lane - 2] = src[lane - 2];
+  }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+}
+
+// -S phi of a particle in x cell c0 of the tile's row (yl, zl).
+template <int N>
+__device__ __forceinline__ void gather_tile_stencil(const float* sm, int c0, int yl, int zl, const int (&w)[3],
+                                                    float (&a)[3]) {
+  using Cfg = GatherTile<N>;
+  constexpr int P = Cfg::PITCH;
+  const float* b = sm + (zl * Cfg::YA + yl + 2) * P + 4 + c0;
+  float px[2][2][6], py[2][2][4], pz[2][2][4];
+  constexpr int kOff[4] = {-2, -1, 2, 3};
+#pragma unroll
+  for (int dz = 0; dz < 2; ++dz) {
+    const float* bz = b + dz * Cfg::YA * P;
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+      for (int j = 0; j < 6; ++j) px[dz][dy][j] = bz[dy * P + j - 2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      py[dz][0][q] = bz[kOff[q] * P];
+      py[dz][1][q] = bz[kOff[q] * P + 1];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int pl = zl + kOff[q];            // plane of the tile, in [-2, TZ + 2]
+    int r = pl * Cfg::YA + 2;
+    if (kOff[q] < 0 && pl < 0) r = Cfg::RA + (pl + 2) * (Cfg::TY + 1);
+    if (kOff[q] > 0 && pl > Cfg::TZ) r = Cfg::RA + (pl - Cfg::TZ + 1) * (Cfg::TY + 1);
+    const float* bz = sm + (r + yl) * P + 4 + c0;
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy) {
+      pz[dy][0][q] = bz[dy * P];
+      pz[dy][1][q] = bz[dy * P + 1];
+    }
+  }
+  fd_combine<float>(px, py, pz, w, a);
+}
+
+// Tile blockIdx.x of TILES: the forces of the particles of its rows by sorted slot.
+template <int N>
+__global__ void __launch_bounds__(GatherTile<N>::THREADS, GatherTile<N>::CTAS)
+k_gather_tile_acc(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start, float scale,
+                  const float* __restrict__ phi, float* __restrict__ accs) {
+  using Cfg = GatherTile<N>;
+  constexpr int TY = Cfg::TY, TZ = Cfg::TZ;
+  constexpr int YM = (N < 32 ? N : 32) - 1;   // the record holds y mod 32
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* sm = reinterpret_cast<float*>(smem_raw);
+  const int y0 = (blockIdx.x % (N / TY)) * TY, z0 = (blockIdx.x / (N / TY)) * TZ;
+  // the rows y0 .. y0 + TY - 1 of a plane are one run of sorted slots: TZ runs,
+  // concatenated in a virtual index j
+  int pre[TZ + 1], off[TZ];
+  pre[0] = 0;
+#pragma unroll
+  for (int q = 0; q < TZ; ++q) {
+    const int r = (z0 + q) * N + y0;
+    const int b = row_start[r];
+    off[q] = b - pre[q];
+    pre[q + 1] = pre[q] + row_start[r + TY] - b;
+  }
+  const int total = pre[TZ];
+  if (total == 0) return;                 // uniform over the CTA
+  gather_tile_load<N>(phi, sm, y0, z0);
+  for (int j = threadIdx.x; j < total; j += Cfg::THREADS) {
+    int zl = 0, o = off[0];
+#pragma unroll
+    for (int q = 1; q < TZ; ++q)
+      if (j >= pre[q]) {
+        o = off[q];
+        zl = q;
+      }
+    const int64_t i = j + o;
+    const unsigned long long r = rec[i];
+    const int w[3] = {(int)(r & 0xffffu), (int)((r >> 16) & 0xffffu), (int)((r >> 32) & 0xffffu)};
+    float a[3];
+    gather_tile_stencil<N>(sm, (int)(r >> 48) & 0x7ff, ((int)(r >> 59) - y0) & YM, zl, w, a);
+    reinterpret_cast<float4*>(accs)[i] = make_float4(a[0] * scale, a[1] * scale, a[2] * scale, 0.0f);
   }
 }
 
