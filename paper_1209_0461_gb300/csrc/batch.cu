@@ -200,14 +200,18 @@ struct PCol {
 };
 
 // Bin sums of rows [item per, (item + 1) per) into partials row `item`.
+template <int N>
 struct PBins {
   static constexpr int THREADS = kBinWarps * 32;
   __device__ static void run(const BoxArgs& b, int item) {
     const int rows = b.g.n * b.g.n;
     const int per = (rows + b.bin_chunks - 1) / b.bin_chunks;
     const int r0 = item * per, r1 = min(rows, r0 + per);
-    bin_power_rows<T, false>(reinterpret_cast<const C*>(b.g.spec), b.g.n, b.nu.nk, b.thr, b.inv_lr, b.kf,
-                             b.partials, r0, r1, kBinWarps, item);
+    const C* spec = reinterpret_cast<const C*>(b.g.spec);
+    if constexpr (N >= 64)
+      bin_power_rows_n<T, N>(spec, b.nu.nk, b.thr, b.inv_lr, b.partials, r0, r1, kBinWarps, item);
+    else
+      bin_power_rows<T, false>(spec, b.g.n, b.nu.nk, b.thr, b.inv_lr, b.kf, b.partials, r0, r1, kBinWarps, item);
   }
 };
 
@@ -342,7 +346,7 @@ void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEve
   launch_pass<PDeposit<N>>(p, kBpDeposit, PDeposit<N>::SMEM, s);
   launch_pass<PCol<N, -1, false, false>>(p, kBpY, PCol<N, -1, false, false>::SMEM, s);
   launch_pass<PCol<N, -1, true, false>>(p, kBpZ, PCol<N, -1, true, false>::SMEM, s);
-  launch_pass<PBins>(p, kBpBins, kBinWarps * (size_t)p.nk * sizeof(double) + (size_t)(p.nk + 1) * sizeof(int), s);
+  launch_pass<PBins<N>>(p, kBpBins, kBinWarps * (size_t)p.nk * sizeof(double) + (size_t)(p.nk + 1) * sizeof(int), s);
   launch_pass<PBinReduce>(p, kBpBinReduce, 0, s);
   cudaStreamWaitEvent(s, ev_join, 0);
   launch_pass<PFinish>(p, kBpFinish, 0, s);

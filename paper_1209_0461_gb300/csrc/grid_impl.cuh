@@ -455,8 +455,26 @@ int NUPM_FN(bins)(const GridArgs& g, bool lattice, int nk, const int* thr, float
       nblk = wave((const void*)k_bin_power<T, true>, sh);
       k_bin_power<T, true><<<nblk, kBinWarps * 32, sh, s>>>(spec, g.n, nk, thr, inv_lr, kf, partials);
     } else {
-      nblk = wave((const void*)k_bin_power<T, false>, sh);
-      k_bin_power<T, false><<<nblk, kBinWarps * 32, sh, s>>>(spec, g.n, nk, thr, inv_lr, kf, partials);
+      // at least four rows a warp: on small grids the partial rows and their
+      // reduction cost more than the sums
+      const int most = g.n * g.n / (4 * kBinWarps);
+      auto run = [&](auto kern) {
+        nblk = wave((const void*)kern, sh);
+        nblk = nblk < most ? nblk : most;
+        kern<<<nblk, kBinWarps * 32, sh, s>>>(spec, nk, thr, inv_lr, partials);
+      };
+      switch (g.n) {
+        case 64: run(k_bin_power_n<T, 64>); break;
+        case 128: run(k_bin_power_n<T, 128>); break;
+        case 192: run(k_bin_power_n<T, 192>); break;
+        case 256: run(k_bin_power_n<T, 256>); break;
+        case 512: run(k_bin_power_n<T, 512>); break;
+        case 1024: run(k_bin_power_n<T, 1024>); break;
+        default:   // rows shorter than a warp
+          nblk = wave((const void*)k_bin_power<T, false>, sh);
+          nblk = nblk < most ? nblk : most;
+          k_bin_power<T, false><<<nblk, kBinWarps * 32, sh, s>>>(spec, g.n, nk, thr, inv_lr, kf, partials);
+      }
     }
   }
   k_bin_reduce<<<(nv * nk + 31) / 32, 1024, 0, s>>>(partials, nblk, nv * nk, out);

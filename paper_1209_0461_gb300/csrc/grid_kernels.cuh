@@ -631,6 +631,59 @@ __device__ __forceinline__ void bin_row_staged(const cx<T> (&f)[kBinLaneMax], cx
   __syncwarp();
 }
 
+// Power sums of rows row0 + warp, row0 + warp + row_step, ... below row1 for a
+// grid of N >= 64 points (E = N / 64 modes a lane, known at compile time), the
+// next row's modes loaded while this row is summed; their sum to partials[slot].
+// (bin_row unrolled for 16 modes a lane whatever the row, and one row's loads
+// in flight: 136 us for twelve 128^3 boxes, 45 us at 192^3.)
+template <typename T, int N>
+__device__ __forceinline__ void bin_power_rows_n(const cx<T>* __restrict__ spec, int nk, const int* __restrict__ thr,
+                                                 float inv_lr, double* __restrict__ partials, int row0, int row1,
+                                                 int row_step, int64_t slot) {
+  constexpr int M = N / 2, E = M / 32;
+  static_assert(M % 32 == 0 && E <= kBinLaneMax, "whole lanes");
+  constexpr bool kAhead = E * sizeof(cx<T>) <= 64;   // registers for a second row
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* all = reinterpret_cast<double*>(smem_raw);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* acc = all + warp * nk;
+  int* Ts = reinterpret_cast<int*>(all + kBinWarps * nk);
+  for (int i = threadIdx.x; i < kBinWarps * nk; i += blockDim.x) all[i] = 0.0;
+  for (int i = threadIdx.x; i <= nk; i += blockDim.x) Ts[i] = thr[i];
+  __syncthreads();
+  cx<T> f[kBinLaneMax], fn[kBinLaneMax], g = {(T)0, (T)0}, gn = {(T)0, (T)0};
+  auto load = [&](int row, cx<T>(&d)[kBinLaneMax], cx<T>& p) {
+    const cx<T>* r = spec + (int64_t)row * M + lane * E;
+#pragma unroll
+    for (int i = 0; i < E; ++i) d[i] = r[i];
+    if (lane == 0)   // the packed slot of the partner row (-z, -y)
+      p = spec[((int64_t)partner_index(row / N, N) * N + partner_index(row % N, N)) * M];
+  };
+  int row = row0 + warp;
+  if (kAhead && row < row1) load(row, fn, gn);
+  for (; row < row1; row += row_step) {
+    if constexpr (kAhead) {
+#pragma unroll
+      for (int i = 0; i < E; ++i) f[i] = fn[i];
+      g = gn;
+      if (row + row_step < row1) load(row + row_step, fn, gn);
+    } else {
+      load(row, f, g);
+    }
+    const int kz = signed_freq(row / N, N), ky = signed_freq(row % N, N);
+    bin_row_staged<T, E>(f, g, kz * kz + ky * ky, lane, Ts, nk, inv_lr, acc);
+  }
+  bin_flush_partials<T, false>(all, nk, partials, slot);
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(kBinWarps * 32)
+k_bin_power_n(const cx<T>* __restrict__ spec, int nk, const int* __restrict__ thr, float inv_lr,
+              double* __restrict__ partials) {
+  bin_power_rows_n<T, N>(spec, nk, thr, inv_lr, partials, blockIdx.x * kBinWarps, N * N, gridDim.x * kBinWarps,
+                         blockIdx.x);
+}
+
 // FP32 power sums with the rows staged by TMA: each warp runs a
 // kBinStages-deep ring of row buffers in shared memory (two: 5 CTAs per SM
 // at 1024^3, where three allowed 3 and the combine went short of warps).  A tensor map views

@@ -423,8 +423,10 @@ __device__ __forceinline__ void bin_reduce_group(const double* __restrict__ part
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = i0 + lane;
   double acc = 0.0;
-  if (i < len)
+  if (i < len) {
+#pragma unroll 8
     for (int b = warp; b < nblk; b += kReduceWarps) acc += partials[(int64_t)b * len + i];
+  }
   red[warp][lane] = acc;
   __syncthreads();
   if (warp == 0) {
