@@ -12,7 +12,7 @@
 // transform, real-space 4-point gradient in the gather):
 //   row count, row scan (one CTA per box; it also clears the counts for the
 //   next kick), row scatter, deposit + x, y, z, bin sums + their fixed-order
-//   reduction, response panels, finish, bin list, fac table, Green plane,
+//   reduction, response nodes and panels, finish + bin list, fac table, Green plane,
 //   Green + z inverse, y inverse, x inverse, gather + kick.
 #include <type_traits>
 #include <cuda_runtime.h>
@@ -31,7 +31,6 @@ using C = cx<float>;
 
 constexpr int kSortSteps = 4;                  // warp batches per row-sort item and warp
 constexpr int kSortChunk = 256 * kSortBatch * kSortSteps;   // particles per row-sort item (a CTA of 256)
-constexpr int kFinishGroup = 128;               // bins per finish item
 constexpr int kFacGroup = 256;                  // fac-table entries per item
 constexpr int kPlaneGroup = 256;                // Green-plane entries per item
 constexpr int kScanThreads = 1024;
@@ -224,6 +223,16 @@ struct PBinReduce {
   }
 };
 
+// Quadrature points of the whole history intervals (kNodeGroup entries an item).
+constexpr int kNodeGroup = 128;
+struct PNodes {
+  static constexpr int THREADS = kNodeGroup;
+  static constexpr size_t SMEM = 0;
+  __device__ static void run(const BoxArgs& b, int item) {
+    if (b.nu.ns > 0) nu_node_entry(b.nu, item * kNodeGroup + threadIdx.x);
+  }
+};
+
 // On the side stream: two CTAs per SM at most, so that the passes of the main
 // stream keep the rest of each SM (a full-occupancy persistent launch would
 // hold every slot until the panels are done and starve them).
@@ -234,16 +243,15 @@ struct PPanels {
   __device__ static void run(const BoxArgs& b, int item) { nu_panels_item(b.nu, item * 4 + (threadIdx.x >> 5)); }
 };
 
+// Finish of every bin and the list of the non-empty ones (nk <= 1024).
 struct PFinish {
-  static constexpr int THREADS = kFinishGroup;
-  static constexpr size_t SMEM = 0;
-  __device__ static void run(const BoxArgs& b, int item) { nu_finish_bin(b.nu, item * kFinishGroup + threadIdx.x); }
-};
-
-struct PRlist {
   static constexpr int THREADS = 1024;
   static constexpr size_t SMEM = 0;
-  __device__ static void run(const BoxArgs& b, int) { nu_rlist_block(b.nu.bins, b.nu.R, b.nu.nk, b.nu.rlist); }
+  __device__ static void run(const BoxArgs& b, int) {
+    nu_finish_bin(b.nu, threadIdx.x);
+    __syncthreads();
+    nu_rlist_block(b.nu.bins, b.nu.R, b.nu.nk, b.nu.rlist);
+  }
 };
 
 struct PFac {
@@ -338,6 +346,7 @@ void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEve
   // they run on the side stream beside the deposit and the transforms
   cudaEventRecord(ev_fork, s);
   cudaStreamWaitEvent(side, ev_fork, 0);
+  launch_pass<PNodes>(p, kBpNodes, 0, side);
   launch_pass<PPanels>(p, kBpPanels, 0, side);
   cudaEventRecord(ev_join, side);
   launch_pass<PCount>(p, kBpCount, 0, s);
@@ -350,7 +359,6 @@ void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEve
   launch_pass<PBinReduce>(p, kBpBinReduce, 0, s);
   cudaStreamWaitEvent(s, ev_join, 0);
   launch_pass<PFinish>(p, kBpFinish, 0, s);
-  launch_pass<PRlist>(p, kBpRlist, 0, s);
   launch_pass<PFac>(p, kBpFac, 2 * (size_t)p.nk * sizeof(double), s);
   launch_pass<PPlane0>(p, kBpPlane0, 0, s);
   launch_pass<PZInv<N>>(p, kBpZInv, PZInv<N>::SMEM, s);
@@ -399,7 +407,7 @@ int deposit_rows(int n) {
 
 bool batch_supported(int n) { return col_width(n) > 0; }
 
-void batch_items(int n, int64_t np, int nk, int ns, int bin_chunks, int* items) {
+void batch_items(int n, int64_t np, int nk, int ns, int n_hist_max, int quad, int bin_chunks, int* items) {
   const int m = n / 2;
   items[kBpCount] = items[kBpScatter] = (int)((np + kSortChunk - 1) / kSortChunk);
   items[kBpScan] = 1;
@@ -407,9 +415,9 @@ void batch_items(int n, int64_t np, int nk, int ns, int bin_chunks, int* items) 
   items[kBpY] = items[kBpZ] = items[kBpZInv] = items[kBpYInv] = (m / col_width(n)) * n;
   items[kBpBins] = bin_chunks;
   items[kBpBinReduce] = (nk + 31) / 32;
+  items[kBpNodes] = ns > 0 ? (n_hist_max + 1) * quad / kNodeGroup + 1 : 0;
   items[kBpPanels] = (nk * ns * kNuChunks + 3) / 4;
-  items[kBpFinish] = (nk + kFinishGroup - 1) / kFinishGroup;
-  items[kBpRlist] = 1;
+  items[kBpFinish] = 1;
   items[kBpFac] = (kFacTable + kFacGroup - 1) / kFacGroup;
   items[kBpPlane0] = (n * n + kPlaneGroup - 1) / kPlaneGroup;
   items[kBpXInv] = n * n / row_group(n);

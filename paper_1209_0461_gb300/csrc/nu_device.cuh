@@ -165,53 +165,93 @@ __device__ static double nu_K_warp(double y, const NuArgs& A, int lane) {
 // shared memory.  Returns the number of panels, pts[p + 1] .. pts[p] the p-th.
 // (One lane merging the two lists took most of the kernel: 150 serial steps of
 // dependent FP64 operations at 128 nodes, repeated by every warp of the bin.)
-__device__ __forceinline__ int nu_break_points(const double* hu, int n, double ue, double ui, double ell, double* pts) {
+// Comparisons are on order_key: an FP64 comparison costs as much as any other
+// FP64 operation, and ten warps a bin place the same points.  gr: scratch of the graded points.
+__device__ __forceinline__ long long order_key(double v) {   // orders as v does
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ int nu_break_points(const long long* hk, const double* hu, int n, double ue, double ui,
+                                               double ell, double* gr, double* pts) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
+  const long long ke = order_key(ue), ki = order_key(ui);
   // nodes inside (u_i, u_e): [j0, j1)
   int j0 = 0, j1 = 0;
   for (int i = lane; i < n; i += 32) {
-    j0 += hu[i] <= ui ? 1 : 0;
-    j1 += hu[i] < ue ? 1 : 0;
+    j0 += hk[i] <= ki ? 1 : 0;
+    j1 += hk[i] < ke ? 1 : 0;
   }
   j0 = __reduce_add_sync(full, j0);
   j1 = __reduce_add_sync(full, j1);
   // graded points above u_i: a prefix of m = -2, -1, ... (they fall with m)
   int G = 0;
   for (int base = 0; base < kMaxGraded; base += 32) {
-    const bool in = ue - ell * exp2_int(base + lane - 2) > ui;
-    const unsigned m = __ballot_sync(full, in);
+    const double u = ue - ell * exp2_int(base + lane - 2);
+    gr[base + lane] = u;
+    const unsigned m = __ballot_sync(full, order_key(u) > ki);
     G += __popc(m);
     if (m != full) break;
   }
-  if (G > kMaxGraded) G = kMaxGraded;
+  __syncwarp();
   const int room = kMaxPanels - 1;   // entries after u_e, u_i included
   int np = j1 - j0 + G + 1;
   if (np > room) np = room;
   if (lane == 0) pts[0] = ue;
   for (int g = lane; g < G; g += 32) {
-    const double u = ue - ell * exp2_int(g - 2);
+    const long long k = order_key(gr[g]);
     int lo = j0, hi = j1;                // nodes above u: [lo, j1)
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (hu[mid] > u) hi = mid; else lo = mid + 1;
+      if (hk[mid] > k) hi = mid; else lo = mid + 1;
     }
     const int r = 1 + g + (j1 - lo);
-    if (r < np) pts[r] = u;
+    if (r < np) pts[r] = gr[g];
   }
   for (int j = j0 + lane; j < j1; j += 32) {
-    const double u = hu[j];
     int lo = 0, hi = G;                  // graded points at or above u: [0, lo)
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (ue - ell * exp2_int(mid - 2) >= u) lo = mid + 1; else hi = mid;
+      if (order_key(gr[mid]) >= hk[j]) lo = mid + 1; else hi = mid;
     }
     const int r = 1 + (j1 - 1 - j) + lo;
-    if (r < np) pts[r] = u;
+    if (r < np) pts[r] = hu[j];
   }
   if (lane == 0) pts[np] = ui;
   __syncwarp();
   return ue > ui ? np : 0;
+}
+
+// H(a) at the response's scale factor.
+__device__ __forceinline__ double nu_hubble(const NuArgs& A) {
+  return A.rel ? sqrt(rel_e2(A.a, A.bg)) : sqrt(A.omega_m * exp(-3.0 * A.ue) + A.omega_l);
+}
+
+// What a quadrature point of a whole interval of the history needs and no bin
+// changes: (s_end - s(u), weight / (a H)) at node q of interval k = seg + 1, from
+// max(node seg, u_i) to node seg + 1 (u_e after the last); entry i = k quad + q.
+// Most panels are whole intervals, and their points then cost 36 FP64
+// operations (I(x) and the sums) instead of 110.  Entry (n_hist + 1) quad:
+// (s_end, H(a)).  A.nodes is null where the history is too short for the table's
+// own launch to pay (nu_args).
+__device__ __forceinline__ void nu_node_entry(const NuArgs& A, int i) {
+  const int n = A.n_hist, Q = A.quad;
+  if (!A.nodes || i > (n + 1) * Q) return;
+  if (i == (n + 1) * Q) {
+    A.nodes[i] = make_double2(s_table(A, A.ue), nu_hubble(A));
+    return;
+  }
+  const int k = i / Q, q = i - k * Q;
+  const double lo = k > 0 ? fmax(A.hist_u[k - 1], A.ui) : A.ui;
+  const double hi = k < n ? A.hist_u[k] : A.ue;
+  const double half = 0.5 * (hi - lo);
+  const double u = lo + half * (A.gl[q] + 1.0);
+  const double ap = exp(u);
+  // 1 / (a H): a H = sqrt(Omega_M / a + Omega_L a^2) for matter + Lambda
+  double iaH;
+  if (A.rel) iaH = 1.0 / (ap * sqrt(rel_e2(ap, A.bg)));
+  else iaH = rsqrt(A.omega_m / ap + A.omega_l * (ap * ap));
+  A.nodes[i] = make_double2(s_table(A, A.ue) - s_table(A, u), half * A.gl[kMaxQuad + q] * iaH);
 }
 
 // Body: chunk `item` (< nk ns kNuChunks) of a (bin, species), one warp (warp w
@@ -222,9 +262,16 @@ __device__ __forceinline__ int nu_break_points(const double* hu, int n, double u
 __device__ __forceinline__ void nu_panels_item(const NuArgs& A, int item) {
   __shared__ double pts_s[4][kMaxPanels + 1];
   __shared__ double hu_s[kMaxPanels];
+  __shared__ long long hk_s[kMaxPanels];
+  __shared__ double gr_s[4][kMaxGraded];
+  __shared__ short list_s[4][kMaxPanels];   // panels: cut ones from the front, whole intervals from the back
+  __shared__ short seg_s[4][kMaxPanels];
   __syncthreads();   // (batched form: the previous item is done with the scratch)
   const int n = A.n_hist;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) hu_s[i] = A.hist_u[i];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    hu_s[i] = A.hist_u[i];
+    hk_s[i] = order_key(hu_s[i]);
+  }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (item >= A.nk * A.ns * kNuChunks) return;
@@ -239,55 +286,83 @@ __device__ __forceinline__ void nu_panels_item(const NuArgs& A, int item) {
     return;
   }
   const double kb = A.bins[A.nk + b] / cnt;
-  const double s_end = s_table(A, A.ue);
+  const int Q = A.quad;
+  const double2 top = A.nodes ? A.nodes[(n + 1) * Q] : make_double2(s_table(A, A.ue), nu_hubble(A));
+  const double s_end = top.x, Ha = top.y;
   const double kappa = kb * A.kappa_scale[s];
-  const double Ha = A.rel ? sqrt(rel_e2(A.a, A.bg)) : sqrt(A.omega_m * exp(-3.0 * A.ue) + A.omega_l);
   const double ell = (kappa > 0.0) ? A.a * A.a * Ha / kappa : 1e300;
   double* pts = pts_s[warp];
-  const int np = nu_break_points(hu_s, n, A.ue, A.ui, ell, pts);
-  const int Q = A.quad;
+  const int np = nu_break_points(hk_s, hu_s, n, A.ue, A.ui, ell, gr_s[warp], pts);
   double jh = 0.0, wc = 0.0;
-  for (int i = chunk * 32 + lane; i < np * Q; i += 32 * A.nchunks) {
-    const int p = i / Q, q = i - p * Q;
-    const double hi = pts[p], lo = pts[p + 1];
-    if (!(hi > lo)) continue;
-    const double half = 0.5 * (hi - lo);
-    // P_M^{1/2} on this panel: h(u) = h0 + (h1 - h0) (u - u0) / (u1 - u0) (history part)
-    // plus the current-node hat on the last interval; seg: the last node below hi
-    int l = 0, r = n;
-    while (l < r) {
-      const int mid = (l + r) >> 1;
-      if (hu_s[mid] < hi) l = mid + 1; else r = mid;
+  // each panel's seg (the last node below its upper end), and the panels split
+  // into those cut by a graded point and the whole intervals
+  int ncut = 0, nwhole = 0;
+  for (int p0 = 0; p0 < np; p0 += 32) {
+    const int p = p0 + lane;
+    bool some = false, whole = false;
+    if (p < np) {
+      const long long hi = order_key(pts[p]), lo = order_key(pts[p + 1]);
+      int l = 0, r = n;
+      while (l < r) {
+        const int mid = (l + r) >> 1;
+        if (hk_s[mid] < hi) l = mid + 1; else r = mid;
+      }
+      const int seg = l - 1;
+      seg_s[warp][p] = (short)seg;
+      some = hi > lo;
+      whole = some && A.nodes && lo == (seg >= 0 ? hk_s[seg] : order_key(A.ui)) &&
+              hi == (seg + 1 < n ? hk_s[seg + 1] : order_key(A.ue));
     }
-    const int seg = l - 1;
-    const double u = lo + half * (A.gl[q] + 1.0);
-    const double wq = half * A.gl[kMaxQuad + q];
-    const double ap = exp(u);
-    // 1 / (a H): a H = sqrt(Omega_M / a + Omega_L a^2) for matter + Lambda
-    double iaH;
-    if (A.rel) iaH = 1.0 / (ap * sqrt(rel_e2(ap, A.bg)));
-    else iaH = rsqrt(A.omega_m / ap + A.omega_l * (ap * ap));
-    const double ds = s_end - s_table(A, u);
-    const double x = kappa * ds;
-    const double I = A.use_fit ? nu_I_fit(x) : nu_I_table(x, A.icheb);
-    const double base = wq * I * ds * iaH;
+    const unsigned mw = __ballot_sync(0xffffffffu, whole), mc = __ballot_sync(0xffffffffu, some && !whole);
+    const unsigned below = (1u << lane) - 1;
+    if (whole) list_s[warp][kMaxPanels - 1 - (nwhole + __popc(mw & below))] = (short)p;
+    else if (some) list_s[warp][ncut + __popc(mc & below)] = (short)p;
+    nwhole += __popc(mw);
+    ncut += __popc(mc);
+  }
+  __syncwarp();
+  auto I_of = [&](double x) { return A.use_fit ? nu_I_fit(x) : nu_I_table(x, A.icheb); };
+  // P_M^{1/2} on a panel: h(u) = h0 + (h1 - h0) tau, tau = (u - u0) / (u1 - u0)
+  // (history part), plus the current-node hat on the last interval
+  auto add = [&](int seg, double base, double tau) {
     if (n == 0) {                       // h == h_cur on [u_i, u_e]
       wc += base;
     } else if (seg < 0) {               // constant h_0 before the first node
       jh += base * A.hist[b];
     } else {
-      const bool last = seg == n - 1;
-      const double u0 = hu_s[seg], u1 = last ? A.ue : hu_s[seg + 1];
       const double h0 = A.hist[(int64_t)seg * A.nk + b];
-      const double tau = (u - u0) / (u1 - u0);
-      if (last) {
+      if (seg == n - 1) {
         jh += base * h0 * (1.0 - tau);
         wc += base * tau;
       } else {
-        const double h1 = A.hist[(int64_t)(seg + 1) * A.nk + b];
-        jh += base * (h0 + (h1 - h0) * tau);
+        jh += base * (h0 + (A.hist[(int64_t)(seg + 1) * A.nk + b] - h0) * tau);
       }
     }
+  };
+  for (int i = chunk * 32 + lane; i < ncut * Q; i += 32 * A.nchunks) {
+    const int p = list_s[warp][i / Q], q = i % Q;
+    const int seg = seg_s[warp][p];
+    const double hi = pts[p], lo = pts[p + 1];
+    const double half = 0.5 * (hi - lo);
+    const double u = lo + half * (A.gl[q] + 1.0);
+    const double wq = half * A.gl[kMaxQuad + q];
+    const double ap = exp(u);
+    double iaH;                         // as nu_node_entry
+    if (A.rel) iaH = 1.0 / (ap * sqrt(rel_e2(ap, A.bg)));
+    else iaH = rsqrt(A.omega_m / ap + A.omega_l * (ap * ap));
+    const double ds = s_end - s_table(A, u);
+    double tau = 0.0;
+    if (seg >= 0) {
+      const double u0 = hu_s[seg], u1 = seg == n - 1 ? A.ue : hu_s[seg + 1];
+      tau = (u - u0) / (u1 - u0);
+    }
+    add(seg, wq * I_of(kappa * ds) * ds * iaH, tau);
+  }
+  for (int i = chunk * 32 + lane; i < nwhole * Q; i += 32 * A.nchunks) {
+    const int p = list_s[warp][kMaxPanels - 1 - i / Q], q = i % Q;
+    const int seg = seg_s[warp][p];
+    const double2 t = A.nodes[(seg + 1) * Q + q];
+    add(seg, t.y * I_of(kappa * t.x) * t.x, 0.5 * (A.gl[q] + 1.0));
   }
   // fixed-order warp reduction
   for (int off = 16; off > 0; off >>= 1) {

@@ -25,6 +25,8 @@
 
 namespace nupm {
 
+__global__ void k_nu_nodes(NuArgs A) { nu_node_entry(A, blockIdx.x * blockDim.x + threadIdx.x); }
+
 __global__ void k_nu_panels(NuArgs A) { nu_panels_item(A, blockIdx.x * 4 + (threadIdx.x >> 5)); }
 
 // Finish of every bin and the list of the non-empty ones, in one CTA (nk <= 1024).
@@ -60,7 +62,9 @@ void launch_I_table(double* coef, cudaStream_t s) { k_I_table<<<kISeg, kICoef, 0
 
 void launch_nu_panels(const NuArgs& a, cudaStream_t s) {
   const int items = a.nk * a.ns * kNuChunks;
-  if (items > 0) k_nu_panels<<<(items + 3) / 4, 128, 0, s>>>(a);
+  if (items <= 0) return;
+  if (a.nodes) k_nu_nodes<<<(a.n_hist + 1) * a.quad / 32 + 1, 32, 0, s>>>(a);
+  k_nu_panels<<<(items + 3) / 4, 128, 0, s>>>(a);
 }
 
 void launch_nu_finish(const NuArgs& a, cudaStream_t s) {

@@ -96,6 +96,7 @@ struct NuArgs {
   double stab_u0, stab_inv_h, stab_h;
   const double* gl;               // [2][quad] nodes, weights on [-1, 1]
   const double* icheb;            // [kISeg][kICoef] Chebyshev pieces of I(x)
+  double2* nodes;                 // [n_hist + 1][quad] points of the whole intervals, then (s_end, H) (nu_node_entry), or null
   double* parts;                  // [ns][nk][kNuChunks][3] IC, J_hist, W_cur per panel chunk
   int nchunks;                    // chunks in use (<= kNuChunks), from a bound on the panel count
   double* rlist;                  // [2 nk + 1]: ln k_b and R_b of the non-empty bins, then their count
@@ -258,7 +259,7 @@ struct BoxArgs {
   double* psum;           // the box's sum w |delta|^2 per bin
 };
 enum BatchPass {
-  kBpCount, kBpScan, kBpScatter, kBpDeposit, kBpY, kBpZ, kBpBins, kBpBinReduce, kBpPanels, kBpFinish, kBpRlist,
+  kBpCount, kBpScan, kBpScatter, kBpDeposit, kBpY, kBpZ, kBpBins, kBpBinReduce, kBpNodes, kBpPanels, kBpFinish,
   kBpFac, kBpPlane0, kBpZInv, kBpYInv, kBpXInv, kBpGather, kBpPasses
 };
 struct BatchPlan {
@@ -270,7 +271,7 @@ struct BatchPlan {
 };
 // Items of each pass for one box (grid n, np particles, nk bins, ns response
 // species, bin_chunks partials rows); the grid sizes the batch supports.
-void batch_items(int n, int64_t np, int nk, int ns, int bin_chunks, int* items);
+void batch_items(int n, int64_t np, int nk, int ns, int n_hist_max, int quad, int bin_chunks, int* items);
 bool batch_supported(int n);
 // The kick's passes on stream s; the response panels on `side`, forked after
 // the staging copies (ev_fork) and joined before the finish (ev_join).

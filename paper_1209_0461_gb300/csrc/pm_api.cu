@@ -47,6 +47,7 @@ struct pm_ctx {
   double* d_hist_u = nullptr;
   double* d_gl = nullptr;
   double* d_parts = nullptr;  // [ns][nk][3]
+  double2* d_nodes = nullptr; // [n_hist_max + 1][quad]
   double* d_R = nullptr;
   double* d_pnu = nullptr;
   double* d_pm = nullptr;
@@ -514,7 +515,7 @@ void release(pm_ctx* c) {
                   c->d_stab, c->d_hist_u, c->d_gl, c->d_parts, c->d_R, c->d_pnu, c->d_pm, c->d_rlist, c->d_gtab,
                   c->d_dtab, c->d_wtab, c->d_plane0, c->d_fac, c->d_rowc, c->d_rows, c->d_rowcur,
                   c->d_scantot, c->d_perm, c->d_rec, c->d_status, c->d_hist_u2, c->d_rtab, c->d_icheb, c->d_hist_own,
-                  c->d_prev[0], c->d_prev[1], c->d_inv, c->d_accs};
+                  c->d_prev[0], c->d_prev[1], c->d_inv, c->d_accs, c->d_nodes};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_hist_u) cudaFreeHost(c->h_hist_u);
@@ -735,6 +736,8 @@ int pm_init(const pm_params* params, const double* sqrtPnu_init, const double* t
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_hist_u2, (size_t)(p.n_hist_max + 1) * sizeof(double), "history ln a");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_gl, 2 * kMaxQuad * sizeof(double), "quadrature");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_parts, (size_t)nspec * c->nk * kNuChunks * 3 * sizeof(double), "response parts");
+  if (rc == PM_OK)
+    rc = dalloc(c, (void**)&c->d_nodes, ((size_t)(p.n_hist_max + 1) * c->quad + 1) * sizeof(double2), "response nodes");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_rlist, (2 * (size_t)c->nk + 1) * sizeof(double), "ratio list");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_R, (size_t)c->nk * sizeof(double), "ratio");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_pnu, (size_t)c->nk * sizeof(double), "P_nu");
@@ -1035,6 +1038,9 @@ NuArgs nu_args(pm_ctx* c, double a, const double* sqrtPM_hist, int32_t n_hist, c
     A.nchunks = ch < 1 ? 1 : (ch > kNuChunks ? kNuChunks : ch);
   }
   A.parts = c->d_parts;
+  // the table of the whole intervals' points takes a launch of its own: 32 bins
+  // on 16 nodes lose it (137.8 against 134.1 us a kick), 256 on 128 gain 30 us
+  A.nodes = (int64_t)c->nk * n_hist >= 2048 ? c->d_nodes : nullptr;
   A.rlist = c->d_rlist;
   A.R = c->d_R;
   A.pnu = c->d_pnu;
@@ -1086,7 +1092,7 @@ int pm_nu_response(pm_ctx* c, double a, const double* a_hist, const double* sqrt
     return fail(c, PM_ERR_ORDER, "pm_nu_response before pm_deposit");
   }
   const bool nu = c->ns > 0 && c->f_nu > 0;
-  Stage stage(c, PM_ST_RESPONSE, (nu && !use_prep ? 1 : 0) + 2);   // [panels,] finish + bin list, table
+  Stage stage(c, PM_ST_RESPONSE, (nu && !use_prep ? 1 + (c->nk * (int64_t)n_hist >= 2048) : 0) + 2);   // [nodes, panels,] finish + bin list, table
   NuArgs A = nu_args(c, a, sqrtPM_hist, n_hist, sqrtPnu_prev, ratio_out, sqrtPnu_out, sqrtPM_out);
   if (use_prep) A.hist_u = c->d_hist_u2;
   if (nu && !use_prep) launch_nu_panels(A, c->stream);
@@ -1132,7 +1138,7 @@ int pm_nu_prepare(pm_ctx* c, double a, const double* a_hist, const double* sqrtP
     A.hist_u = c->d_hist_u2;
     A.bins = c->d_bins_lattice;   // |k| of the bins: the lattice's (the deposit may rewrite d_bins meanwhile)
     launch_nu_panels(A, c->side);
-    c->st_launch[PM_ST_RESPONSE] += 1;
+    c->st_launch[PM_ST_RESPONSE] += A.nodes ? 2 : 1;
     if (t0) {
       cudaEvent_t t1 = take_event(c);
       cudaEventRecord(t1, c->side);
@@ -1749,7 +1755,7 @@ int pm_batch_create(pm_ctx* const* ctxs, int32_t nbox, void* cuda_stream, pm_bat
     B->bin_chunks[b] = chunks;
     const int ns = (c->ns > 0 && c->f_nu > 0) ? c->ns : 0;
     int items[kBpPasses];
-    batch_items(c->n, c->np, c->nk, ns, chunks, items);
+    batch_items(c->n, c->np, c->nk, ns, c->p.n_hist_max, c->quad, chunks, items);
     for (int p = 0; p < kBpPasses; ++p) B->first[(size_t)p * (nbox + 1) + b + 1] = items[p];
   }
   for (int p = 0; p < kBpPasses; ++p)
