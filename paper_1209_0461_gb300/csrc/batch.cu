@@ -279,7 +279,8 @@ struct PZInv {
   using CC = ColNarrow<T, N>;
   static constexpr int THREADS = CC::THREADS;
   static constexpr size_t SMEM =
-      (size_t)CC::SMEM_WORDS * sizeof(C) + kFacTable * sizeof(float) + (size_t)CC::E * CC::THREADS * sizeof(T);
+      (size_t)CC::SMEM_WORDS * sizeof(C) + (green_stages_fac<T, N>() ? kFacTable * sizeof(float) : 0) +
+      (size_t)(N / 2 + 1) * CC::W * sizeof(T);
   __device__ static void run(const BoxArgs& b, int item) {
     constexpr int M = N / 2, NX = M / CC::W;
     C* f = reinterpret_cast<C*>(b.g.g);

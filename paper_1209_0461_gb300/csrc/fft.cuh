@@ -369,6 +369,21 @@ k_fft_col(cx<T>* __restrict__ data, int64_t other_stride, int64_t elem_stride,
 // from plane0[ky][kz] (k_green_plane0).  NOUT = 1: the potential alone (the
 // gradient is then taken in real space by the gather).  grid = (M / W, N)
 // ---------------------------------------------------------------------------
+// G = coeff fac(u) / n^2, u = ln sqrt(n^2), fac linear in u on the table.
+__device__ __forceinline__ float green_from_fac(const float* __restrict__ fac, int n2, float fac_inv_du, float coeff) {
+  const float tt = 0.5f * __logf((float)n2) * fac_inv_du;
+  const int j = min((int)tt, kFacTableDev - 2);
+  const float fr = tt - (float)j;
+  const float f0 = fac[j];
+  return coeff * (f0 + fr * (fac[j + 1] - f0)) / (float)n2;
+}
+// The fac table (8 KB) in shared memory: only for tiles of many more factors
+// than its 2048 entries; otherwise it is read through L1.
+template <typename T, int N>
+__host__ __device__ constexpr bool green_stages_fac() {
+  return sizeof(T) == 4 && N > 256;
+}
+
 template <typename T, int N, class Cfg, int NOUT>
 __device__ __forceinline__ void fft_z_inv_green_tile(const cx<T>* __restrict__ spec, cx<T>* __restrict__ out_phi,
                                                      cx<T>* __restrict__ out_dz, const cx<T>* __restrict__ plane0,
@@ -380,11 +395,12 @@ __device__ __forceinline__ void fft_z_inv_green_tile(const cx<T>* __restrict__ s
   constexpr int M = N / 2, E = Cfg::E, NT = Cfg::NT, W = Cfg::W, RL = last_radix<T, N, P>();
   constexpr int64_t ES = (int64_t)N * M;   // element stride along z
   constexpr bool kFac = sizeof(T) == 4;    // FP32: G from the fac table, no n^2 gathers
+  constexpr bool kStage = green_stages_fac<T, N>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int c = threadIdx.x % W;
   const int t = threadIdx.x / W;
   float* fac_s = reinterpret_cast<float*>(smem_raw + (size_t)Cfg::SMEM_WORDS * sizeof(cx<T>));
-  if constexpr (kFac) {
+  if constexpr (kStage) {
     for (int j = threadIdx.x; j < kFacTableDev; j += blockDim.x) fac_s[j] = fac[j];
     __syncthreads();
   }
@@ -394,30 +410,10 @@ __device__ __forceinline__ void fft_z_inv_green_tile(const cx<T>* __restrict__ s
   const int base2 = ky * ky + x2 * x2;
   const int64_t off = (int64_t)iy * M + x2;
   ColSmem<T, W, Cfg::PAD> sm{reinterpret_cast<cx<T>*>(smem_raw), c};
-  const T wyx = wtab ? wtab[iy] * wtab[x2] : (T)1;
-  // Green factors of this thread's elements, once per tile, into its own
-  // shared-memory slots (layout [i][thread]): keeps them out of registers
-  T* gs = reinterpret_cast<T*>(fac_s + (kFac ? kFacTableDev : 0));
+  // Green factors of the tile, [|kz|][column]: kz and -kz share theirs, so half
+  // of a factor an element, worked out while the tile's loads travel
+  T* gs = reinterpret_cast<T*>(fac_s + (kStage ? kFacTableDev : 0));
   const bool col0 = x2 == 0;
-#pragma unroll 1
-  for (int i = 0; i < E; ++i) {
-    const int iz = t + NT * i;
-    const int kz = iz < N / 2 ? iz : iz - N;
-    const int n2 = max(base2 + kz * kz, 1);            // >= 1 unless col0
-    T g;
-    if constexpr (kFac) {
-      // G = coeff fac(u) / n^2, u = ln sqrt(n^2), fac linear in u on the table
-      const float tt = 0.5f * __logf((float)n2) * fac_inv_du;
-      const int j = min((int)tt, kFacTableDev - 2);
-      const float fr = tt - (float)j;
-      const float fv = fac_s[j] + fr * (fac_s[j + 1] - fac_s[j]);
-      g = (T)(coeff * fv / (float)n2);
-    } else {
-      g = gtab[n2];
-    }
-    if (wtab) g *= wyx * wtab[iz];
-    gs[i * Cfg::THREADS + threadIdx.x] = col0 ? (T)1 : g;
-  }
   // branch-free loads: the packed column x2 = 0 reads its pre-multiplied
   // plane0 values (element stride 1), every other column the spectrum
   const cx<T>* src = col0 ? plane0 + (int64_t)iy * N : spec + off;
@@ -427,11 +423,25 @@ __device__ __forceinline__ void fft_z_inv_green_tile(const cx<T>* __restrict__ s
     cx<T> v[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) v[i] = src[(int64_t)(t + NT * i) * sstride];
+    if (pass == 0) {
+      const T wyx = wtab ? wtab[iy] * wtab[x2] : (T)1;
+#pragma unroll 1
+      for (int kz = t; kz <= N / 2; kz += NT) {
+        const int n2 = max(base2 + kz * kz, 1);            // >= 1 unless col0
+        T g;
+        if constexpr (kFac) g = green_from_fac(kStage ? fac_s : fac, n2, fac_inv_du, coeff);
+        else g = gtab[n2];
+        if (wtab) g *= wyx * wtab[kz];
+        gs[kz * W + c] = col0 ? (T)1 : g;
+      }
+      __syncthreads();
+    }
 #pragma unroll
     for (int i = 0; i < E; ++i) {
-      cx<T> f = cscale(v[i], gs[i * Cfg::THREADS + threadIdx.x]);
+      const int iz = t + NT * i;
+      cx<T> f = cscale(v[i], gs[(i < E / 2 ? iz : N - iz) * W + c]);
       if (pass == 1) {
-        const T d = dtab[t + NT * i];
+        const T d = dtab[iz];
         f = {d * f.y, -d * f.x};                 // -i D(kz) f
       }
       v[i] = f;

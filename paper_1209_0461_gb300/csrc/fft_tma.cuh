@@ -241,7 +241,7 @@ struct ColTmaZCfg {
   static constexpr size_t XCH_BYTES = (size_t)ColSmem<T, W, PAD>::words(N) * sizeof(cx<T>);
   static constexpr size_t BUF_BYTES = XCH_BYTES > TILE_BYTES ? XCH_BYTES : TILE_BYTES;
   static constexpr size_t FAC_BYTES = sizeof(T) == 4 ? 2048 * sizeof(float) : 0;
-  static constexpr size_t GS_BYTES = (size_t)E * THREADS * sizeof(T);   // Green factors [E][THREADS]
+  static constexpr size_t GS_BYTES = (size_t)(N / 2 + 1) * W * sizeof(T);   // Green factors [|kz|][column]
   static constexpr size_t SMEM = BUF_BYTES + FAC_BYTES + GS_BYTES + 64;
   static constexpr int TILES_PER_ROW = M / W;
   static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
@@ -288,29 +288,23 @@ k_col_tma_z(const __grid_constant__ CUtensorMap map, ColTmaArgs<T> A) {
   int k = 0;
   for (int item = first; item < items; item += step, ++k) {
     if constexpr (MODE != kColFwdZ) {
-      // Green factors of this tile (each thread its own slots) while its copy
-      // is in flight; the packed column x2 = 0 reads its plane0 values later
+      // Green factors of this tile, one for kz and -kz, while its copy is in
+      // flight (the barrier after the wait publishes them; the previous tile's
+      // reads lie before its exchange barriers); the packed column x2 = 0 reads
+      // its plane0 values later
       const int x2 = (item % Cfg::TILES_PER_ROW) * W + c, y = item / Cfg::TILES_PER_ROW;
       const int ky = y < N / 2 ? y : y - N;
       const int base2 = ky * ky + x2 * x2;
       const T wyx = A.wtab ? A.wtab[y] * A.wtab[x2] : (T)1;
       if (x2 != 0) {
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-          const int iz = t + NT * i;
-          const int kz = iz < N / 2 ? iz : iz - N;
+#pragma unroll 4
+        for (int kz = t; kz <= N / 2; kz += NT) {
           const int n2 = base2 + kz * kz;
           T gval;
-          if constexpr (kFac) {
-            const float tt = 0.5f * __logf((float)n2) * A.fac_inv_du;
-            const int j = min((int)tt, 2048 - 2);
-            const float fr = tt - (float)j;
-            gval = (T)(A.coeff * (fac_s[j] + fr * (fac_s[j + 1] - fac_s[j])) / (float)n2);
-          } else {
-            gval = A.gtab[n2];
-          }
-          if (A.wtab) gval *= wyx * A.wtab[iz];
-          gs[i * Cfg::THREADS + threadIdx.x] = gval;
+          if constexpr (kFac) gval = green_from_fac(fac_s, n2, A.fac_inv_du, A.coeff);
+          else gval = A.gtab[n2];
+          if (A.wtab) gval *= wyx * A.wtab[kz];
+          gs[kz * W + c] = gval;
         }
       }
     }
@@ -352,7 +346,7 @@ k_col_tma_z(const __grid_constant__ CUtensorMap map, ColTmaArgs<T> A) {
           if (x2 == 0) {   // packed column: its pre-multiplied kx = 0 / N/2 values
             f = A.plane0[(int64_t)y * N + iz];
           } else {
-            f = cscale(v[i], gs[i * Cfg::THREADS + threadIdx.x]);
+            f = cscale(v[i], gs[(i < E / 2 ? iz : N - iz) * W + c]);
           }
           if (tr == 1) {
             const T d = A.dtab[iz];

@@ -16,12 +16,12 @@ using T = NUPM_T;
 using C = cx<T>;
 constexpr int kSMs = 152;
 
-// Shared memory of the Green z pass: exchange buffer, fac table (FP32) and
-// the per-thread Green factors.
+// Shared memory of the Green z pass: exchange buffer, fac table (FP32, long
+// columns) and the Green factors of |kz| = 0 .. N/2.
 template <int N, class CC>
 constexpr size_t green_smem() {
-  return (size_t)CC::SMEM_WORDS * sizeof(C) + (sizeof(T) == 4 ? kFacTable * sizeof(float) : 0) +
-         (size_t)CC::E * CC::THREADS * sizeof(T);
+  return (size_t)CC::SMEM_WORDS * sizeof(C) + (green_stages_fac<T, N>() ? kFacTable * sizeof(float) : 0) +
+         (size_t)(N / 2 + 1) * CC::W * sizeof(T);
 }
 template <class CC>
 constexpr size_t col_smem() {
