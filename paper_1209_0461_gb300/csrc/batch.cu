@@ -33,7 +33,6 @@ constexpr int kSortSteps = 4;                  // warp batches per row-sort item
 constexpr int kSortChunk = 256 * kSortBatch * kSortSteps;   // particles per row-sort item (a CTA of 256)
 constexpr int kFacGroup = 256;                  // fac-table entries per item
 constexpr int kPlaneGroup = 256;                // Green-plane entries per item
-constexpr int kScanThreads = 1024;
 
 // The persistent loop: take (box, item) pairs from `counter` until the pass's
 // total is reached.  first[b] = the pass's first item of box b, first[nbox] =
@@ -72,87 +71,13 @@ struct PCount {
   }
 };
 
-// Exclusive scan of the box's N^2 + 1 row counts into row_start and
-// row_cursor by one CTA, kScanPer consecutive values a thread per round
-// (16-byte loads and stores) with a carried offset; the counts are cleared
-// for the next kick.
-constexpr int kScanPer = 16;
+// Exclusive scan of the box's N^2 + 1 row counts into row_start and row_cursor
+// by one CTA (row_scan_cta), which clears the counts for the next kick.
 struct PScan {
-  static constexpr int THREADS = kScanThreads;
+  static constexpr int THREADS = kScanBlock;
   static constexpr size_t SMEM = 0;
   __device__ static void run(const BoxArgs& b, int) {
-    __shared__ int wsum[32];
-    __shared__ int carry_s;
-    const int len = b.g.n * b.g.n + 1;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carry_s = 0;
-    __syncthreads();
-    for (int r0 = 0; r0 < len; r0 += kScanPer * kScanThreads) {
-      const int i0 = r0 + kScanPer * tid;
-      const bool whole = i0 + kScanPer <= len;   // i0 is a multiple of 16: 16-byte aligned
-      int v[kScanPer], s = 0;
-      if (whole) {
-#pragma unroll
-        for (int q = 0; q < kScanPer / 4; ++q) {
-          const int4 x = reinterpret_cast<const int4*>(b.g.row_count + i0)[q];
-          v[4 * q] = x.x;
-          v[4 * q + 1] = x.y;
-          v[4 * q + 2] = x.z;
-          v[4 * q + 3] = x.w;
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k) v[k] = i0 + k < len ? b.g.row_count[i0 + k] : 0;
-      }
-#pragma unroll
-      for (int k = 0; k < kScanPer; ++k) s += v[k];
-      int incl = s;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-      }
-      if (lane == 31) wsum[warp] = incl;
-      __syncthreads();
-      if (warp == 0) {
-        const int w0 = wsum[lane];
-        int wi = w0;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, wi, off);
-          if (lane >= off) wi += y;
-        }
-        wsum[lane] = wi - w0;
-      }
-      __syncthreads();
-      int e = carry_s + wsum[warp] + incl - s;
-      int ex[kScanPer];
-#pragma unroll
-      for (int k = 0; k < kScanPer; ++k) {
-        ex[k] = e;
-        e += v[k];
-      }
-      if (whole) {
-#pragma unroll
-        for (int q = 0; q < kScanPer / 4; ++q) {
-          const int4 x = make_int4(ex[4 * q], ex[4 * q + 1], ex[4 * q + 2], ex[4 * q + 3]);
-          reinterpret_cast<int4*>(b.g.row_start + i0)[q] = x;
-          reinterpret_cast<int4*>(b.g.row_cursor + i0)[q] = x;
-          reinterpret_cast<int4*>(b.g.row_count + i0)[q] = make_int4(0, 0, 0, 0);
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < kScanPer; ++k)
-          if (i0 + k < len) {
-            b.g.row_start[i0 + k] = ex[k];
-            b.g.row_cursor[i0 + k] = ex[k];
-            b.g.row_count[i0 + k] = 0;
-          }
-      }
-      __syncthreads();   // every thread has read carry_s
-      if (tid == kScanThreads - 1) carry_s = e;
-      __syncthreads();
-    }
+    row_scan_cta(b.g.row_count, b.g.row_start, b.g.row_cursor, b.g.n * b.g.n + 1);
   }
 };
 

@@ -603,7 +603,10 @@ struct FusedCfg {
   using P = FusedPlan<T, M>;
   static constexpr int E = P::R1;
   static constexpr int NT = M / E;
-  static constexpr int G = 32 / NT;                 // rows per warp
+  // rows per warp: all its lanes, but two at most on grids of up to 32 points,
+  // where eight rows one after another left most SMs idle (18 us at 32^3; the
+  // lanes past them repeat the last row's transform)
+  static constexpr int G = (N <= 32 && 32 / NT > 2) ? 2 : 32 / NT;
   static constexpr int WARPS = 4;
   static constexpr int ROWS = G * WARPS;            // rows per CTA
   static constexpr int THREADS = 32 * WARPS;
@@ -736,7 +739,8 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
   if (__any_sync(0xffffffffu, ovf) && lane == 0 && status) atomicCAS(status, 0, PM_ERR_OVERFLOW);
   __syncwarp();
   // forward x transform of the warp's rows (as k_fft_x_fwd), NT lanes a row
-  const int t = lane % NT, r = lane / NT;
+  const int t = lane % NT, r = lane / NT < G ? lane / NT : G - 1;
+  const bool mine = lane < G * NT;   // not a repeat
   const int64_t grow = row0 + r;
   unsigned char* rowp = wrows + r * Cfg::ROW_BYTES;
   const uint2* lo2 = reinterpret_cast<const uint2*>(rowp);                 // low words of cells 2e, 2e+1
@@ -791,7 +795,7 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
     const cx<T> wo = cmul(twid_table<-1>(tw_n, k), od);
     cx<T> out = {ev.x + wo.y, ev.y - wo.x};
     if (j == 0 && t == 0) out = {zk.x + zk.y, zk.x - zk.y};
-    dst[k] = out;
+    if (mine) dst[k] = out;
   }
 }
 

@@ -380,14 +380,18 @@ int NUPM_FN(deposit)(const GridArgs& g, const void* pos, cudaStream_t s) {
 
 int NUPM_FN(row_sort)(const GridArgs& g, const void* pos, cudaStream_t s) {
   const int rows = g.n * g.n;
-  cudaMemsetAsync(g.row_count, 0, (size_t)(rows + 1) * sizeof(int), s);
+  // row_count is zero here: cleared at pm_init and by every sort's scan
   const int blocks = grid_blocks(g.np, 256, g.part_ctas_per_sm);
   if (g.np > 0) k_row_count<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.cell, g.row_count, g.status);
   const int len = rows + 1;
   const int nb = (len + 2 * kScanBlock - 1) / (2 * kScanBlock);
-  k_scan_blocks<<<nb, kScanBlock, 0, s>>>(g.row_count, g.row_start, g.scan_tot, len);
-  k_scan_totals<<<1, kScanBlock, 0, s>>>(g.scan_tot, nb);
-  k_scan_add<<<(len + 255) / 256, 256, 0, s>>>(g.row_start, g.scan_tot, len, g.row_cursor);
+  if (g.n <= kScanOneMax) {
+    k_scan_one<<<1, kScanBlock, 0, s>>>(g.row_count, g.row_start, g.row_cursor, len);
+  } else {
+    k_scan_blocks<<<nb, kScanBlock, 0, s>>>(g.row_count, g.row_start, g.scan_tot, len);
+    k_scan_totals<<<1, kScanBlock, 0, s>>>(g.scan_tot, nb);
+    k_scan_add<<<(len + 255) / 256, 256, 0, s>>>(g.row_start, g.scan_tot, len, g.row_cursor);
+  }
   if (g.np > 0)
     k_row_scatter<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.cell, g.row_cursor, g.perm, g.rec, g.inv);
   return PM_OK;

@@ -401,12 +401,15 @@ __device__ __forceinline__ void nu_finish_bin(const NuArgs& A, int b) {
     double ic = 0.0, jh = 0.0, wc = 0.0, guess = 0.0;
     for (int s = 0; s < A.ns; ++s) {
       double qi = 0.0, qj = 0.0, qw = 0.0;
-      for (int ch = 0; ch < A.nchunks; ++ch) {   // fixed chunk order
-        const double* q = A.parts + (((int64_t)s * A.nk + b) * kNuChunks + ch) * 3;
-        qi += q[0];
-        qj += q[1];
-        qw += q[2];
-      }
+      // fixed chunk order; unrolled, so that the loads travel together
+      const double* q = A.parts + ((int64_t)s * A.nk + b) * kNuChunks * 3;
+#pragma unroll
+      for (int ch = 0; ch < kNuChunks; ++ch)
+        if (ch < A.nchunks) {
+          qi += q[3 * ch];
+          qj += q[3 * ch + 1];
+          qw += q[3 * ch + 2];
+        }
       ic += A.w_species[s] * qi;
       jh += A.w_species[s] * qj;
       wc += A.w_species[s] * qw;

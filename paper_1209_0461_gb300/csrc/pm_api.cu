@@ -103,7 +103,6 @@ struct pm_ctx {
   // state
   bool deposited = false, deposit_grid_valid = false, have_response = false, have_kick = false;
   bool power_set = false;         // bins replaced by pm_set_power (no spectrum behind them)
-  bool counts_dirty = true;       // row counts hold a direct row sort's values (a batched kick clears them)
   int wide_y = -1, wide_z = -1, part_cps = 16;   // tuning (pm_autotune)
   int gather_rows = 0;                            // tuning: gather in the sort's row order
   bool perm_valid = false;                        // the last deposit's sort wrote perm
@@ -749,6 +748,7 @@ int pm_init(const pm_params* params, const double* sqrtPnu_init, const double* t
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_fac, kFacTable * sizeof(float), "fac table");
   const size_t nrow1 = (size_t)n * n + 1;
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_rowc, nrow1 * sizeof(int), "row counts");
+  if (rc == PM_OK) rc = cuda_check(c, cudaMemset(c->d_rowc, 0, nrow1 * sizeof(int)), "row count clear");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_rows, nrow1 * sizeof(int), "row starts");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_rowcur, nrow1 * sizeof(int), "row cursors");
   if (rc == PM_OK) rc = dalloc(c, (void**)&c->d_scantot, 2048 * sizeof(int), "scan totals");
@@ -884,9 +884,8 @@ int pm_deposit(pm_ctx* c, const void* pos) {
     }
   } else {
     {
-      Stage st(c, PM_ST_DEPOSIT, 5);
+      Stage st(c, PM_ST_DEPOSIT, c->n <= 64 ? 3 : 5);
       rc = c->fp64 ? row_sort_f64(g, pos, c->stream) : row_sort_f32(g, pos, c->stream);
-      c->counts_dirty = true;
     }
     if (rc == PM_OK) {
       Stage st(c, PM_ST_FFT_X_FWD, 1);
@@ -1846,12 +1845,6 @@ int pm_batch_kick(pm_batch* B, const void* const* pos, void* const* vel, const d
                                                    cudaMemcpyDeviceToDevice, B->stream), "lattice bins restore");
       if (rc != PM_OK) return B->err = c->err, rc;
       c->power_set = false;
-    }
-    if (c->counts_dirty) {   // the batched count adds to zeros; its scan clears them again
-      const int rc = cuda_check(c, cudaMemsetAsync(c->d_rowc, 0, ((size_t)c->n * c->n + 1) * sizeof(int), B->stream),
-                                "row count clear");
-      if (rc != PM_OK) return B->err = c->err, rc;
-      c->counts_dirty = false;
     }
     for (int j = 0; j < nh; ++j) hh[(size_t)b * B->hist_stride + j] = log(ah[j]);
     any_hist = any_hist || nh > 0;

@@ -5,13 +5,20 @@
 
 namespace nupm {
 
-// Block b scans in[b*2048 .. b*2048+2047] (exclusive) into out, total -> totals[b].
-__global__ void k_scan_blocks(const int* __restrict__ in, int* __restrict__ out, int* __restrict__ totals, int n) {
+__global__ void __launch_bounds__(kScanBlock) k_scan_one(int* __restrict__ count, int* __restrict__ start,
+                                                         int* __restrict__ cursor, int len) {
+  row_scan_cta(count, start, cursor, len);
+}
+
+// Block b scans in[b*2048 .. b*2048+2047] (exclusive) into out, total -> totals[b], and clears in.
+__global__ void k_scan_blocks(int* __restrict__ in, int* __restrict__ out, int* __restrict__ totals, int n) {
   __shared__ int warp_sum[kScanBlock / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t i0 = (int64_t)blockIdx.x * 2 * kScanBlock + 2 * tid;
   const int a = i0 < n ? in[i0] : 0;
   const int b = i0 + 1 < n ? in[i0 + 1] : 0;
+  if (i0 < n) in[i0] = 0;
+  if (i0 + 1 < n) in[i0 + 1] = 0;
   int s = a + b;
   int incl = s;
 #pragma unroll

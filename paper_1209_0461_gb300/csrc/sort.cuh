@@ -65,6 +65,7 @@ __device__ __forceinline__ unsigned long long pack_record(const int (&c)[3], con
 // Each warp takes kSortBatch x 32 consecutive particles per step (all their
 // loads in flight first); the match below sees every lane of the warp.
 constexpr int kSortBatch = 4;
+constexpr int kScanBlock = 1024;   // threads of the scan kernels (k_scan_blocks: 2 values per thread)
 
 // One warp's kSortBatch x 32 particles from `base` on (the warp-uniform body
 // of k_row_count; also run by the batched form).
@@ -154,11 +155,94 @@ __global__ void k_row_scatter(const void* __restrict__ pos, int64_t np, int n, C
     row_scatter_warp<T>(pos, np, n, cell, cursor, perm, rec, base, inv);
 }
 
-// Exclusive scan of n values in three launches: per-block scans of 2048
-// values (block totals out), a single-block scan of the totals, and the add.
-constexpr int kScanBlock = 1024;   // threads; 2 values per thread
+// Exclusive scan of len row counts into start and cursor by one CTA of
+// kScanBlock threads, kScanPer consecutive values a thread per round (16-byte
+// loads and stores) with a carried offset; the counts are cleared for the next sort.
+constexpr int kScanPer = 16;
+__device__ __forceinline__ void row_scan_cta(int* __restrict__ count, int* __restrict__ start,
+                                             int* __restrict__ cursor, int len) {
+  __shared__ int wsum[32];
+  __shared__ int carry_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) carry_s = 0;
+  __syncthreads();
+  for (int r0 = 0; r0 < len; r0 += kScanPer * kScanBlock) {
+    const int i0 = r0 + kScanPer * tid;
+    const bool whole = i0 + kScanPer <= len;   // i0 is a multiple of 16: 16-byte aligned
+    int v[kScanPer], s = 0;
+    if (whole) {
+#pragma unroll
+      for (int q = 0; q < kScanPer / 4; ++q) {
+        const int4 x = reinterpret_cast<const int4*>(count + i0)[q];
+        v[4 * q] = x.x;
+        v[4 * q + 1] = x.y;
+        v[4 * q + 2] = x.z;
+        v[4 * q + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kScanPer; ++k) v[k] = i0 + k < len ? count[i0 + k] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) s += v[k];
+    int incl = s;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += y;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      const int w0 = wsum[lane];
+      int wi = w0;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, wi, off);
+        if (lane >= off) wi += y;
+      }
+      wsum[lane] = wi - w0;
+    }
+    __syncthreads();
+    int e = carry_s + wsum[warp] + incl - s;
+    int ex[kScanPer];
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+      ex[k] = e;
+      e += v[k];
+    }
+    if (whole) {
+#pragma unroll
+      for (int q = 0; q < kScanPer / 4; ++q) {
+        const int4 x = make_int4(ex[4 * q], ex[4 * q + 1], ex[4 * q + 2], ex[4 * q + 3]);
+        reinterpret_cast<int4*>(start + i0)[q] = x;
+        reinterpret_cast<int4*>(cursor + i0)[q] = x;
+        reinterpret_cast<int4*>(count + i0)[q] = make_int4(0, 0, 0, 0);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < kScanPer; ++k)
+        if (i0 + k < len) {
+          start[i0 + k] = ex[k];
+          cursor[i0 + k] = ex[k];
+          count[i0 + k] = 0;
+        }
+    }
+    __syncthreads();   // every thread has read carry_s
+    if (tid == kScanBlock - 1) carry_s = e;
+    __syncthreads();
+  }
+}
+__global__ void k_scan_one(int* __restrict__ count, int* __restrict__ start, int* __restrict__ cursor, int len);
+// Grids whose rows one CTA scans in one round: one launch of 5 us for three of
+// 3 us each (at 128 points it takes two rounds and 13 us: twelve such boxes in a
+// graph lost 1.5%).
+constexpr int kScanOneMax = 64;
 
-__global__ void k_scan_blocks(const int* __restrict__ in, int* __restrict__ out, int* __restrict__ totals,
+// Exclusive scan of n values in three launches (the first clears its input): per-block scans of 2048
+// values (block totals out), a single-block scan of the totals, and the add.
+
+__global__ void k_scan_blocks(int* __restrict__ in, int* __restrict__ out, int* __restrict__ totals,
                               int n);
 __global__ void k_scan_totals(int* __restrict__ totals, int nb);
 __global__ void k_scan_add(int* __restrict__ out, const int* __restrict__ totals, int n, int* __restrict__ cursor);
