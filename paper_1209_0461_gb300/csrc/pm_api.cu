@@ -461,9 +461,13 @@ int encode_col_map(pm_ctx* c, CUtensorMap* map, void* base, int fields, bool alo
 GridArgs grid_args(const pm_ctx* c) {
   GridArgs g;
   g.wide_y = c->wide_y;
-  g.wide_z = c->wide_z;
   g.part_ctas_per_sm = c->part_cps;
   g.fd_grad = !(c->p.flags & (PM_SPECTRAL_GRADIENT | PM_FUSED_GATHER | PM_TMA_COLUMNS));
+  // built-in z passes: the TMA-staged ones with the bin sums on FP32 grids of 1024
+  // points (512^3 particles 17.18 -> 16.79 ms, 256^3 13.32 -> 12.48 ms a kick); on 256
+  // and 512 points, whose planes L2 holds longer, the plain wide tiles (2.20
+  // against 2.25 ms at 512, 0.864 against 0.879 ms at 256; FP64 27.05 against 27.66 ms)
+  g.wide_z = c->wide_z < 0 && c->n == 1024 && !c->fp64 && c->tma_z16 && g.fd_grad ? 2 : c->wide_z;
   g.n = c->n;
   g.np = c->np;
   g.box = c->box;
@@ -488,7 +492,7 @@ GridArgs grid_args(const pm_ctx* c) {
   g.scan_tot = c->d_scantot;
   g.perm = ((c->p.flags & PM_FUSED_GATHER) || c->gather_rows == 1) ? c->d_perm : nullptr;
   g.inv = c->gather_rows == 2 ? c->d_inv : nullptr;
-  g.bins_in_z = !c->fp64 && c->tma_z16 && c->wide_z == 2 && c->nk <= 256;
+  g.bins_in_z = !c->fp64 && c->tma_z16 && g.wide_z == 2 && c->nk <= 256;
   g.bin_thr = c->d_thr;
   g.bin_inv_lr = c->bin_inv_lr;
   g.bin_nk = c->nk;
