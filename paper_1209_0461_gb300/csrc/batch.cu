@@ -220,7 +220,7 @@ template <int N>
 struct PXInv {
   using RC = RowCfg<T, N>;
   static constexpr int THREADS = RC::THREADS;
-  static constexpr size_t SMEM = (size_t)RC::ROWS * RC::ROW_WORDS * sizeof(C);
+  static constexpr size_t SMEM = (size_t)RC::ROWS * RC::INV_ROW_WORDS * sizeof(C);
   __device__ static void run(const BoxArgs& b, int item) {
     fft_x_inv_rows<T, N>(reinterpret_cast<C*>(b.g.g), reinterpret_cast<const C*>(b.g.tw_m),
                          reinterpret_cast<const C*>(b.g.tw_n), reinterpret_cast<const T*>(b.g.dtab), false, item);

@@ -47,8 +47,9 @@ void ensure_attrs() {
   static bool done = false;
   if (done) return;
   const int row_smem = (int)((size_t)RC::ROWS * RC::ROW_WORDS * sizeof(C));
+  const int xinv_smem = (int)((size_t)RC::ROWS * RC::INV_ROW_WORDS * sizeof(C));
   cudaFuncSetAttribute(k_fft_x_fwd<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, row_smem);
-  cudaFuncSetAttribute(k_fft_x_inv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, row_smem);
+  cudaFuncSetAttribute(k_fft_x_inv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, xinv_smem);
   col_attrs<N, ColNarrow<T, N>>();
   col_attrs<N, ColWide<T, N>>();
   done = true;
@@ -242,7 +243,8 @@ void fft_pass_n(const GridArgs& g, int pass, cudaStream_t s) {
     case kPassXInv:
       // x with the x gradient on field 0 (phi -> d/dx phi); fields 1, 2 as they
       // are.  Real-space gradient: the potential alone.
-      k_fft_x_inv<T, N><<<dim3((unsigned)(rows / RC::ROWS), 1, g.fd_grad ? 1 : 3), RC::THREADS, row_smem, s>>>(
+      k_fft_x_inv<T, N><<<dim3((unsigned)(rows / RC::ROWS), 1, g.fd_grad ? 1 : 3), RC::THREADS,
+                          (size_t)RC::ROWS * RC::INV_ROW_WORDS * sizeof(C), s>>>(
           reinterpret_cast<C*>(g.g), g.field_elems, twm, twn, reinterpret_cast<const T*>(g.dtab),
           g.fd_grad ? 0 : 1);
       break;
