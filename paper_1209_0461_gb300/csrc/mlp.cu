@@ -250,9 +250,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) k_mlp_backward(MlpArgs A) {
   float* outs = sm + MlpSmem::OUT;
   float* dout = sm + MlpSmem::DOUT;
   float* red = sm + MlpSmem::RED;
-  for (int idx = tid; idx < kW * kW; idx += kBwdThreads) {
-    const int j = idx / kW, k = idx % kW;                // W2[j][k]
-    W2s[k * kWP + j] = bf(A.W2[idx]);
+  // W2, eight BF16 a load and all of a thread's loads in flight (2-byte loads took
+  // sixteen round trips, 3 us of a minibatch that is one tile a CTA)
+  uint4 wv[kW * kW / 8 / kBwdThreads];
+#pragma unroll
+  for (int q = 0; q < kW * kW / 8 / kBwdThreads; ++q) wv[q] = reinterpret_cast<const uint4*>(A.W2)[tid + q * kBwdThreads];
+#pragma unroll
+  for (int q = 0; q < kW * kW / 8 / kBwdThreads; ++q) {
+    const int idx = 8 * (tid + q * kBwdThreads), j = idx / kW, k = idx % kW;   // W2[j][k .. k + 7]
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&wv[q]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      W2s[(k + 2 * e) * kWP + j] = __low2float(h[e]);
+      W2s[(k + 2 * e + 1) * kWP + j] = __high2float(h[e]);
+    }
   }
   float dW2[2][32], dW1[2][kMaxIn], db1[2] = {0.0f, 0.0f}, db2[2] = {0.0f, 0.0f}, dw3[2] = {0.0f, 0.0f};
   float db3 = 0.0f, loss = 0.0f, w3[2], b1[2], b2[2];
