@@ -1547,7 +1547,8 @@ int pm_autotune(pm_ctx* c, const void* pos, void* vel, double a, const double* a
     return rc;
   };
   static const int kStY[2] = {PM_ST_FFT_Y_FWD, PM_ST_FFT_Y_INV};
-  static const int kStZ[2] = {PM_ST_FFT_Z_FWD, PM_ST_FFT_Z_INV};
+  // the bin sums count with the z passes: wide_z = 2 makes them in the forward one
+  static const int kStZ[3] = {PM_ST_FFT_Z_FWD, PM_ST_FFT_Z_INV, PM_ST_BINS};
   static const int kStP[2] = {PM_ST_DEPOSIT, PM_ST_INTERP};
   int rc = PM_OK;
   double t0 = 0.0, t1 = 0.0;
@@ -1556,18 +1557,19 @@ int pm_autotune(pm_ctx* c, const void* pos, void* vel, double a, const double* a
   for (int pass = 0; pass < 2 && rc == PM_OK; ++pass) {
     int& knob = pass == 0 ? c->wide_y : c->wide_z;
     const int* st = pass == 0 ? kStY : kStZ;
+    const int nst = pass == 0 ? 2 : 3;
     knob = 0;
-    rc = measure(st, 2, &t0);
+    rc = measure(st, nst, &t0);
     if (rc != PM_OK) break;
     knob = 1;
-    rc = measure(st, 2, &t1);
+    rc = measure(st, nst, &t1);
     if (rc != PM_OK) break;
     knob = t1 < t0 ? 1 : 0;
     if (pass == 1 && c->tma_z16) {   // TMA-staged z passes
       double t2 = 0.0;
       const int prev = knob;
       knob = 2;
-      rc = measure(st, 2, &t2);
+      rc = measure(st, nst, &t2);
       if (rc != PM_OK) break;
       knob = t2 < (t1 < t0 ? t1 : t0) ? 2 : prev;
     }
