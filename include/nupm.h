@@ -431,7 +431,7 @@ NUPM_API void pm_graph_free(pm_graph* graph);
 /* ---- batched kicks (the batched form) ----
  * Boxes of ONE grid size stepped together: each pass of the kick (row count,
  * row scan, row scatter, deposit + x, y, z, bin sums and their reduction,
- * response panels, finish, bin list, fac table, Green plane, Green + z
+ * response nodes and panels, finish + bin list, fac table, Green plane, Green + z
  * inverse, y inverse, x inverse, gather + kick) is one persistent kernel over
  * all boxes, whose CTAs take (box, item) pairs -- particle chunks, row or
  * column tiles, response panels -- from an atomic counter until the pass's

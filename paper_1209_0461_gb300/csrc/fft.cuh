@@ -594,11 +594,12 @@ k_fft_x_fwd(const unsigned long long* __restrict__ grid, cx<T>* __restrict__ spe
 // deposit grid, no memset, no atomics to DRAM.  With `keep` set the sums are
 // also written out (inspection).
 //
-// Bound: issue slots and the shared-memory pipe (16 atomic adds a particle
-// and the exchanges).  A record is read by four warps (L1 and L2 after the
-// first) where a CTA tile of 2 x 4 rows read it 1.9 times, but there two
-// thirds of the corner adds fell outside the tile, and phases waited at
-// barriers.
+// Bound: the shared-memory pipe (16 atomic adds a particle at 2.5 wavefronts, and
+// the exchanges: LSU data pipe 85%, ALU 56% at 256^3).  A record is read by four
+// warps (L1 and L2 after the first) where a CTA tile of 2 x 4 rows read it 1.9
+// times, but there half of the corner adds issued fell outside the tile, and
+// phases waited at barriers: 3.90 -> 2.77 ms at 1024^3 points / 512^3 particles,
+// 0.281 -> 0.135 ms at 256^3.
 // ---------------------------------------------------------------------------
 template <typename T, int N>
 struct FusedCfg {

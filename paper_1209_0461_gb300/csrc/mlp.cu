@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) k_mlp_backward(MlpArgs A) {
   float* dout = sm + MlpSmem::DOUT;
   float* red = sm + MlpSmem::RED;
   // W2, eight BF16 a load and all of a thread's loads in flight (2-byte loads took
-  // sixteen round trips, 3 us of a minibatch that is one tile a CTA)
+  // sixteen round trips, 2 us of a minibatch that is one tile a CTA)
   uint4 wv[kW * kW / 8 / kBwdThreads];
 #pragma unroll
   for (int q = 0; q < kW * kW / 8 / kBwdThreads; ++q) wv[q] = reinterpret_cast<const uint4*>(A.W2)[tid + q * kBwdThreads];
