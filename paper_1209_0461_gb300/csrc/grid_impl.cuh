@@ -29,7 +29,7 @@ constexpr size_t col_smem() {
 }
 
 // Opt the FFT kernels of size N into their dynamic shared memory (once per
-// process; every kernel of this size gets its attribute on first use).
+// device; every kernel of this size gets its attribute on first use).
 template <int N, class CC>
 void col_attrs() {
   cudaFuncSetAttribute(k_fft_col<T, N, -1, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)col_smem<CC>());
@@ -42,17 +42,17 @@ void col_attrs() {
                        (int)col_smem<CC>());
 }
 template <int N>
-void ensure_attrs() {
+void ensure_attrs(int device) {
   using RC = RowCfg<T, N>;
-  static bool done = false;
-  if (done) return;
+  static DeviceSet done;
+  if (done.has(device)) return;
   const int row_smem = (int)((size_t)RC::ROWS * RC::ROW_WORDS * sizeof(C));
   const int xinv_smem = (int)((size_t)RC::ROWS * RC::INV_ROW_WORDS * sizeof(C));
   cudaFuncSetAttribute(k_fft_x_fwd<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, row_smem);
   cudaFuncSetAttribute(k_fft_x_inv<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, xinv_smem);
   col_attrs<N, ColNarrow<T, N>>();
   col_attrs<N, ColWide<T, N>>();
-  done = true;
+  done.add(device);
 }
 
 // Column passes with tile config CC: forward y / z, Green z, gradient y.
@@ -99,10 +99,10 @@ void col_pass(const GridArgs& g, int pass, cudaStream_t s) {
 template <int N, int MODE>
 void col_tma_n(const GridArgs& g, const CUtensorMap* map, cudaStream_t s) {
   using Cfg = ColTmaCfg<T, N>;
-  static bool attr = false;
-  if (!attr) {
+  static DeviceSet attr;
+  if (!attr.has(g.device)) {
     cudaFuncSetAttribute(k_col_tma<T, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    attr = true;
+    attr.add(g.device);
   }
   ColTmaArgs<T> a;
   a.spec = reinterpret_cast<C*>(g.spec);
@@ -154,10 +154,10 @@ static inline int z_fwd_grid(const GridArgs& g) {
 template <int N, int MODE>
 void col_tma_z_n(const GridArgs& g, cudaStream_t s) {
   using Cfg = ColTmaZCfg<T, N>;
-  static bool attr = false;
-  if (!attr) {
+  static DeviceSet attr;
+  if (!attr.has(g.device)) {
     cudaFuncSetAttribute(k_col_tma_z<T, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    attr = true;
+    attr.add(g.device);
   }
   ColTmaArgs<T> a;
   a.spec = reinterpret_cast<C*>(g.spec);
@@ -182,10 +182,10 @@ void col_tma_z_n(const GridArgs& g, cudaStream_t s) {
     // in a split-buffer form).  With bins_in_z it also sums the bins' power.
     if (g.bins_in_z) {
       using FC = ColTmaZFwdCfg<N, true>;
-      static bool battr = false;
-      if (!battr) {
+      static DeviceSet battr;
+      if (!battr.has(g.device)) {
         cudaFuncSetAttribute(k_col_tma_z_fwd<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC::SMEM);
-        battr = true;
+        battr.add(g.device);
       }
       a.thr = g.bin_thr;
       a.inv_lr = g.bin_inv_lr;
@@ -194,10 +194,10 @@ void col_tma_z_n(const GridArgs& g, cudaStream_t s) {
       k_col_tma_z_fwd<N, true><<<grid, FC::THREADS, FC::SMEM, s>>>(*g.tmap_z16, a);
     } else {
       using FC = ColTmaZFwdCfg<N, false>;
-      static bool fattr = false;
-      if (!fattr) {
+      static DeviceSet fattr;
+      if (!fattr.has(g.device)) {
         cudaFuncSetAttribute(k_col_tma_z_fwd<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FC::SMEM);
-        fattr = true;
+        fattr.add(g.device);
       }
       k_col_tma_z_fwd<N, false><<<grid, FC::THREADS, FC::SMEM, s>>>(*g.tmap_z16, a);
     }
@@ -230,7 +230,7 @@ void fft_pass_n(const GridArgs& g, int pass, cudaStream_t s) {
   constexpr int M = N / 2;
   using RC = RowCfg<T, N>;
   const size_t row_smem = (size_t)RC::ROWS * RC::ROW_WORDS * sizeof(C);
-  ensure_attrs<N>();
+  ensure_attrs<N>(g.device);
   const int64_t rows = (int64_t)N * N;
   const C* twn = reinterpret_cast<const C*>(g.tw_n);
   const C* twm = reinterpret_cast<const C*>(g.tw_m);
@@ -263,10 +263,10 @@ void fft_pass_n(const GridArgs& g, int pass, cudaStream_t s) {
 template <int N>
 void deposit_fft_x_n(const GridArgs& g, const void* pos, bool keep, cudaStream_t s) {
   using F = FusedCfg<T, N>;
-  static bool attr = false;
-  if (!attr) {
+  static DeviceSet attr;
+  if (!attr.has(g.device)) {
     cudaFuncSetAttribute(k_deposit_fft_x<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::SMEM);
-    attr = true;
+    attr.add(g.device);
   }
   k_deposit_fft_x<T, N><<<N * N / F::ROWS, F::THREADS, F::SMEM, s>>>(
       g.rec, g.row_start, reinterpret_cast<C*>(g.spec), DepositScale{g.scale, g.scale_hi, g.scale_lo}, reinterpret_cast<const C*>(g.tw_m),
@@ -277,10 +277,10 @@ void deposit_fft_x_n(const GridArgs& g, const void* pos, bool keep, cudaStream_t
 template <int N>
 void xinv_interp_n(const GridArgs& g, const void* pos, void* vel, double kick, void* acc_out, cudaStream_t s) {
   using X = XiCfg<T, N>;
-  static bool attr = false;
-  if (!attr) {
+  static DeviceSet attr;
+  if (!attr.has(g.device)) {
     cudaFuncSetAttribute(k_xinv_interp<T, N, Quant<T>>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::SMEM);
-    attr = true;
+    attr.add(g.device);
   }
   const int items = (N / X::TZ) * (N / X::LY);
   const int grid = items < g.sm_count ? items : g.sm_count;
@@ -315,10 +315,10 @@ int grid_blocks(int64_t work, int threads, int ctas_per_sm = 16) {
 template <int N>
 void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
   using Cfg = GatherTile<N>;
-  static bool attr = false;
-  if (!attr) {
+  static DeviceSet attr;
+  if (!attr.has(g.device)) {
     cudaFuncSetAttribute(k_gather_tile_acc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    attr = true;
+    attr.add(g.device);
   }
   k_gather_tile_acc<N><<<Cfg::TILES, Cfg::THREADS, Cfg::SMEM, s>>>(
       g.rec, g.row_start, scale, reinterpret_cast<const float*>(g.g), reinterpret_cast<float*>(g.accs));

@@ -7,6 +7,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "../../include/nupm.h"
 
 namespace nupm {
@@ -133,6 +135,20 @@ void launch_fac_table(float* fac, double umax, double kf, double f_nu, const dou
 void launch_green_table(bool fp64, void* gtab, long long n2max, double kf, double coeff,
                         double f_nu, const double* rlist, int nk, cudaStream_t s);
 
+// The devices on which a kernel's attributes were already set: a kernel's dynamic
+// shared memory above 48 KB is allowed per device, by cudaFuncSetAttribute.
+// Threads that meet here at the same time set the same values twice.
+class DeviceSet {
+ public:
+  bool has(int device) const { return device < 64 && (bits_.load(std::memory_order_acquire) >> device & 1) != 0; }
+  void add(int device) {
+    if (device < 64) bits_.fetch_or(1ull << device, std::memory_order_release);
+  }
+
+ private:
+  std::atomic<unsigned long long> bits_{0};
+};
+
 // Cell size of the grid and 65536 / d as a 64-bit mantissa (bit 63 set) and a
 // biased exponent, for the FP64 positions' quantisation in integers (quant_fast
 // in grid_kernels.cuh); re = -65536 (no fast path) where 65536 / d is near the
@@ -168,6 +184,7 @@ constexpr int kPassXFwd = 0, kPassYFwd = 1, kPassZFwd = 2, kPassZInv = 3, kPassY
 
 // precision-dispatched grid launchers (grid_f32.cu / grid_f64.cu)
 struct GridArgs {
+  int device;                     // the context's device
   int n;
   int64_t np;
   double box, delta, scale;       // scale = N^3 / (Np 2^48)

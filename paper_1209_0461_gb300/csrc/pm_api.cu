@@ -72,7 +72,7 @@ struct pm_ctx {
   // FP32 spectrum rows as [N^2][32][N/64] for the staged bin sums
   bool tma_bins = false;
   alignas(64) CUtensorMap tm_bins;
-  int sm_count = 152;
+  int sm_count = 152, device = 0;
   double green_coeff = 0;     // -1.5 Omega_M / (a kf^2 N^3) of the last response
   int* d_status = nullptr;
   // pinned host staging
@@ -505,6 +505,7 @@ GridArgs grid_args(const pm_ctx* c) {
   g.tmap_g_y = c->tma ? &c->tm_g_y : nullptr;
   g.tmap_z16 = c->tma_z16 ? &c->tm_z16 : nullptr;
   g.tmap_bins = c->tma_bins ? &c->tm_bins : nullptr;
+  g.device = c->device;
   g.sm_count = c->sm_count;
   g.fac = c->d_fac;
   g.fac_inv_du = (float)((kFacTable - 1) / (0.5 * log((double)c->n2max)));
@@ -818,9 +819,8 @@ int pm_init(const pm_params* params, const double* sqrtPnu_init, const double* t
   }
   if (rc == PM_OK) rc = build_s_table(c, 0.0 > log(c->a_init) ? 0.0 : log(c->a_init) + 1.0);
   if (rc == PM_OK) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev);
+    cudaGetDevice(&c->device);
+    cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device);
     if (p.flags & PM_TMA_COLUMNS) {
       const int w = c->fp64 ? 4 : 8;   // 64-byte row segments
       rc = encode_col_map(c, &c->tm_spec_y, c->spec, 1, false, w);
