@@ -311,7 +311,15 @@ int grid_blocks(int64_t work, int threads, int ctas_per_sm = 16) {
   return (int)b;
 }
 
-// Forces by sorted slot from shared-memory tiles (FP32 grids of up to 512 points; false otherwise).
+// Forces by sorted slot from shared-memory tiles (false: not for this grid and
+// particle number).  A CTA takes at most `cap` particles of a tile: twice the mean, or
+// where a wave holds many tiles as many as make the longest part a sixteenth of the pass.
+// The tiles want half a particle a cell, or staging their rows costs more than it
+// saves: with the velocity pass on clustered particles, tiles against
+// k_interp_rows_acc, 37 / 33 us for a quarter and 45 / 50 us for a half at 128^3
+// points, 0.171 / 0.173 and 0.267 / 0.300 ms at 256^3, 1.34 / 1.23 and 2.15 / 2.38 ms
+// at 512^3.  And 128 points: 64^3 has fewer tiles than a wave holds, and parts do
+// not even that out (one filament 29 / 24 us).
 template <int N>
 void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
   using Cfg = GatherTile<N>;
@@ -320,16 +328,17 @@ void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
     cudaFuncSetAttribute(k_gather_tile_acc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     attr.add(g.device);
   }
-  k_gather_tile_acc<N><<<Cfg::TILES, Cfg::THREADS, Cfg::SMEM, s>>>(
-      g.rec, g.row_start, scale, reinterpret_cast<const float*>(g.g), reinterpret_cast<float*>(g.accs));
+  const int helpers = 2 * g.sm_count;
+  const int64_t mean = g.np / Cfg::TILES + 1, share = g.np / ((int64_t)16 * g.sm_count * Cfg::CTAS);
+  const unsigned cap = (unsigned)(2 * mean > share ? 2 * mean : share);
+  k_gather_tile_acc<N><<<helpers + Cfg::TILES, Cfg::THREADS, Cfg::SMEM, s>>>(
+      g.rec, g.row_start, helpers, cap, scale, reinterpret_cast<const float*>(g.g), reinterpret_cast<float*>(g.accs));
 }
 template <typename U>
 bool gather_tiled(const GridArgs& g, U scale, cudaStream_t s) {
   if constexpr (sizeof(U) == 4) {
+    if (2 * g.np < (int64_t)g.n * g.n * g.n) return false;
     switch (g.n) {
-      case 16: gather_tile_n<16>(g, scale, s); return true;
-      case 32: gather_tile_n<32>(g, scale, s); return true;
-      case 64: gather_tile_n<64>(g, scale, s); return true;
       case 128: gather_tile_n<128>(g, scale, s); return true;
       case 192: gather_tile_n<192>(g, scale, s); return true;
       case 256: gather_tile_n<256>(g, scale, s); return true;

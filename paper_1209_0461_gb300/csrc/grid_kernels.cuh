@@ -1325,8 +1325,9 @@ __global__ void k_kick_inv(const int* __restrict__ inv, const T* __restrict__ ac
   }
 }
 
-// k_interp_rows_acc from shared memory, FP32 grids of up to 512 points (longer
-// rows do not fit).  A CTA owns the particles that the deposit's sort placed
+// k_interp_rows_acc from shared memory, FP32 grids of 128 to 512 points (longer
+// rows do not fit, smaller grids have too few tiles: gather_tiled).  A CTA owns the
+// particles that the deposit's sort placed
 // in TZ x TY grid rows (whole rows along x) and stages the potential rows their
 // stencils touch: TZ + 1 planes of TY + 5 rows and, for the z differences, TY + 1
 // rows of the two planes on either side; each row with a halo of its periodic
@@ -1347,6 +1348,7 @@ struct GatherTile {
   static constexpr int THREADS = N <= 256 ? 384 : 512;    // 36 warps per SM in three CTAs, 32 in two at 512
   static constexpr int CTAS = N <= 256 ? 3 : 2;
   static constexpr int TILES = (N / TY) * (N / TZ);
+  static constexpr int LOOK = 8;                          // tiles a thread looks at together
   static_assert(N % 4 == 0 && CTAS * (SMEM + 1024) <= 227 * 1024, "tile shared memory");
 };
 
@@ -1419,32 +1421,32 @@ __device__ __forceinline__ void gather_tile_stencil(const float* sm, int c0, int
   fd_combine<float>(px, py, pz, w, a);
 }
 
-// Tile blockIdx.x of TILES: the forces of the particles of its rows by sorted slot.
+// The forces by sorted slot of particles [from, to) of a tile's rows.  Ends with a barrier.
 template <int N>
-__global__ void __launch_bounds__(GatherTile<N>::THREADS, GatherTile<N>::CTAS)
-k_gather_tile_acc(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start, float scale,
-                  const float* __restrict__ phi, float* __restrict__ accs) {
+__device__ __forceinline__ void gather_tile_part(const unsigned long long* __restrict__ rec,
+                                                 const int* __restrict__ row_start, float scale,
+                                                 const float* __restrict__ phi, float* __restrict__ accs, float* sm,
+                                                 int tile, unsigned from, unsigned to) {
   using Cfg = GatherTile<N>;
   constexpr int TY = Cfg::TY, TZ = Cfg::TZ;
-  constexpr int YM = (N < 32 ? N : 32) - 1;   // the record holds y mod 32
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* sm = reinterpret_cast<float*>(smem_raw);
-  const int y0 = (blockIdx.x % (N / TY)) * TY, z0 = (blockIdx.x / (N / TY)) * TZ;
+  constexpr int YM = 31;                      // the record holds y mod 32
+  const int y0 = (tile % (N / TY)) * TY, z0 = (tile / (N / TY)) * TZ;
   // the rows y0 .. y0 + TY - 1 of a plane are one run of sorted slots: TZ runs,
   // concatenated in a virtual index j
-  int pre[TZ + 1], off[TZ];
+  unsigned pre[TZ + 1];
+  int off[TZ];
   pre[0] = 0;
 #pragma unroll
   for (int q = 0; q < TZ; ++q) {
     const int r = (z0 + q) * N + y0;
     const int b = row_start[r];
-    off[q] = b - pre[q];
-    pre[q + 1] = pre[q] + row_start[r + TY] - b;
+    off[q] = b - (int)pre[q];
+    pre[q + 1] = pre[q] + (unsigned)(row_start[r + TY] - b);
   }
-  const int total = pre[TZ];
-  if (total == 0) return;                 // uniform over the CTA
+  if (to > pre[TZ]) to = pre[TZ];
+  if (from >= to) return;                 // uniform over the CTA
   gather_tile_load<N>(phi, sm, y0, z0);
-  for (int j = threadIdx.x; j < total; j += Cfg::THREADS) {
+  for (unsigned j = from + threadIdx.x; j < to; j += Cfg::THREADS) {
     int zl = 0, o = off[0];
 #pragma unroll
     for (int q = 1; q < TZ; ++q)
@@ -1452,12 +1454,79 @@ k_gather_tile_acc(const unsigned long long* __restrict__ rec, const int* __restr
         o = off[q];
         zl = q;
       }
-    const int64_t i = j + o;
+    const int64_t i = (int64_t)j + o;
     const unsigned long long r = rec[i];
     const int w[3] = {(int)(r & 0xffffu), (int)((r >> 16) & 0xffffu), (int)((r >> 32) & 0xffffu)};
     float a[3];
     gather_tile_stencil<N>(sm, (int)(r >> 48) & 0x7ff, ((int)(r >> 59) - y0) & YM, zl, w, a);
     reinterpret_cast<float4*>(accs)[i] = make_float4(a[0] * scale, a[1] * scale, a[2] * scale, 0.0f);
+  }
+  __syncthreads();
+}
+
+// The last TILES CTAs take a tile each, its first `cap` particles.  What a tile
+// holds beyond them goes in parts of `cap` to the helpers, the CTAs before those
+// (dispatched first): part c of tile t to helper (hash(t) + c) mod helpers.  A helper
+// looks through all tiles and stages the rows of its parts again; without parts
+// they cost 1 us at 128 points, 3 us at 256.  Without helpers a
+// box with much of its mass in a few rows waits for a few CTAs: half of 256^3
+// particles in one filament on 256^3 points 6.4 ms with the velocity pass, 0.51 ms
+// with them (0.59 ms by k_interp_rows_acc; an even box 0.43 ms).
+template <int N>
+__global__ void __launch_bounds__(GatherTile<N>::THREADS, GatherTile<N>::CTAS)
+k_gather_tile_acc(const unsigned long long* __restrict__ rec, const int* __restrict__ row_start, int helpers,
+                  unsigned cap, float scale, const float* __restrict__ phi, float* __restrict__ accs) {
+  using Cfg = GatherTile<N>;
+  constexpr int TY = Cfg::TY, TZ = Cfg::TZ, LOOK = Cfg::LOOK;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* sm = reinterpret_cast<float*>(smem_raw);
+  if ((int)blockIdx.x >= helpers) {
+    gather_tile_part<N>(rec, row_start, scale, phi, accs, sm, (int)blockIdx.x - helpers, 0, cap);
+    return;
+  }
+  __shared__ int pick;
+  // first part of tile t that falls to this helper, in [1, helpers]
+  auto first = [&](int t) {
+    const unsigned turn = ((unsigned)t * 2654435761u >> 16) % (unsigned)helpers;
+    return (blockIdx.x + (unsigned)helpers - turn - 1) % (unsigned)helpers + 1;
+  };
+  auto particles = [&](int t) {
+    const int y0 = (t % (N / TY)) * TY, z0 = (t / (N / TY)) * TZ;
+    unsigned total = 0;
+#pragma unroll
+    for (int q = 0; q < TZ; ++q) {
+      const int r = (z0 + q) * N + y0;
+      total += (unsigned)(row_start[r + TY] - row_start[r]);
+    }
+    return total;
+  };
+  for (int t0 = 0; t0 < Cfg::TILES; t0 += LOOK * Cfg::THREADS) {
+    unsigned total[LOOK], mine = 0;   // bit k: tile t0 + k THREADS + threadIdx.x has a part for this helper
+#pragma unroll
+    for (int k = 0; k < LOOK; ++k) {
+      const int t = t0 + k * Cfg::THREADS + (int)threadIdx.x;
+      total[k] = t < Cfg::TILES ? particles(t) : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < LOOK; ++k) {
+      const int t = t0 + k * Cfg::THREADS + (int)threadIdx.x;
+      if (total[k] > cap && (unsigned long long)first(t) * cap < total[k]) mine |= 1u << k;
+    }
+    for (;;) {
+      if (threadIdx.x == 0) pick = Cfg::TILES;
+      if (!__syncthreads_or((int)mine)) break;
+      const int t = t0 + (__ffs((int)mine) - 1) * Cfg::THREADS + (int)threadIdx.x;
+      if (mine) atomicMin(&pick, t);
+      __syncthreads();
+      const int tile = pick;
+      if (mine && t == tile) mine &= mine - 1;
+      const unsigned all = particles(tile);
+      for (unsigned long long from = (unsigned long long)first(tile) * cap; from < all;
+           from += (unsigned long long)helpers * cap) {
+        const unsigned long long to = from + cap;
+        gather_tile_part<N>(rec, row_start, scale, phi, accs, sm, tile, (unsigned)from, to < all ? (unsigned)to : all);
+      }
+    }
   }
 }
 
