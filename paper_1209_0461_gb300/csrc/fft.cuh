@@ -672,19 +672,27 @@ __device__ __forceinline__ bool deposit_segment(const unsigned long long* __rest
   return ovf;
 }
 
-// The deposit of one node row (gz, gy) by one warp into its zeroed sums.
-// Returns true where a sum wrapped past 2^64.
-template <int N, int kHi>
-__device__ __forceinline__ bool deposit_row_warp(const unsigned long long* __restrict__ rec,
-                                                 const int* __restrict__ row_start, int gz, int gy, unsigned* lo) {
-  int b[4], len[4], total = 0;   // source rows: bit 0 set = row gy (else gy - 1), bit 1 = plane gz (else gz - 1)
+// The four source rows of a node row (gz, gy): bit 0 of s set = row gy (else
+// gy - 1), bit 1 = plane gz (else gz - 1).
+template <int N>
+struct SourceRows {
+  int b[4], len[4], total = 0;
+  __device__ __forceinline__ SourceRows(const int* __restrict__ row_start, int gz, int gy) {
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int r = ((gz + N - 1 + (s >> 1)) % N) * N + (gy + N - 1 + (s & 1)) % N;
-    b[s] = row_start[r];
-    len[s] = row_start[r + 1] - b[s];
-    total += len[s];
+    for (int s = 0; s < 4; ++s) {
+      const int r = ((gz + N - 1 + (s >> 1)) % N) * N + (gy + N - 1 + (s & 1)) % N;
+      b[s] = row_start[r];
+      len[s] = row_start[r + 1] - b[s];
+      total += len[s];
+    }
   }
+};
+
+// The deposit of one node row into its zeroed sums, part `part` of PARTS of
+// every source row.  Returns true where a sum wrapped past 2^64.
+template <int N, int kHi, int PARTS = 1>
+__device__ __forceinline__ bool deposit_row_warp(const unsigned long long* __restrict__ rec, const SourceRows<N>& src,
+                                                 unsigned* lo, int part = 0) {
   // A cell's sum wraps past 2^64 only with 65536 or more contributions of up
   // to 2^48 each; a row with fewer records cannot overflow, and only one with
   // more reads back its high-word adds to detect a wrap (PM_ERR_OVERFLOW).
@@ -692,9 +700,14 @@ __device__ __forceinline__ bool deposit_row_warp(const unsigned long long* __res
 #pragma unroll 1
   for (int s = 0; s < 4; ++s) {
     const int sy = (s & 1) ? -1 : 1, ay = (s & 1) ? 65536 : 0, sz = (s & 2) ? -1 : 1, az = (s & 2) ? 65536 : 0;
-    const int bs = s == 0 ? b[0] : s == 1 ? b[1] : s == 2 ? b[2] : b[3];
-    const int ls = s == 0 ? len[0] : s == 1 ? len[1] : s == 2 ? len[2] : len[3];
-    if (total < 65536) deposit_segment<kHi, false>(rec + bs, ls, sy, ay, sz, az, lo);
+    int bs = s == 0 ? src.b[0] : s == 1 ? src.b[1] : s == 2 ? src.b[2] : src.b[3];
+    int ls = s == 0 ? src.len[0] : s == 1 ? src.len[1] : s == 2 ? src.len[2] : src.len[3];
+    if constexpr (PARTS > 1) {
+      const int per = ls / PARTS;
+      bs += per * part;
+      ls = part == PARTS - 1 ? ls - per * part : per;
+    }
+    if (src.total < 65536) deposit_segment<kHi, false>(rec + bs, ls, sy, ay, sz, az, lo);
     else ovf |= deposit_segment<kHi, true>(rec + bs, ls, sy, ay, sz, az, lo);
   }
   return ovf;
@@ -706,6 +719,9 @@ struct DepositScale {
   double s;
   float hi, lo;
 };
+
+// Records of a node row from which its CTA's warps share it (grids of 512 points on).
+constexpr int kLongRow = 32768;
 
 // Rows ROWS bx .. ROWS (bx + 1) - 1.
 template <typename T, int N>
@@ -725,11 +741,33 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
   for (int i = lane; i < (int)(G * Cfg::ROW_BYTES / 16); i += 32) reinterpret_cast<uint4*>(wrows)[i] = uint4{0, 0, 0, 0};
   __syncwarp();
   bool ovf = false;
+  bool shared = false;
+  if constexpr (N >= 512) {
+    // a row of very many records would be one warp's serial chain of shared-memory
+    // round trips: the CTA's warps then share its rows (2% of 256^3 particles in one of
+    // 512^2 rows: 1.11 ms, 2.24 by one warp; FP64 5.06 and 6.40; even boxes as without).  Small
+    // grids have their time in the adds themselves.
+    int most = 0;
+    for (int g = 0; g < G; ++g) most = max(most, SourceRows<N>(row_start, (row0 + g) / N, (row0 + g) % N).total);
+    shared = __syncthreads_or(most >= kLongRow);
+    if (shared) {
 #pragma unroll 1
-  for (int g = 0; g < G; ++g) {
-    const int row = row0 + g;
-    ovf |= deposit_row_warp<N, Cfg::HI>(rec, row_start, row / N, row % N,
-                                        reinterpret_cast<unsigned*>(wrows + g * Cfg::ROW_BYTES));
+      for (int k = 0; k < Cfg::ROWS; ++k) {
+        const int row = bx * Cfg::ROWS + k;
+        ovf |= deposit_row_warp<N, Cfg::HI, Cfg::WARPS>(
+            rec, SourceRows<N>(row_start, row / N, row % N),
+            reinterpret_cast<unsigned*>(smem_raw + (size_t)k * Cfg::ROW_BYTES), warp);
+      }
+      __syncthreads();
+    }
+  }
+  if (!shared) {
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+      const int row = row0 + g;
+      ovf |= deposit_row_warp<N, Cfg::HI>(rec, SourceRows<N>(row_start, row / N, row % N),
+                                          reinterpret_cast<unsigned*>(wrows + g * Cfg::ROW_BYTES));
+    }
   }
   __syncwarp();
   if (lane < G) {   // word N is cell 0's
