@@ -1066,7 +1066,7 @@ __device__ __forceinline__ void fd_combine(const T (&px)[2][2][6], const T (&py)
 // at 256^3), 4-byte loads of the x runs too (0.372; 3.55 against 3.09 ms at
 // 1024^3).  With wrapped indices for all particles and a run-time test of n in
 // every wrap it took 0.365 and 3.19 ms.
-template <typename T, bool POW2>
+template <typename T, bool POW2, bool PAIRS = sizeof(T) == 4>
 __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, const int (&c)[3], const int (&w)[3],
                                            T (&a)[3]) {
   uint32_t yo[6], zo[6];   // row offsets; indices < 2^30 for n <= 1024
@@ -1081,7 +1081,11 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
   constexpr int kFar[4] = {0, 1, 4, 5};
   // (FP64 takes the wrapped indices throughout: its bound is the FP64 pipe, and
   // both branches' 56 values in flight would spill)
-  if (sizeof(T) == 4 && c[0] >= 2 && c[0] + 4 <= n) {
+  const bool inside = sizeof(T) == 4 && c[0] >= 2 && c[0] + 4 <= n;
+  int xs[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) xs[j] = wrap_near<POW2>(c[0], j - 2, n);
+  if (inside) {
     const T* b = phi + c[0];
     const int odd = c[0] & 1;
 #pragma unroll
@@ -1096,6 +1100,26 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
 #pragma unroll
         for (int j = 0; j < 6; ++j) px[dz][dy][j] = (T)(odd ? w8[j + 1] : w8[j]);
       }
+  } else {
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy) {
+        const T* r = phi + (zo[2 + dz] + yo[2 + dy]);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) px[dz][dy][j] = r[xs[j]];
+      }
+  }
+  // the pairs (x0, x0 + 1) of the far rows: decided by the warp, not by the lane, or a
+  // warp with one particle at an end of its row would load all pairs twice (16 million
+  // particles in no order: 0.93 -> 0.83 ms on 16^3 points, 1.59 -> 1.55 ms on 128^3).
+  // Without PAIRS always by the wrapped indices: in the row order most warps have such a
+  // particle, and its kernel has no registers for both (96 spilled 48 bytes and
+  // ran 5% slower)
+  bool all = false;
+  if constexpr (PAIRS) all = __all_sync(__activemask(), inside);
+  if (all) {
+    const T* b = phi + c[0];
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
@@ -1113,17 +1137,6 @@ __device__ __forceinline__ void fd_stencil(const T* __restrict__ phi, int n, con
         pz[dy][1][q] = r[1];
       }
   } else {
-    int xs[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) xs[j] = wrap_near<POW2>(c[0], j - 2, n);
-#pragma unroll
-    for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-      for (int dy = 0; dy < 2; ++dy) {
-        const T* r = phi + (zo[2 + dz] + yo[2 + dy]);
-#pragma unroll
-        for (int j = 0; j < 6; ++j) px[dz][dy][j] = r[xs[j]];
-      }
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
@@ -1234,7 +1247,7 @@ k_interp_rows_fd(const unsigned long long* __restrict__ rec, const int* __restri
       const int c[3] = {(int)(r >> 48) & 0x7ff, cy, cz};
       const int w[3] = {(int)(r & 0xffffu), (int)((r >> 16) & 0xffffu), (int)((r >> 32) & 0xffffu)};
       T a[3];
-      fd_stencil<T, POW2>(phi, n, c, w, a);
+      fd_stencil<T, POW2, false>(phi, n, c, w, a);
       const T u[3] = {u0, u1, u2};
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
