@@ -267,7 +267,7 @@ void launch_pass(const BatchPlan& p, int pass, size_t smem, cudaStream_t s) {
 }
 
 template <int N>
-void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
+int batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
   // the response panels read the bins' lattice |k| sums and the history only:
   // they run on the side stream beside the deposit and the transforms
   cudaEventRecord(ev_fork, s);
@@ -277,6 +277,10 @@ void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEve
   cudaEventRecord(ev_join, side);
   launch_pass<PCount>(p, kBpCount, 0, s);
   launch_pass<PScan>(p, kBpScan, 0, s);
+  if (cudaPeekAtLastError() != cudaSuccess) {   // no scatter by an earlier sort's cursors
+    cudaStreamWaitEvent(s, ev_join, 0);
+    return PM_ERR_CUDA;
+  }
   launch_pass<PScatter>(p, kBpScatter, 0, s);
   launch_pass<PDeposit<N>>(p, kBpDeposit, PDeposit<N>::SMEM, s);
   launch_pass<PCol<N, -1, false, false>>(p, kBpY, PCol<N, -1, false, false>::SMEM, s);
@@ -291,6 +295,7 @@ void batch_kick_n(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEve
   launch_pass<PCol<N, +1, false, true>>(p, kBpYInv, PCol<N, +1, false, true>::SMEM, s);
   launch_pass<PXInv<N>>(p, kBpXInv, PXInv<N>::SMEM, s);
   launch_pass<PGather<N>>(p, kBpGather, 0, s);
+  return PM_OK;
 }
 
 }  // namespace
@@ -352,15 +357,14 @@ void batch_items(int n, int64_t np, int nk, int ns, int n_hist_max, int quad, in
 
 int batch_kick(const BatchPlan& p, cudaStream_t s, cudaStream_t side, cudaEvent_t ev_fork, cudaEvent_t ev_join) {
   switch (p.n) {
-    case 16: batch_kick_n<16>(p, s, side, ev_fork, ev_join); break;
-    case 32: batch_kick_n<32>(p, s, side, ev_fork, ev_join); break;
-    case 64: batch_kick_n<64>(p, s, side, ev_fork, ev_join); break;
-    case 128: batch_kick_n<128>(p, s, side, ev_fork, ev_join); break;
-    case 192: batch_kick_n<192>(p, s, side, ev_fork, ev_join); break;
-    case 256: batch_kick_n<256>(p, s, side, ev_fork, ev_join); break;
+    case 16: return batch_kick_n<16>(p, s, side, ev_fork, ev_join);
+    case 32: return batch_kick_n<32>(p, s, side, ev_fork, ev_join);
+    case 64: return batch_kick_n<64>(p, s, side, ev_fork, ev_join);
+    case 128: return batch_kick_n<128>(p, s, side, ev_fork, ev_join);
+    case 192: return batch_kick_n<192>(p, s, side, ev_fork, ev_join);
+    case 256: return batch_kick_n<256>(p, s, side, ev_fork, ev_join);
     default: return PM_ERR_UNSUPPORTED;
   }
-  return PM_OK;
 }
 
 }  // namespace nupm

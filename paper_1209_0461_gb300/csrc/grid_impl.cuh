@@ -391,7 +391,8 @@ int NUPM_FN(deposit)(const GridArgs& g, const void* pos, cudaStream_t s) {
 
 int NUPM_FN(row_sort)(const GridArgs& g, const void* pos, cudaStream_t s) {
   const int rows = g.n * g.n;
-  // row_count is zero here: cleared at pm_init and by every sort's scan
+  // row_count is zero here: cleared at pm_init, by every sort's scan, and by the
+  // caller where a scan did not run
   const int blocks = grid_blocks(g.np, 256, g.part_ctas_per_sm);
   if (g.np > 0) k_row_count<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.cell, g.row_count, g.status);
   const int len = rows + 1;
@@ -403,6 +404,8 @@ int NUPM_FN(row_sort)(const GridArgs& g, const void* pos, cudaStream_t s) {
     k_scan_totals<<<1, kScanBlock, 0, s>>>(g.scan_tot, nb);
     k_scan_add<<<(len + 255) / 256, 256, 0, s>>>(g.row_start, g.scan_tot, len, g.row_cursor);
   }
+  // the scatter writes where the cursors say: not by those of an earlier sort
+  if (cudaPeekAtLastError() != cudaSuccess) return PM_ERR_CUDA;
   if (g.np > 0)
     k_row_scatter<T><<<blocks, 256, 0, s>>>(pos, g.np, g.n, g.cell, g.row_cursor, g.perm, g.rec, g.inv);
   return PM_OK;

@@ -101,6 +101,7 @@ struct pm_ctx {
   int prev_cur = 0;
   bool have_prev = false;
   // state
+  bool counts_dirty = false;      // a row count ran whose scan did not (begin_counts)
   bool deposited = false, deposit_grid_valid = false, have_response = false, have_kick = false;
   bool power_set = false;         // bins replaced by pm_set_power (no spectrum behind them)
   int wide_y = -1, wide_z = -1, part_cps = 16;   // tuning (pm_autotune)
@@ -864,6 +865,58 @@ int pm_init(const pm_params* params, const double* sqrtPnu_init, const double* t
   return PM_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The row counts are zero between sorts: every scan clears what its count added.
+// A sort brackets its count and scan with these two.  Where a launch between them
+// failed (the first use of a kernel on a full device, say), the counts are cleared at
+// once, or if that fails too before the next count.  What a stream captures does
+// not run, so there the state of the counts stays what it was.
+struct CountsState {
+  bool was_dirty = false;
+};
+int begin_counts(pm_ctx* c, cudaStream_t s, CountsState* st) {
+  st->was_dirty = c->counts_dirty;
+  if (st->was_dirty) {
+    const int rc = cuda_check(c, cudaMemsetAsync(c->d_rowc, 0, ((size_t)c->n * c->n + 1) * sizeof(int), s), "row count clear");
+    if (rc != PM_OK) return rc;
+  }
+  c->counts_dirty = true;
+  return PM_OK;
+}
+void end_counts(pm_ctx* c, cudaStream_t s, CountsState* st, bool scanned) {
+  if (st->was_dirty || !scanned) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      c->counts_dirty = st->was_dirty;
+      return;
+    }
+  }
+  if (!scanned && cudaMemsetAsync(c->d_rowc, 0, ((size_t)c->n * c->n + 1) * sizeof(int), s) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  c->counts_dirty = false;
+}
+
+// The deposit's row sort.
+int sort_rows(pm_ctx* c, const GridArgs& g, const void* pos) {
+  CountsState st;
+  int rc = begin_counts(c, c->stream, &st);
+  if (rc != PM_OK) return rc;
+  rc = c->fp64 ? row_sort_f64(g, pos, c->stream) : row_sort_f32(g, pos, c->stream);
+  if (rc != PM_OK) cuda_check(c, cudaGetLastError(), "pm_deposit row sort");
+  end_counts(c, c->stream, &st, rc == PM_OK);
+  return rc;
+}
+
+}  // namespace
+
+extern "C" {
+
 int pm_deposit(pm_ctx* c, const void* pos) {
   if (!c) return PM_ERR_INVALID;
   if (!pos) return fail(c, PM_ERR_INVALID, "pm_deposit: pos is NULL");
@@ -889,8 +942,9 @@ int pm_deposit(pm_ctx* c, const void* pos) {
   } else {
     {
       Stage st(c, PM_ST_DEPOSIT, c->n <= 64 ? 3 : 5);
-      rc = c->fp64 ? row_sort_f64(g, pos, c->stream) : row_sort_f32(g, pos, c->stream);
+      rc = sort_rows(c, g, pos);
     }
+    if (rc == PM_ERR_CUDA) return rc;
     if (rc == PM_OK) {
       Stage st(c, PM_ST_FFT_X_FWD, 1);
       rc = c->fp64 ? deposit_fft_x_f64(g, pos, keep, c->stream) : deposit_fft_x_f32(g, pos, keep, c->stream);
@@ -1886,13 +1940,19 @@ int pm_batch_kick(pm_batch* B, const void* const* pos, void* const* vel, const d
     B->err = std::string("pm_batch_kick: ") + cudaGetErrorString(e);
     return PM_ERR_CUDA;
   }
-  int rc = batch_kick(B->plan, B->stream, B->side, B->ev_fork, B->ev_join);
-  if (rc != PM_OK) return B->err = "pm_batch_kick: unsupported grid", rc;
+  std::vector<CountsState> counts(nbox);
+  for (int b = 0; b < nbox; ++b) {
+    const int rc = begin_counts(B->ctx[b], B->stream, &counts[b]);
+    if (rc != PM_OK) return B->err = B->ctx[b]->err, rc;
+  }
+  const int rc = batch_kick(B->plan, B->stream, B->side, B->ev_fork, B->ev_join);
   e = cudaGetLastError();
+  for (int b = 0; b < nbox; ++b) end_counts(B->ctx[b], B->stream, &counts[b], rc == PM_OK && e == cudaSuccess);
   if (e != cudaSuccess) {
     B->err = std::string("pm_batch_kick launch: ") + cudaGetErrorString(e);
     return PM_ERR_CUDA;
   }
+  if (rc != PM_OK) return B->err = "pm_batch_kick: unsupported grid", rc;
   for (int b = 0; b < nbox; ++b) {   // each context now holds this kick's results
     pm_ctx* c = B->ctx[b];
     c->deposited = true;
