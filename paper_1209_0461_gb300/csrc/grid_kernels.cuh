@@ -954,7 +954,7 @@ __device__ __forceinline__ void fold_weights(T f0, T f1, T (&e)[6]) {
 // GB300 issues two of those a cycle and SM, and this takes about ten integer ones)
 __device__ __forceinline__ double exact_pow2(unsigned u, int sh, bool neg) {
   const int lz = __clz(u);
-  const unsigned m = (u << lz) << 1;                      // mantissa below the leading one
+  const unsigned m = __funnelshift_lc(0u, u, lz) << 1;    // mantissa below the leading one (a shift by 32 is defined: u = 0)
   const unsigned hi = ((unsigned)(1023 + 31 - lz - sh) << 20) | (m >> 12) | (neg ? 0x80000000u : 0u);
   return __hiloint2double(u ? (int)hi : 0, (int)(m << 20));
 }
