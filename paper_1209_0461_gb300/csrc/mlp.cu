@@ -108,6 +108,13 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t a0, const
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
 }
 
+// Two packed BF16 values with those that are not finite replaced by zero.
+__device__ __forceinline__ uint32_t finite_part(uint32_t w) {
+  if ((w & 0x7f80u) == 0x7f80u) w &= 0xffff0000u;
+  if ((w & 0x7f800000u) == 0x7f800000u) w &= 0xffffu;
+  return w;
+}
+
 // One warp per 16 samples.  Lane (g, q) = (lane / 4, lane % 4) holds rows g and
 // g + 8; layer 1 is evaluated straight into the A fragments of layer 2: per k
 // tile of 16 hidden units the lane needs units 2q, 2q + 1, 2q + 8, 2q + 9 of
@@ -128,11 +135,15 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 3) k_mlp_forward(MlpArgs A) {
   float2* bw = reinterpret_cast<float2*>(smf + FwdSmem::BW);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
   float* xs = reinterpret_cast<float*>(smf + FwdSmem::X) + warp * 16 * kXP;
-  // fragment (kt, nt, lane): W2[8 nt + g][16 kt + 2q + {0, 1}] and + 8
+  // fragment (kt, nt, lane): W2[8 nt + g][16 kt + 2q + {0, 1}] and + 8; weights that
+  // are not finite apart (below)
+  bool odd = false;
   for (int i = threadIdx.x; i < 8 * 16 * 32; i += blockDim.x) {
     const int l = i & 31, nt = (i >> 5) & 15, kt = i >> 9;
     const __nv_bfloat16* w = A.W2 + (8 * nt + (l >> 2)) * kW + 16 * kt + 2 * (l & 3);
-    Bs[i] = make_uint2(*reinterpret_cast<const uint32_t*>(w), *reinterpret_cast<const uint32_t*>(w + 8));
+    const uint2 b = make_uint2(*reinterpret_cast<const uint32_t*>(w), *reinterpret_cast<const uint32_t*>(w + 8));
+    Bs[i] = make_uint2(finite_part(b.x), finite_part(b.y));
+    odd = odd || Bs[i].x != b.x || Bs[i].y != b.y;
   }
   for (int i = threadIdx.x; i < kW * kMaxIn; i += blockDim.x) {
     const int u = i / kMaxIn, c = i % kMaxIn;
@@ -142,7 +153,28 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 3) k_mlp_forward(MlpArgs A) {
     b1s[i] = A.b1[i];
     bw[i] = make_float2(A.b2[i], bf(A.w3[i]));
   }
-  __syncthreads();
+  odd = __syncthreads_or(odd);
+  // units u, u + 1 of layer 1 for two rows of inputs: h[row][unit]
+  auto layer1 = [&](const float (&x)[2][kMaxIn], int u, float (&h)[2][2]) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      float acc0 = b1s[u + e], acc1 = acc0;
+#pragma unroll
+      for (int c = 0; c < kMaxIn; c += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(W1s + (u + e) * kW1P + c);
+        acc0 = fmaf(w.x, x[0][c], acc0);
+        acc1 = fmaf(w.x, x[1][c], acc1);
+        acc0 = fmaf(w.y, x[0][c + 1], acc0);
+        acc1 = fmaf(w.y, x[1][c + 1], acc1);
+        acc0 = fmaf(w.z, x[0][c + 2], acc0);
+        acc1 = fmaf(w.z, x[1][c + 2], acc1);
+        acc0 = fmaf(w.w, x[0][c + 3], acc0);
+        acc1 = fmaf(w.w, x[1][c + 3], acc1);
+      }
+      h[0][e] = tanhf(acc0);
+      h[1][e] = tanhf(acc1);
+    }
+  };
   const float b3 = A.b3[0];
   const int64_t tiles = (A.n + 15) / 16;
   for (int64_t t = (int64_t)blockIdx.x * kFwdWarps + warp; t < tiles; t += (int64_t)gridDim.x * kFwdWarps) {
@@ -168,31 +200,38 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 3) k_mlp_forward(MlpArgs A) {
     float z[16][4];
 #pragma unroll
     for (int nt = 0; nt < 16; ++nt) z[nt][0] = z[nt][1] = z[nt][2] = z[nt][3] = 0.0f;
+    // Weights that are not finite (a master weight past the BF16 range is one): times
+    // the high word of h1 alone, which has its sign.  The lower words may be zero or of
+    // the other sign, and their product or the sum would be a NaN.
+    if (odd) {
+#pragma unroll 1
+      for (int kt = 0; kt < 8; ++kt) {
+        uint32_t a[4];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          float h[2][2];
+          layer1(x, 16 * kt + 8 * p + 2 * q, h);
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const __nv_bfloat162 v = __floats2bfloat162_rn(h[r][0], h[r][1]);
+            a[2 * p + r] = *reinterpret_cast<const uint32_t*>(&v);
+          }
+        }
+#pragma unroll
+        for (int nt = 0; nt < 16; ++nt) {
+          const __nv_bfloat16* w = A.W2 + (8 * nt + g) * kW + 16 * kt + 2 * q;
+          const uint2 b = make_uint2(*reinterpret_cast<const uint32_t*>(w), *reinterpret_cast<const uint32_t*>(w + 8));
+          mma_bf16(z[nt], a[0], a[1], a[2], a[3], make_uint2(b.x ^ finite_part(b.x), b.y ^ finite_part(b.y)));
+        }
+      }
+    }
 #pragma unroll 1
     for (int kt = 0; kt < 8; ++kt) {
       uint32_t a[4][3];   // [fragment word][hi, mid, lo]
 #pragma unroll
       for (int p = 0; p < 2; ++p) {   // units 16 kt + 8 p + 2 q + {0, 1}
-        const int u = 16 * kt + 8 * p + 2 * q;
         float h[2][2];                // [row][unit]
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          float acc0 = b1s[u + e], acc1 = acc0;
-#pragma unroll
-          for (int c = 0; c < kMaxIn; c += 4) {
-            const float4 w = *reinterpret_cast<const float4*>(W1s + (u + e) * kW1P + c);
-            acc0 = fmaf(w.x, x[0][c], acc0);
-            acc1 = fmaf(w.x, x[1][c], acc1);
-            acc0 = fmaf(w.y, x[0][c + 1], acc0);
-            acc1 = fmaf(w.y, x[1][c + 1], acc1);
-            acc0 = fmaf(w.z, x[0][c + 2], acc0);
-            acc1 = fmaf(w.z, x[1][c + 2], acc1);
-            acc0 = fmaf(w.w, x[0][c + 3], acc0);
-            acc1 = fmaf(w.w, x[1][c + 3], acc1);
-          }
-          h[0][e] = tanhf(acc0);
-          h[1][e] = tanhf(acc1);
-        }
+        layer1(x, 16 * kt + 8 * p + 2 * q, h);
         split3(h[0][0], h[0][1], a[2 * p]);
         split3(h[1][0], h[1][1], a[2 * p + 1]);
       }
