@@ -105,11 +105,21 @@ class ClockSampler:
 
 def bins_in_z(w, tuning):
     """True when the FP32 bin power sums ride in the TMA-staged forward z pass
-    (wide_z = 2 on a power-of-two grid of 256 or more, at most 256 bins): the
+    (wide_z = 2, chosen or built in (effective_tuning), on a power-of-two grid of 256 or more, at most 256 bins): the
     bins stage then reads only the packed x2 = 0 column."""
     n = w.ngrid
     return (bool(tuning) and tuning[1] == 2 and w.precision == "fp32" and w.n_kbins <= 256
             and n >= 256 and (n & (n - 1)) == 0)
+
+
+def effective_tuning(w, tuning, spectral=False):
+    """The tuning with the library's built-in choice of the z passes in place of
+    None or wide_z = -1: the TMA-staged ones on FP32 grids of 1024 points with
+    the real-space gradient, the plain ones otherwise."""
+    t = list(tuning) if tuning else [-1, -1, 16, 0]
+    if t[1] < 0 and w.precision == "fp32" and w.ngrid == 1024 and not spectral:
+        t[1] = 2
+    return t
 
 
 def stage_bytes(w, stage, fused_interp=True, spectral=False, bins_fused=False):
@@ -462,7 +472,7 @@ def run_gpu(args, w, rank, world):
         per_launch_ms = tot_ms / max(calls, 1)     # memset/reduce ride along in the stage
     fused = stages["interp"][1] == 0
     spectral = bool(args.spectral_gradient)
-    bz = bins_in_z(wr, tuning)
+    bz = bins_in_z(wr, effective_tuning(wr, tuning, spectral))
     alg = stage_bytes(wr, dom, fused, spectral, bz)
     achieved = alg / (per_launch_ms / 1e3) / 1e9
     roof = {"kernel": dom, "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm,
