@@ -80,6 +80,11 @@ constexpr double kIX0 = 0.5, kIH = 0.25;
 constexpr int kISeg = 94, kICoef = 12;
 void launch_I_table(double* coef, cudaStream_t s);
 
+// Whether a response uses the table of the whole intervals' points (NuArgs::nodes),
+// which takes a launch of its own: 32 bins on 16 nodes lose it (137.8 against 134.1 us a
+// kick), 256 on 128 gain 30 us.
+inline bool uses_node_table(int nk, int n_hist) { return (int64_t)nk * n_hist >= 2048; }
+
 // Device inputs of the response kernels (one struct, passed by value).
 struct NuArgs {
   int nk, ns, n_hist, quad, iters, use_fit, ngrid;
@@ -178,6 +183,11 @@ inline CellSize cell_size(double d) {
   if (c.re < 100 || c.re > 2000) c.re = -65536;
   return c;
 }
+
+// Grids (points a side) whose rows one CTA scans in one round: one launch of 5 us for three of
+// 3 us each (at 128 points it takes two rounds and 13 us: twelve such boxes in a
+// graph lost 1.5%).
+constexpr int kScanOneMax = 64;
 
 // FFT passes in launch order of one kick
 constexpr int kPassXFwd = 0, kPassYFwd = 1, kPassZFwd = 2, kPassZInv = 3, kPassYInv = 4, kPassXInv = 5;

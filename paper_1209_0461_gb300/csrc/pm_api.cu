@@ -941,7 +941,7 @@ int pm_deposit(pm_ctx* c, const void* pos) {
     }
   } else {
     {
-      Stage st(c, PM_ST_DEPOSIT, c->n <= 64 ? 3 : 5);
+      Stage st(c, PM_ST_DEPOSIT, c->n <= kScanOneMax ? 3 : 5);   // count, scan, scatter
       rc = sort_rows(c, g, pos);
     }
     if (rc == PM_ERR_CUDA) return rc;
@@ -1095,9 +1095,7 @@ NuArgs nu_args(pm_ctx* c, double a, const double* sqrtPM_hist, int32_t n_hist, c
     A.nchunks = ch < 1 ? 1 : (ch > kNuChunks ? kNuChunks : ch);
   }
   A.parts = c->d_parts;
-  // the table of the whole intervals' points takes a launch of its own: 32 bins
-  // on 16 nodes lose it (137.8 against 134.1 us a kick), 256 on 128 gain 30 us
-  A.nodes = (int64_t)c->nk * n_hist >= 2048 ? c->d_nodes : nullptr;
+  A.nodes = uses_node_table(c->nk, n_hist) ? c->d_nodes : nullptr;
   A.rlist = c->d_rlist;
   A.R = c->d_R;
   A.pnu = c->d_pnu;
@@ -1149,7 +1147,8 @@ int pm_nu_response(pm_ctx* c, double a, const double* a_hist, const double* sqrt
     return fail(c, PM_ERR_ORDER, "pm_nu_response before pm_deposit");
   }
   const bool nu = c->ns > 0 && c->f_nu > 0;
-  Stage stage(c, PM_ST_RESPONSE, (nu && !use_prep ? 1 + (c->nk * (int64_t)n_hist >= 2048) : 0) + 2);   // [nodes, panels,] finish + bin list, table
+  // [nodes, panels,] finish + bin list, table
+  Stage stage(c, PM_ST_RESPONSE, (nu && !use_prep ? 1 + uses_node_table(c->nk, n_hist) : 0) + 2);
   NuArgs A = nu_args(c, a, sqrtPM_hist, n_hist, sqrtPnu_prev, ratio_out, sqrtPnu_out, sqrtPM_out);
   if (use_prep) A.hist_u = c->d_hist_u2;
   if (nu && !use_prep) launch_nu_panels(A, c->stream);

@@ -234,10 +234,6 @@ __device__ __forceinline__ void row_scan_cta(int* __restrict__ count, int* __res
   }
 }
 __global__ void k_scan_one(int* __restrict__ count, int* __restrict__ start, int* __restrict__ cursor, int len);
-// Grids whose rows one CTA scans in one round: one launch of 5 us for three of
-// 3 us each (at 128 points it takes two rounds and 13 us: twelve such boxes in a
-// graph lost 1.5%).
-constexpr int kScanOneMax = 64;
 
 // Exclusive scan of n values in three launches (the first clears its input): per-block scans of 2048
 // values (block totals out), a single-block scan of the totals, and the add.
