@@ -588,14 +588,14 @@ k_fft_x_fwd(const unsigned long long* __restrict__ grid, cx<T>* __restrict__ spe
 // the particles of four source rows, (z - 1, z) x (y - 1, y), whose records
 // (sorted by k_row_scatter) the warp reads; the corner's y and z weights then
 // depend on the source row alone and every lane has two corners, x and x + 1.
-// No other warp adds to the row, so nothing waits on a barrier: the deposit,
-// the exchanges of the transform and the split step's partners (a lane
+// No other warp adds to the row (but for very long ones, kLongRow), so nothing waits
+// on a barrier: the deposit, the exchanges of the transform and the split step's partners (a lane
 // shuffle: X[M - k] sits in lane NT - t) are the warp's own.  No global
 // deposit grid, no memset, no atomics to DRAM.  With `keep` set the sums are
 // also written out (inspection).
 //
 // Bound: the shared-memory pipe (16 atomic adds a particle at 2.5 wavefronts, and
-// the exchanges: LSU data pipe 85%, ALU 56% at 256^3).  A record is read by four
+// the exchanges: LSU data pipe 93%, ALU 54% at 256^3).  A record is read by four
 // warps (L1 and L2 after the first) where a CTA tile of 2 x 4 rows read it 1.9
 // times, but there half of the corner adds issued fell outside the tile, and
 // phases waited at barriers: 3.90 -> 2.77 ms at 1024^3 points / 512^3 particles,
@@ -860,8 +860,8 @@ k_deposit_fft_x(const unsigned long long* __restrict__ rec, const int* __restric
 // Body of one group of rows (bx) of one field (`data` its base); grad: apply -i D(kx) first.
 // FP32 rows of up to 512 points (RowCfg::WARP): a row belongs to NT lanes of one
 // warp, the split step's partner X[M - k] of k = t + NT i sits in lane NT - t at
-// E - 1 - i (lane 0: its own E - i) and comes by a shuffle, and the exchanges wait for the warp alone: 37 -> 27 us at 256^3, 0.201 ->
-// 0.166 ms at 512^3.  (At 1024 points, 32 elements a lane, holding both the row and
+// E - 1 - i (lane 0: its own E - i) and comes by a shuffle, and the exchanges wait
+// for the warp alone: 37 -> 27 us at 256^3, 0.201 -> 0.166 ms at 512^3.  (At 1024 points, 32 elements a lane, holding both the row and
 // its split costs occupancy and the pass ran 2.07 instead of 1.52 ms; FP64 is bound
 // by its FP64 pipe: 0.532 against 0.510 ms at 256^3.)
 template <typename T, int N>

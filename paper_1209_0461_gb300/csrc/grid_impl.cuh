@@ -269,8 +269,9 @@ void deposit_fft_x_n(const GridArgs& g, const void* pos, bool keep, cudaStream_t
     attr.add(g.device);
   }
   k_deposit_fft_x<T, N><<<N * N / F::ROWS, F::THREADS, F::SMEM, s>>>(
-      g.rec, g.row_start, reinterpret_cast<C*>(g.spec), DepositScale{g.scale, g.scale_hi, g.scale_lo}, reinterpret_cast<const C*>(g.tw_m),
-      reinterpret_cast<const C*>(g.tw_n), keep ? reinterpret_cast<unsigned long long*>(g.g) : nullptr, g.status);
+      g.rec, g.row_start, reinterpret_cast<C*>(g.spec), DepositScale{g.scale, g.scale_hi, g.scale_lo},
+      reinterpret_cast<const C*>(g.tw_m), reinterpret_cast<const C*>(g.tw_n),
+      keep ? reinterpret_cast<unsigned long long*>(g.g) : nullptr, g.status);
 }
 
 // Fused inverse x + interpolation + kick of size N (persistent grid).

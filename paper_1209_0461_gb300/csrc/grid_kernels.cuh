@@ -1060,10 +1060,10 @@ __device__ __forceinline__ void fd_combine(const T (&px)[2][2][6], const T (&py)
 // address a row serves its loads by constant offsets; the few particles there
 // take the wrapped indices.  FP32 x runs: aligned 8-byte loads from x0 - 2
 // rounded down to even (three, a fourth when x0 is odd).
-// Bound: the L1 data pipe (two wavefronts a load: 32 neighbouring particles
-// span two 128-byte lines) and the load queue; 64 KB-register CTAs (14 or 16
-// of 64 threads per SM) spill and run slower (0.40 and 0.44 ms against 0.345
-// at 256^3), 4-byte loads of the x runs too (0.372; 3.55 against 3.09 ms at
+// Bound: the L1 data pipe, 95 to 98% (two wavefronts a load and more: 32
+// neighbouring particles span two 128-byte lines; in no order nine) and the load
+// queue; CTAs held to fewer registers (14 or 16 of 64 threads per SM) spill and run
+// slower (0.40 and 0.44 ms against 0.345 at 256^3), 4-byte loads of the x runs too (0.372; 3.55 against 3.09 ms at
 // 1024^3).  With wrapped indices for all particles and a run-time test of n in
 // every wrap it took 0.365 and 3.19 ms.
 template <typename T, bool POW2, bool PAIRS = sizeof(T) == 4>
@@ -1341,15 +1341,14 @@ __global__ void k_kick_inv(const int* __restrict__ inv, const T* __restrict__ ac
 }
 
 // k_interp_rows_acc from shared memory, FP32 grids of 128 to 512 points (longer
-// rows do not fit, smaller grids have too few tiles: gather_tiled).  A CTA owns the
-// particles that the deposit's sort placed
-// in TZ x TY grid rows (whole rows along x) and stages the potential rows their
-// stencils touch: TZ + 1 planes of TY + 5 rows and, for the z differences, TY + 1
+// rows do not fit, smaller grids have too few tiles: gather_tiled).  A CTA takes
+// particles that the deposit's sort placed in TZ x TY grid rows (whole rows along
+// x) and stages the potential rows their stencils touch: TZ + 1 planes of TY + 5 rows and, for the z differences, TY + 1
 // rows of the two planes on either side; each row with a halo of its periodic
 // neighbours, so that no index wraps.  A particle's 56 values are then
 // shared-memory reads at constant offsets from a few addresses.  For clustered
 // particles, whose lanes spread over their row, a read from global memory is
-// about ten L1 wavefronts, from shared memory three or four (32 lanes on 32 banks):
+// nine L1 wavefronts, from shared memory 2.4 (32 lanes on 32 banks; LSU data pipe 85%):
 // 512^3 clustered particles on 512^3 points with the velocity pass
 // 5.08 -> 3.66 ms.  (Particles near storage order gain nothing: their lanes read
 // neighbouring cells anyway, and velocities through the permutation cost more,

@@ -123,10 +123,6 @@ __device__ __forceinline__ double s_table(const NuArgs& A, double u) {
 // Beyond y = kMultipoleYMax (where K < 1e-10) the integrated-by-parts value
 // I(y) stands in.
 constexpr double kMultipoleYMax = 256.0;
-// 2^m, m in [-2, 1000], exactly
-__device__ __forceinline__ double exp2_int(int m) { return __hiloint2double((1023 + m) << 20, 0); }
-constexpr int kMaxGraded = 128;   // graded points looked at (ell 2^126 exceeds any ln a range)
-
 __device__ static double sph_j1(double z) {
   if (z < 1e-2) {
     const double z2 = z * z;
@@ -155,6 +151,10 @@ __device__ static double nu_K_warp(double y, const NuArgs& A, int lane) {
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   return -acc / (y * 1.5 * kRelZeta3);
 }
+
+// 2^m, m in [-2, 1000], exactly
+__device__ __forceinline__ double exp2_int(int m) { return __hiloint2double((1023 + m) << 20, 0); }
+constexpr int kMaxGraded = 128;   // graded points looked at (ell 2^126 exceeds any ln a range)
 
 // Break points of one bin's panels in descending order from u_e down to u_i:
 // the stored nodes and the graded points u_e - ell 2^m (m = -2, -1, ...) that

@@ -81,8 +81,11 @@ constexpr int kISeg = 94, kICoef = 12;
 void launch_I_table(double* coef, cudaStream_t s);
 
 // Whether a response uses the table of the whole intervals' points (NuArgs::nodes),
-// which takes a launch of its own: 32 bins on 16 nodes lose it (137.8 against 134.1 us a
-// kick), 256 on 128 gain 30 us.
+// which takes a launch of its own (8 us).  Response with / without it, 8 nodes a panel:
+// 64 bins on 16 history nodes 48.7 / 44.2 us, 64 on 32 48.8 / 50.2, 32 on 64 50.7 / 44.1,
+// 64 on 64 55.3 / 55.2, 64 on 128 61.1 / 68.9, 256 on 128 95.5 / 128.6; with the
+// relativistic background, whose points cost more, 64 on 16 57.9 / 54.5, 64 on 32
+// 60.9 / 67.1, 256 on 128 108 / 206.
 inline bool uses_node_table(int nk, int n_hist) { return (int64_t)nk * n_hist >= 2048; }
 
 // Device inputs of the response kernels (one struct, passed by value).

@@ -467,7 +467,9 @@ GridArgs grid_args(const pm_ctx* c) {
   // built-in z passes: the TMA-staged ones with the bin sums on FP32 grids of 1024
   // points (512^3 particles 17.18 -> 16.79 ms, 256^3 13.32 -> 12.48 ms a kick); on 256
   // and 512 points, whose planes L2 holds longer, the plain wide tiles (2.20
-  // against 2.25 ms at 512, 0.864 against 0.879 ms at 256; FP64 27.05 against 27.66 ms)
+  // against 2.25 ms at 512, 0.864 against 0.879 ms at 256; FP64 27.05 against 27.66 ms).
+  // With more than 256 bins, whose sums then are a pass of their own, too (deposit of
+  // 256^3 particles, 300 bins: 6.58 against 6.95 ms by wide, 7.59 by narrow tiles)
   g.wide_z = c->wide_z < 0 && c->n == 1024 && !c->fp64 && c->tma_z16 && g.fd_grad ? 2 : c->wide_z;
   g.n = c->n;
   g.np = c->np;
