@@ -747,9 +747,11 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
     // round trips: the CTA's warps then share its rows (2% of 256^3 particles in one of
     // 512^2 rows: 1.11 ms, 2.24 by one warp; FP64 5.06 and 6.40; even boxes as without).  Small
     // grids have their time in the adds themselves.
-    int most = 0;
-    for (int g = 0; g < G; ++g) most = max(most, SourceRows<N>(row_start, (row0 + g) / N, (row0 + g) % N).total);
+    const SourceRows<N> src(row_start, row0 / N, row0 % N);
+    int most = src.total;
+    for (int g = 1; g < G; ++g) most = max(most, SourceRows<N>(row_start, (row0 + g) / N, (row0 + g) % N).total);
     shared = __syncthreads_or(most >= kLongRow);
+    if (G == 1 && !shared) ovf = deposit_row_warp<N, Cfg::HI>(rec, src, reinterpret_cast<unsigned*>(wrows));
     if (shared) {
 #pragma unroll 1
       for (int k = 0; k < Cfg::ROWS; ++k) {
@@ -761,7 +763,7 @@ __device__ __forceinline__ void deposit_fft_x_tile(const unsigned long long* __r
       __syncthreads();
     }
   }
-  if (!shared) {
+  if (!shared && (N < 512 || G > 1)) {
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
       const int row = row0 + g;

@@ -329,7 +329,7 @@ void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
     cudaFuncSetAttribute(k_gather_tile_acc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     attr.add(g.device);
   }
-  const int helpers = 2 * g.sm_count;
+  const int helpers = (Cfg::CTAS - 1) * g.sm_count;   // a wave but one CTA per SM
   const int64_t mean = g.np / Cfg::TILES + 1, share = g.np / ((int64_t)16 * g.sm_count * Cfg::CTAS);
   const unsigned cap = (unsigned)(2 * mean > share ? 2 * mean : share);
   k_gather_tile_acc<N><<<helpers + Cfg::TILES, Cfg::THREADS, Cfg::SMEM, s>>>(

@@ -1482,7 +1482,7 @@ __device__ __forceinline__ void gather_tile_part(const unsigned long long* __res
 // holds beyond them goes in parts of `cap` to the helpers, the CTAs before those
 // (dispatched first): part c of tile t to helper (hash(t) + c) mod helpers.  A helper
 // looks through all tiles and stages the rows of its parts again; without parts
-// they cost 1 us at 128 points, 3 us at 256.  Without helpers a
+// they cost 1 us at 128 points, 3 us at 256, 20 us (of 3.4 ms) at 512.  Without helpers a
 // box with much of its mass in a few rows waits for a few CTAs: half of 256^3
 // particles in one filament on 256^3 points 6.4 ms with the velocity pass, 0.51 ms
 // with them (0.59 ms by k_interp_rows_acc; an even box 0.43 ms).
