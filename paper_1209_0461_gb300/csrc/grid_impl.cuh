@@ -312,15 +312,25 @@ int grid_blocks(int64_t work, int threads, int ctas_per_sm = 16) {
   return (int)b;
 }
 
-// Forces by sorted slot from shared-memory tiles (false: not for this grid and
-// particle number).  A CTA takes at most `cap` particles of a tile: twice the mean, or
-// where a wave holds many tiles as many as make the longest part a sixteenth of the pass.
-// The tiles want half a particle a cell, or staging their rows costs more than it
-// saves: with the velocity pass on clustered particles, tiles against
-// k_interp_rows_acc, 37 / 33 us for a quarter and 45 / 50 us for a half at 128^3
-// points, 0.171 / 0.173 and 0.267 / 0.300 ms at 256^3, 1.34 / 1.23 and 2.15 / 2.38 ms
-// at 512^3.  And 128 points: 64^3 has fewer tiles than a wave holds, and parts do
-// not even that out (one filament 29 / 24 us).
+// Whether forces by sorted slot come from shared-memory tiles (FP32 grids of up to 512
+// points), times with the velocity pass, tiles / k_interp_rows_acc:
+//  - half a particle a cell or more, or staging the tiles' rows costs more than it
+//    saves (clustered particles, 37 / 33 us for a quarter and 45 / 50 us for a half at 128^3
+//    points, 0.171 / 0.173 and 0.267 / 0.300 ms at 256^3, 1.34 / 1.23 and 2.15 / 2.38 ms at
+//    512^3), and 128 points: 64^3 has fewer tiles than a wave holds, and parts do
+//    not even that out (262 144 particles, half in a filament, 31 / 24 us);
+//  - or few particles, where the other's threads walk over empty rows: 1000 at 256^3
+//    32 / 2204 us; 65 536 at 64^3 15 / 23 us even and 21 / 24 in one clump, at 256^3
+//    70 / 66 and 70 / 95; 262 144 at 256^3 70 / 49 and 71 / 100 (where few rows hold them 140 to 200 /
+//    100); at 512^3 32 768 373 / 320 and 105 / 949 us, 65 536 458 / 177 and 361 / 325.  16^3
+//    has 16 tiles: up to 8 a cell (32 768 16.7 / 18.6 us).
+inline bool tiles_pay(int n, int64_t np) {
+  const int64_t cells = (int64_t)n * n * n;
+  if (np <= (n == 512 ? 32768 : 65536) && np <= 8 * cells) return true;
+  return n >= 128 && 2 * np >= cells;
+}
+// A CTA takes at most `cap` particles of a tile: twice the mean, or where a wave holds
+// many tiles as many as make the longest part a sixteenth of the pass.
 template <int N>
 void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
   using Cfg = GatherTile<N>;
@@ -329,17 +339,23 @@ void gather_tile_n(const GridArgs& g, float scale, cudaStream_t s) {
     cudaFuncSetAttribute(k_gather_tile_acc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     attr.add(g.device);
   }
-  const int helpers = (Cfg::CTAS - 1) * g.sm_count;   // a wave but one CTA per SM
+  // a wave but one CTA per SM; one per SM for few particles
+  const int helpers = g.np <= 65536 ? g.sm_count : (Cfg::CTAS - 1) * g.sm_count;
   const int64_t mean = g.np / Cfg::TILES + 1, share = g.np / ((int64_t)16 * g.sm_count * Cfg::CTAS);
-  const unsigned cap = (unsigned)(2 * mean > share ? 2 * mean : share);
+  const int64_t cap = 2 * mean > share ? 2 * mean : share;
   k_gather_tile_acc<N><<<helpers + Cfg::TILES, Cfg::THREADS, Cfg::SMEM, s>>>(
-      g.rec, g.row_start, helpers, cap, scale, reinterpret_cast<const float*>(g.g), reinterpret_cast<float*>(g.accs));
+      g.rec, g.row_start, helpers, (unsigned)(cap > 512 ? cap : 512), scale, reinterpret_cast<const float*>(g.g),
+      reinterpret_cast<float*>(g.accs));
 }
+// Forces by sorted slot from tiles (false: not for this grid and particle number).
 template <typename U>
 bool gather_tiled(const GridArgs& g, U scale, cudaStream_t s) {
   if constexpr (sizeof(U) == 4) {
-    if (2 * g.np < (int64_t)g.n * g.n * g.n) return false;
+    if (!tiles_pay(g.n, g.np)) return false;
     switch (g.n) {
+      case 16: gather_tile_n<16>(g, scale, s); return true;
+      case 32: gather_tile_n<32>(g, scale, s); return true;
+      case 64: gather_tile_n<64>(g, scale, s); return true;
       case 128: gather_tile_n<128>(g, scale, s); return true;
       case 192: gather_tile_n<192>(g, scale, s); return true;
       case 256: gather_tile_n<256>(g, scale, s); return true;

@@ -1340,8 +1340,8 @@ __global__ void k_kick_inv(const int* __restrict__ inv, const T* __restrict__ ac
   }
 }
 
-// k_interp_rows_acc from shared memory, FP32 grids of 128 to 512 points (longer
-// rows do not fit, smaller grids have too few tiles: gather_tiled).  A CTA takes
+// k_interp_rows_acc from shared memory, FP32 grids of up to 512 points (longer
+// rows do not fit; where they pay: tiles_pay).  A CTA takes
 // particles that the deposit's sort placed in TZ x TY grid rows (whole rows along
 // x) and stages the potential rows their stencils touch: TZ + 1 planes of TY + 5 rows and, for the z differences, TY + 1
 // rows of the two planes on either side; each row with a halo of its periodic
@@ -1443,7 +1443,7 @@ __device__ __forceinline__ void gather_tile_part(const unsigned long long* __res
                                                  int tile, unsigned from, unsigned to) {
   using Cfg = GatherTile<N>;
   constexpr int TY = Cfg::TY, TZ = Cfg::TZ;
-  constexpr int YM = 31;                      // the record holds y mod 32
+  constexpr int YM = (N < 32 ? N : 32) - 1;   // the record holds y mod 32
   const int y0 = (tile % (N / TY)) * TY, z0 = (tile / (N / TY)) * TZ;
   // the rows y0 .. y0 + TY - 1 of a plane are one run of sorted slots: TZ runs,
   // concatenated in a virtual index j

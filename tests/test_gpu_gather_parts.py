@@ -1,5 +1,5 @@
 """Forces by sorted slot where a few grid rows hold much of the mass: the tiles'
-parts beyond the first, bit for bit, on either side of the particle number from
+parts beyond the first, bit for bit, on either side of the particle numbers between
 which tiles are taken; and no waiting for the few CTAs that own those rows."""
 import numpy as np
 import pytest
@@ -34,7 +34,10 @@ def _forces(pm, pos, rows):
 
 @pytest.mark.parametrize("n,npart,share", [(128, 128 ** 3 // 2 - 1, 0.5), (128, 128 ** 3 // 2, 0.5), (128, 2 ** 21 + 77, 0.9),
                                            (192, 192 ** 3 // 2 + 5, 0.5), (256, 2 ** 23, 0.5), (256, 2 ** 24 + 1, 0.02),
-                                           (512, 2 ** 26 + 3, 0.3), (1024, 2 ** 20, 0.5)])
+                                           (512, 2 ** 26 + 3, 0.3), (1024, 2 ** 20, 0.5),
+                                           (16, 32768, 0.5), (16, 32769, 0.5), (32, 65536, 0.9), (64, 65536, 0.5),
+                                           (64, 65537, 0.5), (192, 20011, 0.9), (256, 65536, 0.5), (256, 1, 0.0),
+                                           (512, 32768, 0.5), (512, 32769, 0.5)])
 def test_parts_are_bit_identical(n, npart, share):
     import torch
     pm = nupm.PM(n, npart, 100.0, 0.3, 0.0, n_kbins=8, precision="fp32")
