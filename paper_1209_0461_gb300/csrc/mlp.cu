@@ -110,9 +110,9 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t a0, const
 
 // Two packed BF16 values with those that are not finite replaced by zero.
 __device__ __forceinline__ uint32_t finite_part(uint32_t w) {
-  if ((w & 0x7f80u) == 0x7f80u) w &= 0xffff0000u;
-  if ((w & 0x7f800000u) == 0x7f800000u) w &= 0xffffu;
-  return w;
+  const uint32_t lo = (w & 0x7f80u) == 0x7f80u ? 0u : 0xffffu;
+  const uint32_t hi = (w & 0x7f800000u) == 0x7f800000u ? 0u : 0xffff0000u;
+  return w & (lo | hi);
 }
 
 // One warp per 16 samples.  Lane (g, q) = (lane / 4, lane % 4) holds rows g and
@@ -137,13 +137,14 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 3) k_mlp_forward(MlpArgs A) {
   float* xs = reinterpret_cast<float*>(smf + FwdSmem::X) + warp * 16 * kXP;
   // fragment (kt, nt, lane): W2[8 nt + g][16 kt + 2q + {0, 1}] and + 8; weights that
   // are not finite apart (below)
-  bool odd = false;
+  uint32_t apart = 0;
   for (int i = threadIdx.x; i < 8 * 16 * 32; i += blockDim.x) {
     const int l = i & 31, nt = (i >> 5) & 15, kt = i >> 9;
     const __nv_bfloat16* w = A.W2 + (8 * nt + (l >> 2)) * kW + 16 * kt + 2 * (l & 3);
     const uint2 b = make_uint2(*reinterpret_cast<const uint32_t*>(w), *reinterpret_cast<const uint32_t*>(w + 8));
-    Bs[i] = make_uint2(finite_part(b.x), finite_part(b.y));
-    odd = odd || Bs[i].x != b.x || Bs[i].y != b.y;
+    const uint2 f = make_uint2(finite_part(b.x), finite_part(b.y));
+    Bs[i] = f;
+    apart |= (f.x ^ b.x) | (f.y ^ b.y);
   }
   for (int i = threadIdx.x; i < kW * kMaxIn; i += blockDim.x) {
     const int u = i / kMaxIn, c = i % kMaxIn;
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 3) k_mlp_forward(MlpArgs A) {
     b1s[i] = A.b1[i];
     bw[i] = make_float2(A.b2[i], bf(A.w3[i]));
   }
-  odd = __syncthreads_or(odd);
+  const bool odd = __syncthreads_or(apart != 0);
   // units u, u + 1 of layer 1 for two rows of inputs: h[row][unit]
   auto layer1 = [&](const float (&x)[2][kMaxIn], int u, float (&h)[2][2]) {
 #pragma unroll
